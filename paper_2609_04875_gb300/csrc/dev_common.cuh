@@ -119,6 +119,44 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
         : "memory");
 }
 
+// The same tcgen05 operations executed by a whole converged warp: one elected lane issues them (elect.sync
+// names the same lane every time, so a commit covers the MMAs issued before it).  Issued this way the
+// operands stay in uniform registers.  Issued by one thread inside a divergent branch, each MMA spent
+// 84-93 cycles on moving its descriptors there, more than the 64 cycles a 128 x 128 x 16 MMA takes: a
+// GB300 microbenchmark ran 16 P V and 16 S MMAs in 2690-2970 cycles from one thread, 2350 from a warp.
+__device__ __forceinline__ void mma_bf16_warp(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                              uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_bf16_ts_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                                 uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_commit_warp(uint32_t bar)
+{
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+        : "memory");
+}
+
 // Split partials (O / l, fp32, HD columns a row) are stored in blocks of 32 rows, 16-byte chunk major:
 // chunk k of row r at [r & ~31][k][r & 31].  Row blocks start at multiples of 32 rows, so a warp whose
 // lane i holds row 32 w + i writes or reads one chunk of its 32 rows as 512 contiguous bytes.

@@ -18,9 +18,10 @@
 //                   shared memory, then out by one TMA store per 64 columns).
 //   warp 8          producer: reads the page table; its lanes issue one TMA
 //                   box per (page, 64-column half) into K and V stage rings.
-//   warp 9          MMA: allocates TMEM; one thread issues tcgen05.mma for
-//                   S_t = Q_t K^T (A, B from shared memory) and
-//                   O_t += P_t V (A = P from TMEM, B = V from shared memory).
+//   warp 9          MMA: allocates TMEM; the converged warp issues tcgen05.mma
+//                   (through one elected lane) for S_t = Q_t K^T (A, B from
+//                   shared memory) and O_t += P_t V (A = P from TMEM, B = V
+//                   from shared memory).
 // Tensor-core order per key tile j (d = 128):  PV_0(j), S_0(j+1), PV_1(j),
 // S_1(j+1), so one softmax group works while the tensor core runs the other
 // group's GEMMs; S_t(j+1) waits for PV_t(j), which reads P_t(j) over S_t.
@@ -299,89 +300,89 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
     } else if (warp == 9 && n_all > 0) {
-        // =================================================== MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
-            constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
-            const int n0 = geo[0].ntiles, n1 = geo[1].ntiles;
-            auto issue_s = [&](int t, int s) {
-                const uint32_t qa = q_smem + t * C::kTileBytes;
-                const uint32_t kb = k_smem0 + s * C::kTileBytes;
+        // =================================================== MMA issuer (the whole warp; one elected lane issues)
+        constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
+        constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
+        // warp-uniform copies (every lane holds the same values already)
+        const int n0 = __shfl_sync(0xffffffffu, geo[0].ntiles, 0), n1 = __shfl_sync(0xffffffffu, geo[1].ntiles, 0);
+        const int n_mma = max(n0, n1);
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024);
+        const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
+        const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
+        auto issue_s = [&](int t, int s) {
+            const uint64_t qd = q_desc + t * (C::kTileBytes >> 4), kd = k_desc + s * (C::kTileBytes >> 4);
 #pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    const uint32_t off = (kk >> 2) * C::kRegionBytes + (kk & 3) * 32;
-                    ptx::mma_bf16(tmem + 128 * t, ptx::smem_desc_sw128(qa + off, 16, 1024),
-                                  ptx::smem_desc_sw128(kb + off, 16, 1024), kIdescQK, kk > 0 ? 1u : 0u);
-                }
-                ptx::mma_commit(b_s_full + 8 * t);
-            };
-            auto issue_pv = [&](int t, int s, bool acc) {
-                const uint32_t vb = v_smem0 + s * C::kTileBytes;
-                const uint32_t tp = C::kSepP ? tmem + 256 + 2 * HD + 64 * t : tmem + 128 * t;  // P_t
-#pragma unroll
-                for (int kk = 0; kk < kBN / 16; ++kk)
-                    mma_bf16_ts(tmem + 256 + HD * t, tp + kk * 8,
-                                ptx::smem_desc_sw128(vb + kk * 16 * 128, C::kRegionBytes, 1024), kIdescPV,
-                                (acc || kk > 0) ? 1u : 0u);
-                ptx::mma_commit(b_o_done + 8 * t);
-            };
-            bool ok = wait_bar(b_q_full, 0, wctx) && wait_bar(b_k_full, 0, wctx);
-            if (ok) {
-                ptx::tc_fence_after();
-                if (n0 > 0) issue_s(0, 0);
-                if (n1 > 0) issue_s(1, 0);
-                if (n0 > 0 || n1 > 0) ptx::mma_commit(b_k_empty);
+            for (int kk = 0; kk < HD / 16; ++kk) {
+                const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
+                mma_bf16_warp(tm + 128 * t, qd + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
             }
-            for (int j = 0; ok && C::kSepP && j < n_all; ++j) {
-                // d = 64: S_t(j+1) once the softmax holds S_t(j) in registers, P V_t(j) once P_t(j) is in
-                const int s = j % C::kStages;
-                const int s1 = (j + 1) % C::kStages;
-                const bool more = j + 1 < n_all;
-                if (more && !wait_bar(b_k_full + 8 * s1, ((j + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
+            mma_commit_warp(b_s_full + 8 * t);
+        };
+        auto issue_pv = [&](int t, int s, bool acc) {
+            const uint64_t vd = v_desc + s * (C::kTileBytes >> 4);
+            const uint32_t tp = C::kSepP ? tm + 256 + 2 * HD + 64 * t : tm + 128 * t;  // P_t
 #pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    if (j + 1 >= (t ? n1 : n0)) continue;
-                    if (!wait_bar(b_s_free + 8 * t, j & 1, wctx)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    issue_s(t, s1);
-                }
-                if (!ok) break;
-                if (more) ptx::mma_commit(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
-                if (!wait_bar(b_v_full + 8 * s, (j / C::kStages) & 1, wctx)) { ok = false; break; }
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    if (j >= (t ? n1 : n0)) continue;
-                    if (!wait_bar(b_p_full + 8 * t, j & 1, wctx)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    issue_pv(t, s, j > 0);
-                }
-                if (!ok) break;
-                ptx::mma_commit(b_v_empty + 8 * s);              // V of tile j consumed by its PV GEMMs
-            }
-            for (int j = 0; ok && !C::kSepP && j < n_all; ++j) {
-                const int s = j % C::kStages;
-                const int s1 = (j + 1) % C::kStages;
-                const bool more = j + 1 < n_all;
-                if (!wait_bar(b_v_full + 8 * s, (j / C::kStages) & 1, wctx)) { ok = false; break; }
-                if (j < n0) {
-                    if (!wait_bar(b_p_full, j & 1, wctx)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    issue_pv(0, s, j > 0);
-                }
-                if (more && !wait_bar(b_k_full + 8 * s1, ((j + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
-                ptx::tc_fence_after();
-                if (j + 1 < n0) issue_s(0, s1);
-                if (j < n1) {
-                    if (!wait_bar(b_p_full + 8, j & 1, wctx)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    issue_pv(1, s, j > 0);
-                }
-                if (j + 1 < n1) issue_s(1, s1);
-                if (more) ptx::mma_commit(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
-                ptx::mma_commit(b_v_empty + 8 * s);              // V of tile j consumed by its PV GEMMs
-            }
+            for (int kk = 0; kk < kBN / 16; ++kk)
+                mma_bf16_ts_warp(tm + 256 + HD * t, tp + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
+                                 (acc || kk > 0) ? 1u : 0u);
+            mma_commit_warp(b_o_done + 8 * t);
+        };
+        bool ok = wait_bar_warp(b_q_full, 0, wctx) && wait_bar_warp(b_k_full, 0, wctx);
+        if (ok) {
+            ptx::tc_fence_after();
+            if (n0 > 0) issue_s(0, 0);
+            if (n1 > 0) issue_s(1, 0);
+            if (n0 > 0 || n1 > 0) mma_commit_warp(b_k_empty);
         }
-        __syncwarp();
+        for (int j = 0; ok && C::kSepP && j < n_mma; ++j) {
+            // d = 64: S_t(j+1) once the softmax holds S_t(j) in registers, P V_t(j) once P_t(j) is in
+            const int s = j % C::kStages;
+            const int s1 = (j + 1) % C::kStages;
+            const bool more = j + 1 < n_mma;
+            if (more && !wait_bar_warp(b_k_full + 8 * s1, ((j + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                if (j + 1 >= (t ? n1 : n0)) continue;
+                if (!wait_bar_warp(b_s_free + 8 * t, j & 1, wctx)) { ok = false; break; }
+                ptx::tc_fence_after();
+                issue_s(t, s1);
+            }
+            if (!ok) break;
+            if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
+            if (!wait_bar_warp(b_v_full + 8 * s, (j / C::kStages) & 1, wctx)) { ok = false; break; }
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                if (j >= (t ? n1 : n0)) continue;
+                if (!wait_bar_warp(b_p_full + 8 * t, j & 1, wctx)) { ok = false; break; }
+                ptx::tc_fence_after();
+                issue_pv(t, s, j > 0);
+            }
+            if (!ok) break;
+            mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its PV GEMMs
+        }
+        for (int j = 0; ok && !C::kSepP && j < n_mma; ++j) {
+            const int s = j % C::kStages;
+            const int s1 = (j + 1) % C::kStages;
+            const bool more = j + 1 < n_mma;
+            if (!wait_bar_warp(b_v_full + 8 * s, (j / C::kStages) & 1, wctx)) { ok = false; break; }
+            if (j < n0) {
+                if (!wait_bar_warp(b_p_full, j & 1, wctx)) { ok = false; break; }
+                ptx::tc_fence_after();
+                issue_pv(0, s, j > 0);
+            }
+            if (more && !wait_bar_warp(b_k_full + 8 * s1, ((j + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
+            ptx::tc_fence_after();
+            if (j + 1 < n0) issue_s(0, s1);
+            if (j < n1) {
+                if (!wait_bar_warp(b_p_full + 8, j & 1, wctx)) { ok = false; break; }
+                ptx::tc_fence_after();
+                issue_pv(1, s, j > 0);
+            }
+            if (j + 1 < n1) issue_s(1, s1);
+            if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
+            mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its PV GEMMs
+        }
     } else if (warp < 8) {
         // =================================================== softmax / epilogue
         ptx::griddep_wait();                     // before this role's first global write
