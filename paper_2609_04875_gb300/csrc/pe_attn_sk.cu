@@ -21,7 +21,7 @@
 //
 // Roles (320 threads) as in replay_attn_kernel: softmax warpgroups 0 and 1
 // (one per q-tile, thread r owns row r), producer warp 8 (page table -> TMA
-// boxes), MMA warp 9 (one thread issues tcgen05.mma).  Every role walks the
+// boxes), MMA warp 9 (converged; one elected lane issues tcgen05.mma).  Every role walks the
 // same sequence of pieces, computed from the kernel parameters; barrier phases
 // run on across pieces (per q-tile tile counts for S / P / O, a global key
 // tile count for the K and V rings, a piece count for Q).  Two more barriers
@@ -433,87 +433,86 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
     } else if (warp == 9) {
-        // =================================================== MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
-            constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
-            auto issue_s = [&](int t, int s) {
-                const uint32_t qa = q_smem + t * C::kTileBytes;
-                const uint32_t kb = k_smem0 + s * C::kTileBytes;
+        // =================================================== MMA issuer (the whole warp; one elected lane issues)
+        constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
+        constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024);
+        const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
+        const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
+        auto issue_s = [&](int t, int s) {
+            const uint64_t qd = q_desc + t * (C::kTileBytes >> 4), kd = k_desc + s * (C::kTileBytes >> 4);
 #pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    const uint32_t off = (kk >> 2) * C::kRegionBytes + (kk & 3) * 32;
-                    ptx::mma_bf16(tmem + 128 * t, ptx::smem_desc_sw128(qa + off, 16, 1024),
-                                  ptx::smem_desc_sw128(kb + off, 16, 1024), kIdescQK, kk > 0 ? 1u : 0u);
-                }
-                ptx::mma_commit(b_s_full + 8 * t);
-            };
-            auto issue_pv = [&](int t, int s, bool acc) {
-                const uint32_t vb = v_smem0 + s * C::kTileBytes;
-#pragma unroll
-                for (int kk = 0; kk < kBN / 16; ++kk)
-                    mma_bf16_ts(tmem + 256 + HD * t, tmem + 128 * t + kk * 8,
-                                ptx::smem_desc_sw128(vb + kk * 16 * 128, C::kRegionBytes, 1024), kIdescPV,
-                                (acc || kk > 0) ? 1u : 0u);
-                ptx::mma_commit(b_o_done + 8 * t);
-            };
-            int gk = 0;              // key tiles consumed so far (ring position)
-            int cnt0 = 0, cnt1 = 0;  // tiles of q-tile 0 / 1 in earlier pieces (S, P, O phases)
-            int seg0 = 0, seg1 = 0;  // earlier pieces in which q-tile 0 / 1 had tiles (o_free phase)
-            bool ok = true;
-            Piece pc;
-            UnitGeo U;
-            for (int k = 0; ok && piece_of(P, cw, k, pc, U); ++k) {
-                const AttnSeq &sq = p.seqs[U.si];
-                const int n0 = q_geo(p, sq, U.pair, 0, pc.lo, pc.hi).ntiles;
-                const int n1 = q_geo(p, sq, U.pair, 1, pc.lo, pc.hi).ntiles;
-                const int n_all = pc.hi - pc.lo;
-                if (!wait_bar(b_q_full, k & 1, wctx) || !wait_bar(b_k_full + 8 * (gk % C::kStages),
-                                                                 (gk / C::kStages) & 1, wctx)) {
-                    ok = false;
-                    break;
-                }
-                ptx::tc_fence_after();
-                const int n_s = max(n0, n1);  // key tiles with S GEMMs; Q is free after the last one
-                if (n0 > 0) issue_s(0, gk % C::kStages);
-                if (n1 > 0) issue_s(1, gk % C::kStages);
-                ptx::mma_commit(b_k_empty + 8 * (gk % C::kStages));
-                if (n_s <= 1) ptx::mma_commit(b_q_empty);
-                for (int j = 0; j < n_all; ++j) {
-                    const int gj = gk + j;
-                    const int s = gj % C::kStages;
-                    const int s1 = (gj + 1) % C::kStages;
-                    const bool more = j + 1 < n_all;
-                    if (!wait_bar(b_v_full + 8 * s, (gj / C::kStages) & 1, wctx)) { ok = false; break; }
-                    if (j < n0) {
-                        // the first P V GEMM of a piece overwrites O_0: the previous piece's epilogue read it
-                        if (j == 0 && seg0 > 0 && !wait_bar(b_o_free, (seg0 - 1) & 1, wctx)) { ok = false; break; }
-                        if (!wait_bar(b_p_full, (cnt0 + j) & 1, wctx)) { ok = false; break; }
-                        ptx::tc_fence_after();
-                        issue_pv(0, s, j > 0);
-                    }
-                    if (more && !wait_bar(b_k_full + 8 * s1, ((gj + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    if (j + 1 < n0) issue_s(0, s1);
-                    if (j < n1) {
-                        if (j == 0 && seg1 > 0 && !wait_bar(b_o_free + 8, (seg1 - 1) & 1, wctx)) { ok = false; break; }
-                        if (!wait_bar(b_p_full + 8, (cnt1 + j) & 1, wctx)) { ok = false; break; }
-                        ptx::tc_fence_after();
-                        issue_pv(1, s, j > 0);
-                    }
-                    if (j + 1 < n1) issue_s(1, s1);
-                    if (j + 2 == n_s) ptx::mma_commit(b_q_empty);    // the piece's last S GEMMs read Q
-                    if (more) ptx::mma_commit(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
-                    ptx::mma_commit(b_v_empty + 8 * s);              // V of tile j consumed by its P V GEMMs
-                }
-                gk += n_all;
-                cnt0 += n0;
-                cnt1 += n1;
-                seg0 += n0 > 0 ? 1 : 0;
-                seg1 += n1 > 0 ? 1 : 0;
+            for (int kk = 0; kk < HD / 16; ++kk) {
+                const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
+                mma_bf16_warp(tm + 128 * t, qd + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
             }
+            mma_commit_warp(b_s_full + 8 * t);
+        };
+        auto issue_pv = [&](int t, int s, bool acc) {
+            const uint64_t vd = v_desc + s * (C::kTileBytes >> 4);
+#pragma unroll
+            for (int kk = 0; kk < kBN / 16; ++kk)
+                mma_bf16_ts_warp(tm + 256 + HD * t, tm + 128 * t + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
+                                 (acc || kk > 0) ? 1u : 0u);
+            mma_commit_warp(b_o_done + 8 * t);
+        };
+        int gk = 0;              // key tiles consumed so far (ring position)
+        int cnt0 = 0, cnt1 = 0;  // tiles of q-tile 0 / 1 in earlier pieces (S, P, O phases)
+        int seg0 = 0, seg1 = 0;  // earlier pieces in which q-tile 0 / 1 had tiles (o_free phase)
+        bool ok = true;
+        Piece pc;
+        UnitGeo U;
+        for (int k = 0; ok && piece_of(P, cw, k, pc, U); ++k) {
+            const AttnSeq &sq = p.seqs[U.si];
+            // warp-uniform copies (every lane holds the same values already)
+            const int n0 = __shfl_sync(0xffffffffu, q_geo(p, sq, U.pair, 0, pc.lo, pc.hi).ntiles, 0);
+            const int n1 = __shfl_sync(0xffffffffu, q_geo(p, sq, U.pair, 1, pc.lo, pc.hi).ntiles, 0);
+            const int n_all = __shfl_sync(0xffffffffu, pc.hi - pc.lo, 0);
+            if (!wait_bar_warp(b_q_full, k & 1, wctx) || !wait_bar_warp(b_k_full + 8 * (gk % C::kStages),
+                                                             (gk / C::kStages) & 1, wctx)) {
+                ok = false;
+                break;
+            }
+            ptx::tc_fence_after();
+            const int n_s = max(n0, n1);  // key tiles with S GEMMs; Q is free after the last one
+            if (n0 > 0) issue_s(0, gk % C::kStages);
+            if (n1 > 0) issue_s(1, gk % C::kStages);
+            mma_commit_warp(b_k_empty + 8 * (gk % C::kStages));
+            if (n_s <= 1) mma_commit_warp(b_q_empty);
+            for (int j = 0; j < n_all; ++j) {
+                const int gj = gk + j;
+                const int s = gj % C::kStages;
+                const int s1 = (gj + 1) % C::kStages;
+                const bool more = j + 1 < n_all;
+                if (!wait_bar_warp(b_v_full + 8 * s, (gj / C::kStages) & 1, wctx)) { ok = false; break; }
+                if (j < n0) {
+                    // the first P V GEMM of a piece overwrites O_0: the previous piece's epilogue read it
+                    if (j == 0 && seg0 > 0 && !wait_bar_warp(b_o_free, (seg0 - 1) & 1, wctx)) { ok = false; break; }
+                    if (!wait_bar_warp(b_p_full, (cnt0 + j) & 1, wctx)) { ok = false; break; }
+                    ptx::tc_fence_after();
+                    issue_pv(0, s, j > 0);
+                }
+                if (more && !wait_bar_warp(b_k_full + 8 * s1, ((gj + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
+                ptx::tc_fence_after();
+                if (j + 1 < n0) issue_s(0, s1);
+                if (j < n1) {
+                    if (j == 0 && seg1 > 0 && !wait_bar_warp(b_o_free + 8, (seg1 - 1) & 1, wctx)) { ok = false; break; }
+                    if (!wait_bar_warp(b_p_full + 8, (cnt1 + j) & 1, wctx)) { ok = false; break; }
+                    ptx::tc_fence_after();
+                    issue_pv(1, s, j > 0);
+                }
+                if (j + 1 < n1) issue_s(1, s1);
+                if (j + 2 == n_s) mma_commit_warp(b_q_empty);    // the piece's last S GEMMs read Q
+                if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
+                mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its P V GEMMs
+            }
+            gk += n_all;
+            cnt0 += n0;
+            cnt1 += n1;
+            seg0 += n0 > 0 ? 1 : 0;
+            seg1 += n1 > 0 ? 1 : 0;
         }
-        __syncwarp();
     } else {
         // =================================================== softmax / epilogue (warps 0-7)
         ptx::griddep_wait();                     // before this role's first global write
