@@ -481,8 +481,8 @@ __global__ void __launch_bounds__(kDecThreads, DecCfg<HD, RB>::kMinBlocks)
 //              a stage freeing as soon as its S^T MMA completes.
 //   warp 6     V producer: the same for V (a V stage is held until
 //              O^T += V^T P^T, after the tile's softmax).
-//   warp 5     MMA: TMEM allocation; one thread issues each S^T and each
-//              O^T += V^T P^T as soon as its operands are in place (S^T up to
+//   warp 5     MMA: TMEM allocation; the converged warp issues each S^T and each
+//              O^T += V^T P^T (through one elected lane) as soon as its operands are in place (S^T up to
 //              two tiles ahead), so loads, softmax and MMAs overlap.
 // The row reference m is a chunk's first tile max (log2 units) and only moves
 // when a tile's weight would pass 2^64 (or a row saw no key yet); then the
@@ -841,106 +841,116 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
         }
     } else if (warp == 5) {
-        // ============================================================ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t kIdS = ptx::idesc_bf16_f32(128, 16, false, false);
-            constexpr uint32_t kIdPV = ptx::idesc_bf16_f32(128, 16, false, true);
-            // S^T cursor: chunk ordinal ns_chunk, tile k_s within it; P V cursor: tiles left in its chunk
-            int ns = 0, np = 0;                    // next S^T tile, next P V tile (ordinals in this CTA)
-            int ns_chunk = 0;                      // chunk ordinal of tile ns
-            int s_left = 0;                        // tiles of chunk ns_chunk not yet given an S^T
-            int pv_tiles[4] = {0, 0, 0, 0};        // tile counts of chunks the S^T cursor has read
-            int np_chunk = 0, p_done = 0;          // P V cursor: chunk ordinal, tiles done in it
-            bool more = true;                      // the S^T cursor may read another chunk
-            int c0 = read_chunk(0);
-            if (c0 >= 0) {
-                const ChunkInfo ci = tc_chunk(p, s_seqs, s_rem_seq, c0);
-                s_left = ci.t1 - ci.t0;
-                pv_tiles[0] = s_left;
-            } else {
-                more = false;
-            }
-            ptx::mbar_arrive(b_ch_empty);
-            uint64_t t_last = ptx::globaltimer();
-            while (s_left > 0 || np < ns) {
-                bool progress = false;
-                // S^T(ns): K landed, S buffer free (P V(ns - 2) issued), Q of its chunk ready
-                if (s_left > 0 && ns <= np + 1) {
-                    const int s = ns % kTcKStages;
-                    const int tile_in = pv_tiles[ns_chunk & 3] - s_left;
-                    if ((tile_in > 0 || ptx::mbar_test_wait(b_q_ready + 8 * (ns_chunk & 1), (ns_chunk >> 1) & 1)) &&
-                        ptx::mbar_test_wait(k_full(s), (ns / kTcKStages) & 1)) {
-                        ptx::tc_fence_after();
-                        const uint32_t ka = sbase + s * C::kTileBytes;
-                        const uint32_t qa = q_smem + (ns_chunk & 1) * 4096;
-#pragma unroll
-                        for (int kk = 0; kk < HD / 16; ++kk) {
-                            const uint32_t off = (kk >> 2) * C::kRegionBytes + (kk & 3) * 32;
-                            const uint32_t qoff = (kk >> 2) * 2048 + (kk & 3) * 32;
-                            ptx::mma_bf16(t_s + 16 * (ns & 1), ptx::smem_desc_sw128(ka + off, 16, 1024),
-                                          ptx::smem_desc_sw128(qa + qoff, 16, 1024), kIdS, kk > 0 ? 1u : 0u);
-                        }
-                        ptx::mma_commit(b_s_full + 8 * (ns & 1));
-                        ptx::mma_commit(k_empty(s));  // the K stage is free once S^T(ns) is done
-                        if (s_left == 1) ptx::mma_commit(b_q_free + 8 * (ns_chunk & 1));  // the chunk's last S^T
-                        ++ns;
-                        if (--s_left == 0 && more) {
-                            // next chunk (the ring entry is read once, then released)
-                            const int c = read_chunk(ns_chunk + 1);
-                            ptx::mbar_arrive(b_ch_empty + 8 * ((ns_chunk + 1) % R));
-                            if (c >= 0) {
-                                ++ns_chunk;
-                                const ChunkInfo ci = tc_chunk(p, s_seqs, s_rem_seq, c);
-                                s_left = ci.t1 - ci.t0;
-                                pv_tiles[ns_chunk & 3] = s_left;
-                            } else {
-                                more = false;
-                            }
-                        }
-                        progress = true;
-                    }
+        // ============================================================ MMA issuer (the whole warp, converged;
+        // one elected lane issues.  Every decision is warp-uniform: probes and clocks go through a vote.)
+        constexpr uint32_t kIdS = ptx::idesc_bf16_f32(128, 16, false, false);
+        constexpr uint32_t kIdPV = ptx::idesc_bf16_f32(128, 16, false, true);
+        constexpr uint32_t kAll = 0xffffffffu;
+        const uint32_t tm = __shfl_sync(kAll, tmem, 0);
+        const uint64_t k_desc = ptx::smem_desc_sw128(sbase, 16, 1024);
+        const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024);
+        const uint64_t v_desc = ptx::smem_desc_sw128(sbase + C::kOffV, C::kRegionBytes, 1024);
+        const uint64_t p_desc = ptx::smem_desc_sw128(p_smem, 16, 1024);
+        auto ready = [&](uint32_t bar, int parity) -> bool {
+            return __all_sync(kAll, ptx::mbar_test_wait(bar, parity));
+        };
+        // chunk ordinal n's tile count (0: no more chunks); its ring entry is released
+        auto next_tiles = [&](int n) -> int {
+            int nt = 0;
+            if (wait_bar_warp(b_ch_full + 8 * (n % R), (n / R) & 1, wctx)) {
+                const int c = s_chunk[n % R];
+                if (c >= 0) {
+                    const ChunkInfo ci = tc_chunk(p, s_seqs, s_rem_seq, c);
+                    nt = ci.t1 - ci.t0;
                 }
-                // O^T += V^T P^T(np): V landed, P^T(np) written, and at a chunk's first tile the epilogue
-                // has read the O^T buffer's previous chunk
-                if (np < ns && ptx::mbar_test_wait(v_full(np % kTcVStages), (np / kTcVStages) & 1) &&
-                    ptx::mbar_test_wait(b_p_full + 8 * (np & 1), (np >> 1) & 1) &&
-                    (p_done > 0 || np_chunk < 2 ||
-                     ptx::mbar_test_wait(b_o_free + 8 * (np_chunk & 1), ((np_chunk - 2) >> 1) & 1))) {
+            }
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(b_ch_empty + 8 * (n % R));
+            return __shfl_sync(kAll, nt, 0);
+        };
+        // S^T cursor: chunk ordinal ns_chunk, tile k_s within it; P V cursor: tiles left in its chunk
+        int ns = 0, np = 0;                    // next S^T tile, next P V tile (ordinals in this CTA)
+        int ns_chunk = 0;                      // chunk ordinal of tile ns
+        int s_left = next_tiles(0);            // tiles of chunk ns_chunk not yet given an S^T
+        uint32_t pv_tiles = s_left;            // tile counts of chunks the S^T cursor has read: byte n & 3
+        int np_chunk = 0, p_done = 0;          // P V cursor: chunk ordinal, tiles done in it
+        bool more = s_left > 0;                // the S^T cursor may read another chunk
+        auto tiles_of = [&](int n) -> int { return (pv_tiles >> (8 * (n & 3))) & 0xffu; };
+        uint64_t t_last = ptx::globaltimer();
+        while (s_left > 0 || np < ns) {
+            bool progress = false;
+            // S^T(ns): K landed, S buffer free (P V(ns - 2) issued), Q of its chunk ready
+            if (s_left > 0 && ns <= np + 1) {
+                const int s = ns % kTcKStages;
+                const int tile_in = tiles_of(ns_chunk) - s_left;
+                if ((tile_in > 0 || ready(b_q_ready + 8 * (ns_chunk & 1), (ns_chunk >> 1) & 1)) &&
+                    ready(k_full(s), (ns / kTcKStages) & 1)) {
                     ptx::tc_fence_after();
-                    const uint32_t vb = sbase + C::kOffV + (np % kTcVStages) * C::kTileBytes;
-                    const uint32_t pb = p_smem + (np & 1) * 4096;
+                    const uint64_t kd = k_desc + s * (C::kTileBytes >> 4);
+                    const uint64_t qd = q_desc + (ns_chunk & 1) * (4096 >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
-                        ptx::mma_bf16(t_o + 16 * (np_chunk & 1),
-                                      ptx::smem_desc_sw128(vb + kk * 16 * 128, C::kRegionBytes, 1024),
-                                      ptx::smem_desc_sw128(pb + (kk >> 2) * 2048 + (kk & 3) * 32, 16, 1024), kIdPV,
-                                      (p_done > 0 || kk > 0) ? 1u : 0u);
-                    }
-                    ptx::mma_commit(v_empty(np % kTcVStages));
-                    ptx::mma_commit(b_o_done + 8 * (np & 1));
-                    ++np;
-                    if (++p_done == pv_tiles[np_chunk & 3]) {
-                        ptx::mma_commit(b_o_item + 8 * (np_chunk & 1));  // the chunk's O^T is complete
-                        ++np_chunk;
-                        p_done = 0;
+                    for (int kk = 0; kk < HD / 16; ++kk)
+                        mma_bf16_warp(tm + 16 * (ns & 1), kd + (((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4),
+                                      qd + (((kk >> 2) * 2048 + (kk & 3) * 32) >> 4), kIdS, kk > 0 ? 1u : 0u);
+                    mma_commit_warp(b_s_full + 8 * (ns & 1));
+                    mma_commit_warp(k_empty(s));  // the K stage is free once S^T(ns) is done
+                    if (s_left == 1) mma_commit_warp(b_q_free + 8 * (ns_chunk & 1));  // the chunk's last S^T
+                    ++ns;
+                    if (--s_left == 0 && more) {
+                        // next chunk (the ring entry is read once, then released)
+                        const int nt = next_tiles(ns_chunk + 1);
+                        if (nt > 0) {
+                            ++ns_chunk;
+                            s_left = nt;
+                            const int sh = 8 * (ns_chunk & 3);
+                            pv_tiles = (pv_tiles & ~(0xffu << sh)) | (static_cast<uint32_t>(nt) << sh);
+                        } else {
+                            more = false;
+                        }
                     }
                     progress = true;
                 }
-                if (progress) {
-                    t_last = ptx::globaltimer();
-                } else {
-                    if (*abort_flag) break;
-                    if (ptx::globaltimer() - t_last > kWaitNs) {  // bounded: give up, record, let every role leave
+            }
+            // O^T += V^T P^T(np): V landed, P^T(np) written, and at a chunk's first tile the epilogue
+            // has read the O^T buffer's previous chunk
+            if (np < ns && ready(v_full(np % kTcVStages), (np / kTcVStages) & 1) &&
+                ready(b_p_full + 8 * (np & 1), (np >> 1) & 1) &&
+                (p_done > 0 || np_chunk < 2 || ready(b_o_free + 8 * (np_chunk & 1), ((np_chunk - 2) >> 1) & 1))) {
+                ptx::tc_fence_after();
+                const uint64_t vd = v_desc + (np % kTcVStages) * (C::kTileBytes >> 4);
+                const uint64_t pd = p_desc + (np & 1) * (4096 >> 4);
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                    mma_bf16_warp(tm + 32 + 16 * (np_chunk & 1), vd + (kk * 16 * 128 >> 4),
+                                  pd + (((kk >> 2) * 2048 + (kk & 3) * 32) >> 4), kIdPV,
+                                  (p_done > 0 || kk > 0) ? 1u : 0u);
+                mma_commit_warp(v_empty(np % kTcVStages));
+                mma_commit_warp(b_o_done + 8 * (np & 1));
+                ++np;
+                if (++p_done == tiles_of(np_chunk)) {
+                    mma_commit_warp(b_o_item + 8 * (np_chunk & 1));  // the chunk's O^T is complete
+                    ++np_chunk;
+                    p_done = 0;
+                }
+                progress = true;
+            }
+            if (progress) {
+                t_last = ptx::globaltimer();
+            } else {
+                if (__any_sync(kAll, *abort_flag != 0)) break;
+                if (__any_sync(kAll, ptx::globaltimer() - t_last > kWaitNs)) {
+                    // bounded: give up, record, let every role leave
+                    if (lane == 0) {
                         *abort_flag = 1;
                         atomicCAS(p.status, 0, kStatusWaitTimeout);
-                        break;
                     }
+                    break;
                 }
             }
         }
         // every tcgen05 op of this CTA completes before TMEM is released
+        mma_commit_warp(b_drain);
         if (lane == 0) {
-            ptx::mma_commit(b_drain);
             const uint64_t start = ptx::globaltimer();
             while (!ptx::mbar_try_wait(b_drain, 0) && ptx::globaltimer() - start < 4000000ull) {
             }
