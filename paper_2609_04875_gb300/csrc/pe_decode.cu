@@ -1182,77 +1182,108 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
 }
 
-// Merge of an item's chunk partials (one block per (sequence, kv-head), thread = d-column), after
-// the decode kernel: M = max_k m_k, O = sum_k 2^(m_k - M) O_k / sum_k 2^(m_k - M) l_k over the item's
-// chunks in its chunk order.  Items held in one chunk were written by the decode kernel itself.
+// Merge of an item's chunk partials, after the decode kernel: M = max_k m_k,
+// O = sum_k 2^(m_k - M) O_k / sum_k 2^(m_k - M) l_k over the item's chunks.
+// Items held in one chunk were written by the decode kernel itself.  One
+// block per (sequence, kv-head) and query row: its 4 x 128/HD groups of HD/4
+// threads (16 bytes of the row each) take every kGroups-th chunk, kOB of
+// them per round trip, with a running maximum; shared memory merges the
+// groups in order.  Bound by the latency of the round trips, so they are
+// what is kept few: one for up to 32 chunks (d = 128).  With one block per
+// item and all rows and chunks in one thread's chain, a 47-chunk merge (12k
+// keys, 8 rows) took 19.7 us, as long as the decode itself; now 3.4 us.
+constexpr int kCombThreads = 128;
 template <int HD, int RB>
-__global__ void __launch_bounds__(128) decode_tc_combine_kernel(const __grid_constant__ DecodeParams p)
+__global__ void __launch_bounds__(kCombThreads) decode_tc_combine_kernel(const __grid_constant__ DecodeParams p)
 {
-    ptx::griddep_wait();  // launched with programmatic serialization: the decode kernel's partials
-    if (static_cast<int>(threadIdx.x) >= HD) return;
+    constexpr int kLanes = HD / 4;                  // threads per row of a chunk
+    constexpr int kGroups = kCombThreads / kLanes;  // chunks in flight side by side
+    constexpr int kOB = 8;                          // and one after another
+    __shared__ float4 s_acc[kGroups][kLanes];
+    __shared__ float s_m[kGroups], s_l[kGroups];
     const int si = static_cast<int>(blockIdx.x) / p.hkv;
     const int kvh = static_cast<int>(blockIdx.x) - si * p.hkv;
-    if (si >= p.n_seqs) return;
+    const int r = static_cast<int>(blockIdx.y);
     const DecodeSeq &sq = p.seqs[si];
     const int nt = tc_tiles(sq);
     const int nfull = nt / sq.cta0;
     const int first = sq.tile0 + kvh * nfull;
     const int rem = sq.rem0 >= 0 ? sq.rem0 + kvh : -1;
     const int cpi = nfull + (rem >= 0 ? 1 : 0);
-    if (cpi <= 1) return;
     const int g = p.group;
-    const int n_rows = sq.n_q * g;
-    const int t = static_cast<int>(threadIdx.x);
+    const int grp = static_cast<int>(threadIdx.x) / kLanes;
+    const int t = static_cast<int>(threadIdx.x) % kLanes;
     const float *pm = p.part + static_cast<int64_t>(p.total_tiles) * RB * HD;
     const float *pl = pm + static_cast<int64_t>(p.total_tiles) * RB;
-    // batches of kOB chunks, every load of a batch issued together (m and l are the same for
-    // every thread: broadcast reads)
-    constexpr int kOB = 32 / RB;
-    float mx[RB], den[RB], acc[RB];
-#pragma unroll
-    for (int r = 0; r < RB; ++r) {
-        mx[r] = -INFINITY;
-        den[r] = 0.f;
-        acc[r] = 0.f;
-    }
-    for (int k0 = 0; k0 < cpi; k0 += kOB) {
-        float mv[kOB][RB], lv[kOB][RB], ov[kOB][RB];
+    ptx::griddep_wait();  // launched with programmatic serialization: the decode kernel's partials
+    // the next kernel's set-up overlaps the merge from here on; let in before the wait, or during the decode
+    // kernel, it slowed the turn-structured rounds by 1-3 % (6.68 ms)
+    ptx::griddep_launch_dependents();
+    if (cpi <= 1 || r >= sq.n_q * g) return;
+    float mx = -INFINITY, den = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = grp; k0 < cpi; k0 += kGroups * kOB) {
+        float mv[kOB], lv[kOB];
+        float4 ov[kOB];
 #pragma unroll
         for (int u = 0; u < kOB; ++u) {
-            const int k = k0 + u;
-            const int64_t c = k < nfull ? first + k : rem;
-#pragma unroll
-            for (int r = 0; r < RB; ++r) {
-                const bool in = k < cpi && r < n_rows;
-                mv[u][r] = in ? __ldcg(pm + c * RB + r) : -INFINITY;
-                lv[u][r] = in ? __ldcg(pl + c * RB + r) : 0.f;
-                ov[u][r] = in ? __ldcg(p.part + (c * RB + r) * HD + t) : 0.f;
-            }
+            const int k = k0 + u * kGroups;
+            const bool in = k < cpi;
+            const int64_t c = (k < nfull || !in) ? first + (in ? k : 0) : rem;
+            mv[u] = in ? __ldcg(pm + c * RB + r) : -INFINITY;
+            lv[u] = in ? __ldcg(pl + c * RB + r) : 0.f;
+            ov[u] = in ? __ldcg(reinterpret_cast<const float4 *>(p.part + (c * RB + r) * HD) + t)
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        float bmx = mx;
 #pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            float bmx = mx[r];
+        for (int u = 0; u < kOB; ++u) bmx = fmaxf(bmx, mv[u]);
+        if (bmx == -INFINITY) continue;  // no visible key so far
+        const float f = mx == -INFINITY ? 0.f : ex2(mx - bmx);
+        den *= f;
+        acc.x *= f;
+        acc.y *= f;
+        acc.z *= f;
+        acc.w *= f;
+        mx = bmx;
 #pragma unroll
-            for (int u = 0; u < kOB; ++u) bmx = fmaxf(bmx, mv[u][r]);
-            const float f = (mx[r] == -INFINITY || bmx == -INFINITY) ? 0.f : ex2(mx[r] - bmx);
-            den[r] *= f;
-            acc[r] *= f;
-            mx[r] = bmx;
-#pragma unroll
-            for (int u = 0; u < kOB; ++u) {
-                const float w = (mv[u][r] == -INFINITY || bmx == -INFINITY) ? 0.f : ex2(mv[u][r] - bmx);
-                den[r] += w * lv[u][r];
-                acc[r] += w * ov[u][r];
-            }
+        for (int u = 0; u < kOB; ++u) {
+            if (mv[u] == -INFINITY) continue;  // O_k and l_k hold nothing
+            const float w = ex2(mv[u] - bmx);
+            den += w * lv[u];
+            acc.x += w * ov[u].x;
+            acc.y += w * ov[u].y;
+            acc.z += w * ov[u].z;
+            acc.w += w * ov[u].w;
         }
     }
-#pragma unroll
-    for (int r = 0; r < RB; ++r) {
-        if (r >= n_rows) continue;
-        const float inv = den[r] > 0.f ? 1.0f / den[r] : 0.f;
-        static_cast<__nv_bfloat16 *>(p.out)[(static_cast<int64_t>(sq.q_row0 + r / g) * p.hq + kvh * g + r % g) * HD +
-                                            t] = __float2bfloat16_rn(acc[r] * inv);
+    s_acc[grp][t] = acc;
+    if (t == 0) {
+        s_m[grp] = mx;
+        s_l[grp] = den;
     }
+    __syncthreads();
+    if (grp != 0) return;
+    float M = -INFINITY;
+#pragma unroll
+    for (int q = 0; q < kGroups; ++q) M = fmaxf(M, s_m[q]);
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    float l = 0.f;
+#pragma unroll
+    for (int q = 0; q < kGroups; ++q) {
+        if (s_m[q] == -INFINITY) continue;
+        const float w = ex2(s_m[q] - M);
+        const float4 x = s_acc[q][t];
+        l += w * s_l[q];
+        o.x += w * x.x;
+        o.y += w * x.y;
+        o.z += w * x.z;
+        o.w += w * x.w;
+    }
+    const float inv = l > 0.f ? 1.0f / l : 0.f;
+    uint2 *dst = reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(p.out) +
+                                           (static_cast<int64_t>(sq.q_row0 + r / g) * p.hq + kvh * g + r % g) * HD) + t;
+    *dst = make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
 }
 
 template <int HD, int RB>
@@ -1275,10 +1306,11 @@ cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const De
     cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, decode_tc_kernel<HD, RB>, tm_k, tm_v, p);
     if (e != cudaSuccess) return e;
+    if (!p.any_split) return cudaSuccess;  // every item was one chunk
     // the merges, also with programmatic serialization (its launch overlaps the decode grid's end)
     cudaLaunchConfig_t ccfg = {};
-    ccfg.gridDim = dim3(static_cast<unsigned>(p.n_seqs * p.hkv));
-    ccfg.blockDim = dim3(128);
+    ccfg.gridDim = dim3(static_cast<unsigned>(p.n_seqs * p.hkv), RB);
+    ccfg.blockDim = dim3(kCombThreads);
     ccfg.dynamicSmemBytes = 0;
     ccfg.stream = st;
     ccfg.attrs = attr;

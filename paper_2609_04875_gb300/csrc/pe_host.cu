@@ -126,7 +126,7 @@ struct pe_cache {
     CUtensorMap tm_k{}, tm_v{};    // tensor-core kernel: 64 x ps boxes
     CUtensorMap tm_kd{}, tm_vd{};  // decode kernel: 64 x min(ps, 64) boxes
     // options
-    int splitkv = -1, num_splits = 0, debug_poison = 0, decode_kernel = 1, dec_chunks_per_sm = 3;
+    int splitkv = -1, num_splits = 0, debug_poison = 0, decode_kernel = 1, dec_chunks_per_sm = 0;
     int attn_kernel = 1;          // prefill kernel: 1 auto, 2 persistent stream-K, 0 one work item per CTA
     int attn_ctas = 0;            // persistent kernel's CTA count (0 = chosen by the planner)
     int attn_order = -1;          // one-item kernel's item order: -1 auto, 0 kv-heads fastest, 1 pairs fastest
@@ -612,6 +612,46 @@ struct AttnItem {
     int32_t n_q;
 };
 
+// Tiles per chunk of a decode launch (tensor-core kernel): the length, 1..8, whose estimated finish
+// is earliest.  In units of a 128-key tile a chunk costs its tiles + kDecChunkCost.  The F full chunks
+// (the longest, taken first) fill ceil(F / N) rounds of the N SMs; the items' remainders first fill the
+// last round's idle SMs, what is left spreads over all of them.  A launch of few tiles so takes the
+// chunk length that gives every SM one or two equal chunks (94 tiles x 8 kv-heads: 152 chunks of at most
+// 5 tiles, not 376 of 2: 20.8 -> 17.4 us a layer with its merge); one of many tiles takes 7 or 8, where a
+// chunk's cost is least (16 agents, 5200 tiles: 67.4 us with either, 4.6 % more with 6).
+constexpr double kDecChunkCost = 0.35;
+int64_t decode_chunk_tiles(const pe_cache *c, const std::vector<AttnItem> &items, size_t lo, size_t hi)
+{
+    const int64_t hkv = c->cfg.num_kv_heads, N = c->num_sms;
+    int64_t best = 8;
+    double best_t = 1e30;
+    for (int64_t ct = 8; ct >= 1; --ct) {
+        int64_t F = 0, R = 0, rem_tiles = 0, rem_max = 0, cpi = 1;
+        for (size_t i = lo; i < hi; ++i) {
+            const int64_t nt = ceil_div(c->len[items[i].seq], 128), rem = nt % ct;
+            F += nt / ct * hkv;
+            R += rem ? hkv : 0;
+            rem_tiles += rem * hkv;
+            rem_max = std::max(rem_max, rem);
+            cpi = std::max(cpi, ceil_div(nt, ct));
+        }
+        const double U = static_cast<double>(ct) + kDecChunkCost;
+        const int64_t rounds = ceil_div(F, N), idle = rounds * N - F;
+        const double rem_cost = static_cast<double>(rem_tiles) + static_cast<double>(R) * kDecChunkCost;
+        double t = static_cast<double>(rounds) * U;
+        // remainders beyond what the idle SMs of the last round hold (each at least one)
+        const double room = static_cast<double>(idle) * U;
+        if (R > 0 && (idle == 0 || rem_cost > room))
+            t += std::max((rem_cost - room) / static_cast<double>(N), static_cast<double>(rem_max) + kDecChunkCost - (idle > 0 ? U : 0.0));
+        t += 0.1 * static_cast<double>(ceil_div(cpi, 32));  // the merge's round trips
+        if (t < best_t - 1e-9) {
+            best_t = t;
+            best = ct;
+        }
+    }
+    return best;
+}
+
 // Decode kernel launches (groups of kMaxSegs sequences).  Key splits: about two
 // waves of the CTAs that fit on the GPU at once, at least 2 tiles per split;
 // "splitkv" = 0 keeps one split, "num_splits" fixes the count.
@@ -640,9 +680,11 @@ pe_status run_decode(pe_cache *c, const std::vector<AttnItem> &items, int32_t la
                 max_rows = std::max<int64_t>(max_rows, static_cast<int64_t>(items[i].n_q) * g);
             }
             const int rb = max_rows <= 4 ? 4 : (max_rows <= 8 ? 8 : 16);
-            // chunks of ceil(tiles / (k x SMs)) tiles, 1..8 (k = "decode_chunks_per_sm", 3 by default)
+            // chunks of 1..8 tiles, the length with the shortest estimated finish; with the option
+            // "decode_chunks_per_sm" = k, ceil(tiles / (k x SMs)) tiles
             const int64_t k_per_sm = c->dec_chunks_per_sm;
-            int64_t force = std::min<int64_t>(8, std::max<int64_t>(1, ceil_div(tiles, k_per_sm * c->num_sms)));
+            int64_t force = k_per_sm > 0 ? std::min<int64_t>(8, std::max<int64_t>(1, ceil_div(tiles, k_per_sm * c->num_sms)))
+                                         : decode_chunk_tiles(c, items, lo, hi);
             if (c->splitkv == 1 && c->num_splits > 0) force = std::min<int64_t>(8, ceil_div(max_tiles, c->num_splits));
             // Chunk ids, longest first: every item's full chunks (sequence-major, kv-head next), then the
             // items' shorter remainder chunks, sequences by decreasing remainder length (ties: batch
@@ -714,6 +756,7 @@ pe_status run_decode(pe_cache *c, const std::vector<AttnItem> &items, int32_t la
             p.ps = cf.page_size;
             p.oob_row = static_cast<int32_t>(c->pool_rows);
             p.scale_log2 = scale * 1.4426950408889634f;
+            p.any_split = any_split ? 1 : 0;
             c->last_split = any_split ? 1 : 0;
             c->last_splits = p.seqs[0].n_splits;
             c->last_ctas = p.total_ctas;
