@@ -629,10 +629,8 @@ cudaError_t launch_bounded_wait_selftest(int32_t *status, uint64_t limit_ns, cud
 template <int HD>
 __global__ void __launch_bounds__(256) splitkv_combine_kernel(const __grid_constant__ AttnParams p)
 {
-    // launched with programmatic serialization after the attention grid: wait
-    // for its partials; the next kernel may start its own set-up meanwhile
-    ptx::griddep_launch_dependents();
-    ptx::griddep_wait();
+    // launched with programmatic serialization after the attention grid: the item is found before the
+    // wait for its partials, and the next kernel may start its own set-up during the merge
     constexpr int kGroups = HD / 32;  // column groups of 32 (8 chunks of 16 bytes)
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -651,27 +649,46 @@ __global__ void __launch_bounds__(256) splitkv_combine_kernel(const __grid_const
     const int qi = qt * (kBM / g) + row / g;
     const int64_t base = sq.part_row0 + static_cast<int64_t>(unit) * sq.n_splits * kBM + row;
     const int ns = sq.n_splits;
-    float mx = -INFINITY;
-    for (int s = 0; s < ns; ++s) mx = fmaxf(mx, p.part_lse[base + static_cast<int64_t>(s) * kBM]);
+    ptx::griddep_wait();
+    ptx::griddep_launch_dependents();
+    // Bound by the latency of its round trips: batches of kB splits, every load of a batch in flight at
+    // once, against a running maximum.  (Taking the maximum first and then the splits two at a time, a
+    // 4-split merge of 532 rows x 8 kv-heads cost 2 us more: 32 layers of it 530 -> 458 us.)
+    constexpr int kB = 4;
+    float mx = -INFINITY, den = 0.f;
     float acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-    float den = 0.f;
-    if (mx != -INFINITY) {
-#pragma unroll 2
-        for (int s = 0; s < ns; ++s) {
-            const int64_t r = base + static_cast<int64_t>(s) * kBM;
-            const float lse = p.part_lse[r];
-            if (lse == -INFINITY) continue;
-            const float w = ex2(lse - mx);
+    for (int s0 = 0; s0 < ns; s0 += kB) {
+        float lse[kB];
+        float4 v[kB][8];
+#pragma unroll
+        for (int u = 0; u < kB; ++u) {
+            const int64_t r = base + static_cast<int64_t>(min(s0 + u, ns - 1)) * kBM;
+            lse[u] = s0 + u < ns ? __ldcg(p.part_lse + r) : -INFINITY;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[u][k] = __ldcg(part_chunk<HD>(p.part_o, r, cg * 8 + k));
+        }
+        float bmx = mx;
+#pragma unroll
+        for (int u = 0; u < kB; ++u) bmx = fmaxf(bmx, lse[u]);
+        if (bmx == -INFINITY) continue;  // no visible key so far
+        const float f = mx == -INFINITY ? 0.f : ex2(mx - bmx);
+        den *= f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc[i] *= f;
+        mx = bmx;
+#pragma unroll
+        for (int u = 0; u < kB; ++u) {
+            if (lse[u] == -INFINITY) continue;  // (its rows may hold anything)
+            const float w = ex2(lse[u] - mx);
             den += w;
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                const float4 v = *part_chunk<HD>(p.part_o, r, cg * 8 + k);
-                acc[4 * k + 0] += w * v.x;
-                acc[4 * k + 1] += w * v.y;
-                acc[4 * k + 2] += w * v.z;
-                acc[4 * k + 3] += w * v.w;
+                acc[4 * k + 0] += w * v[u][k].x;
+                acc[4 * k + 1] += w * v[u][k].y;
+                acc[4 * k + 2] += w * v[u][k].z;
+                acc[4 * k + 3] += w * v[u][k].w;
             }
         }
     }
