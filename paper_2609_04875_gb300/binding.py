@@ -125,21 +125,35 @@ def _check(rc: int):
         raise PEError(rc, _lib.pe_last_error().decode())
 
 
+_i32_types, _i64_types = {}, {}  # array types by length (a program's calls use few lengths)
+
+
+def _int_array(vals, ctype, types):
+    if isinstance(vals, ctypes.Array) and vals._type_ is ctype:
+        return vals
+    if type(vals) is not list:
+        vals = list(vals)
+    n = max(1, len(vals))
+    arr = types.get(n)
+    if arr is None:
+        arr = ctype * n
+        if len(types) < 256:
+            types[n] = arr
+    try:
+        return arr(*vals)
+    except TypeError:  # entries that only int() converts
+        return arr(*[int(v) for v in vals])
+
+
 def i32_array(vals):
     """A ctypes int32 array of ``vals``; the batch calls take it as is, so a
     caller repeating a call with the same ids can convert them once."""
-    if isinstance(vals, ctypes.Array) and vals._type_ is ctypes.c_int32:
-        return vals
-    vals = [int(v) for v in vals]
-    return (ctypes.c_int32 * max(1, len(vals)))(*vals)
+    return _int_array(vals, ctypes.c_int32, _i32_types)
 
 
 def i64_array(vals):
     """A ctypes int64 array of ``vals`` (taken as is by the batch calls)."""
-    if isinstance(vals, ctypes.Array) and vals._type_ is ctypes.c_int64:
-        return vals
-    vals = [int(v) for v in vals]
-    return (ctypes.c_int64 * max(1, len(vals)))(*vals)
+    return _int_array(vals, ctypes.c_int64, _i64_types)
 
 
 _i32_array, _i64_array = i32_array, i64_array
@@ -195,7 +209,7 @@ def _dev_ptr(t, name, device=None):
 
 
 def _same_shape(out, Q):
-    if out is not None and tuple(out.shape) != tuple(Q.shape):
+    if out is not None and out.shape != Q.shape and tuple(out.shape) != tuple(Q.shape):
         raise ValueError(f"out has shape {tuple(out.shape)}, Q {tuple(Q.shape)}: they must match")
 
 
@@ -223,13 +237,18 @@ class PagedKVCache:
                 raise ValueError("init_free_order must list every page")
             cfg.init_free_order = ctypes.cast(self._order, _I32P)
         self._device = None
+        self._raw_stream = self._cur_dev = self._bf16 = None
         if not host_only:
             import torch
             self._device = torch.cuda.current_device()
+            self._bf16 = torch.bfloat16
+            self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            self._cur_dev = getattr(torch._C, "_cuda_getDevice", None)
+        self._default_scale = 1.0 / math.sqrt(head_dim)
         self._pools = (k_pool, v_pool)  # keep caller tensors alive
         if k_pool is not None:
-            cfg.k_pool = self._ptr(k_pool, "k_pool").value
-            cfg.v_pool = self._ptr(v_pool, "v_pool").value
+            cfg.k_pool = _dev_ptr(k_pool, "k_pool", self._device).value
+            cfg.v_pool = _dev_ptr(v_pool, "v_pool", self._device).value
         cfg.workspace_bytes = int(workspace_bytes)
         self.num_layers, self.num_kv_heads, self.head_dim = num_layers, num_kv_heads, head_dim
         self.page_size, self.num_pages, self.max_seqs = page_size, num_pages, max_seqs
@@ -261,10 +280,20 @@ class PagedKVCache:
     def handle(self):
         return self._h
 
+    # The arguments of every call, in as few steps as they take (these run on each call): the current
+    # stream's handle, and a tensor's address once its type, device and layout are seen to be right;
+    # whatever is not plainly right takes the general functions above, which raise.
     def _s(self, stream):
+        if stream is None and self._raw_stream is not None and self._cur_dev is not None:
+            return self._raw_stream(self._cur_dev())
         return ctypes.c_void_p(None) if self.host_only else _stream(stream)
 
     def _ptr(self, t, name):
+        try:
+            if t.dtype is self._bf16 and t.get_device() == self._device and t.is_contiguous():
+                return t.data_ptr()
+        except AttributeError:
+            pass
         return _dev_ptr(t, name, self._device)
 
     # -- sequences -----------------------------------------------------------
@@ -350,10 +379,11 @@ class PagedKVCache:
                                        cu, self._s(stream)))
 
     def _check_kv(self, K, V):
-        if K.shape != V.shape or K.dim() != 4:
+        shape = K.shape
+        if shape != V.shape or len(shape) != 4:
             raise ValueError("K and V must both be [L][n][Hkv][d]")
-        if K.shape[0] != self.num_layers or K.shape[2] != self.num_kv_heads or K.shape[3] != self.head_dim:
-            raise ValueError(f"K shape {tuple(K.shape)} does not match the cache")
+        if shape[0] != self.num_layers or shape[2] != self.num_kv_heads or shape[3] != self.head_dim:
+            raise ValueError(f"K shape {tuple(shape)} does not match the cache")
 
     # -- replay attention ------------------------------------------------------
     def replay_attn(self, seq, layer, Q, out=None, softmax_scale=None, stream=None):
@@ -371,15 +401,16 @@ class PagedKVCache:
 
     def replay_attn_batch(self, seqs, layer, Q, cu_q, out=None, softmax_scale=None, stream=None):
         """Q, out: CUDA bf16 [cu_q[-1]][Hq][d]; rows cu_q[i]:cu_q[i+1] are the last positions of seqs[i]."""
-        import torch
-        if Q.dim() != 3 or Q.shape[2] != self.head_dim or Q.shape[0] != cu_q[-1]:
+        shape = Q.shape
+        if len(shape) != 3 or shape[2] != self.head_dim or shape[0] != cu_q[-1]:
             raise ValueError("Q must be [cu_q[-1]][Hq][d]")
         _same_shape(out, Q)
         if out is None:
+            import torch
             out = torch.empty_like(Q)
-        scale = 1.0 / math.sqrt(self.head_dim) if softmax_scale is None else float(softmax_scale)
+        scale = self._default_scale if softmax_scale is None else float(softmax_scale)
         _check(_lib.pe_replay_attn_batch(self._h, len(seqs), _i32_array(seqs), layer, self._ptr(Q, "Q"),
-                                         _i32_array(cu_q), self._ptr(out, "out"), Q.shape[1], scale,
+                                         _i32_array(cu_q), self._ptr(out, "out"), shape[1], scale,
                                          self._s(stream)))
         return out
 

@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -378,9 +379,8 @@ void apply_crop(pe_cache *c, CropPlan &pl, int32_t *freed_out)
 
 pe_status launch_crops(pe_cache *c, const std::vector<CropPlan> &plans, cudaStream_t st)
 {
-    std::vector<char> buf(sizeof(CropParams));
-    CropParams &p = *reinterpret_cast<CropParams *>(buf.data());
-    std::memset(&p, 0, sizeof p);
+    CropParams p;  // (only the header and the segments in use are written: 18 KB otherwise)
+    std::memset(static_cast<void *>(&p), 0, offsetof(CropParams, segs));
     p.page_table = c->d_table;
     p.seq_len = c->d_len;
     p.k_pool = static_cast<uint4 *>(c->k_pool);
@@ -411,6 +411,7 @@ pe_status launch_crops(pe_cache *c, const std::vector<CropPlan> &plans, cudaStre
             for (int32_t k = 0; k < sg.n_freed; ++k) p.freed[nf + k] = pl.freed[k];
             nf += sg.n_freed;
             sg.tail_page = pl.tail_page;
+            sg.pad_ = 0;
         }
         if (injected_failure(c)) return launch_fault("crop kernel");
         if (c->host_only) continue;
@@ -519,9 +520,9 @@ pe_status apply_appends(pe_cache *c, const std::vector<AppendPlan> &plans, const
                         int64_t n_total, cudaStream_t st)
 {
     const int ps = c->cfg.page_size;
-    std::vector<char> pbuf(sizeof(AppendParams));
-    AppendParams *p = reinterpret_cast<AppendParams *>(pbuf.data());
-    std::memset(p, 0, sizeof(AppendParams));
+    AppendParams pbuf;  // (only the header, the segments and the page ids in use are written: 15 KB otherwise)
+    AppendParams *p = &pbuf;
+    std::memset(static_cast<void *>(p), 0, offsetof(AppendParams, segs));
     {
         p->K = static_cast<const uint4 *>(K);
         p->V = static_cast<const uint4 *>(V);
@@ -536,8 +537,10 @@ pe_status apply_appends(pe_cache *c, const std::vector<AppendPlan> &plans, const
         p->num_pages = c->cfg.num_pages;
         p->n_total = static_cast<int32_t>(n_total);
     }
+    int32_t pages_in_launch = 0;
     auto flush = [&]() -> pe_status {
         if (p->n_segs == 0) return PE_OK;
+        p->n_new = pages_in_launch;
         p->seg_tokens = p->segs[p->n_segs - 1].cum0 + p->segs[p->n_segs - 1].n_tokens;
         const int64_t chunks = static_cast<int64_t>(p->L) * p->seg_tokens * p->hkv * p->dvec;
         if (injected_failure(c)) return launch_fault("append kernel");
@@ -549,7 +552,6 @@ pe_status apply_appends(pe_cache *c, const std::vector<AppendPlan> &plans, const
         p->n_segs = 0;
         return PE_OK;
     };
-    int32_t pages_in_launch = 0;
     for (const AppendPlan &pl : plans) {
         // decided now, on the current references (the planners' page counts agree: settle_batch_cow)
         const std::vector<int32_t> &tt = c->table[pl.seq];
@@ -617,12 +619,14 @@ struct AttnItem {
 // (the longest, taken first) fill ceil(F / N) rounds of the N SMs; the items' remainders first fill the
 // last round's idle SMs, what is left spreads over all of them.  A launch of few tiles so takes the
 // chunk length that gives every SM one or two equal chunks (94 tiles x 8 kv-heads: 152 chunks of at most
-// 5 tiles, not 376 of 2: 20.8 -> 17.4 us a layer with its merge); one of many tiles takes 7 or 8, where a
-// chunk's cost is least (16 agents, 5200 tiles: 67.4 us with either, 4.6 % more with 6).
+// 5 tiles, not 376 of 2: 20.8 -> 17.4 us a layer with its merge); one of many tiles (more than 12 per SM)
+// takes 8, where a chunk's cost is least and the estimates hardly differ (16 agents, 5200 tiles: 67.4 us
+// with 7 or 8, 4.6 % more with 6).
 constexpr double kDecChunkCost = 0.35;
-int64_t decode_chunk_tiles(const pe_cache *c, const std::vector<AttnItem> &items, size_t lo, size_t hi)
+int64_t decode_chunk_tiles(const pe_cache *c, const std::vector<AttnItem> &items, size_t lo, size_t hi, int64_t tiles)
 {
     const int64_t hkv = c->cfg.num_kv_heads, N = c->num_sms;
+    if (tiles > 12 * N) return 8;  // many tiles per SM: the longest chunks
     int64_t best = 8;
     double best_t = 1e30;
     for (int64_t ct = 8; ct >= 1; --ct) {
@@ -665,13 +669,12 @@ pe_status run_decode(pe_cache *c, const std::vector<AttnItem> &items, int32_t la
     // tensor-core form (128-key tiles, one CTA per SM) unless "decode_kernel" = 2: CUDA cores (64-key tiles)
     const bool tc = (d == 128 || d == 64) && c->decode_kernel == 1;
     const int64_t tile_keys = tc ? 128 : kDecKeys;
-    std::vector<char> pbuf(sizeof(DecodeParams));
-    DecodeParams &p = *reinterpret_cast<DecodeParams *>(pbuf.data());
+    DecodeParams p;
     for (size_t lo = 0; lo < items.size(); lo += kMaxSegs) {
         const size_t hi = std::min(items.size(), lo + kMaxSegs);
         if (tc) {
             // chunks of at most 8 tiles; CTAs (one per SM) take them from a counter
-            std::memset(&p, 0, sizeof p);
+            std::memset(static_cast<void *>(&p), 0, offsetof(DecodeParams, seqs));
             int64_t tiles = 0, max_rows = 1, max_tiles = 1;
             for (size_t i = lo; i < hi; ++i) {
                 const int64_t nt = ceil_div(c->len[items[i].seq], 128);
@@ -684,7 +687,7 @@ pe_status run_decode(pe_cache *c, const std::vector<AttnItem> &items, int32_t la
             // "decode_chunks_per_sm" = k, ceil(tiles / (k x SMs)) tiles
             const int64_t k_per_sm = c->dec_chunks_per_sm;
             int64_t force = k_per_sm > 0 ? std::min<int64_t>(8, std::max<int64_t>(1, ceil_div(tiles, k_per_sm * c->num_sms)))
-                                         : decode_chunk_tiles(c, items, lo, hi);
+                                         : decode_chunk_tiles(c, items, lo, hi, tiles);
             if (c->splitkv == 1 && c->num_splits > 0) force = std::min<int64_t>(8, ceil_div(max_tiles, c->num_splits));
             // Chunk ids, longest first: every item's full chunks (sequence-major, kv-head next), then the
             // items' shorter remainder chunks, sequences by decreasing remainder length (ties: batch
@@ -1166,7 +1169,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         int split_tiles = static_cast<int>(max_tiles);
         split = best > 1 || splitkv == 1;
         if (split) split_tiles = static_cast<int>(std::max<int64_t>(1, ceil_div(max_tiles, std::max<int64_t>(best, 1))));
-        std::memset(&p, 0, sizeof p);
+        std::memset(static_cast<void *>(&p), 0, offsetof(AttnParams, seqs));
         p.page_table = c->d_table;
         p.out = out;
         p.status = c->d_status;
@@ -1273,8 +1276,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         return true;
     };
 
-    std::vector<char> pbuf(sizeof(AttnParams));
-    AttnParams &p = *reinterpret_cast<AttnParams *>(pbuf.data());
+    AttnParams p;  // (plan_group writes the header and the sequences in use)
     std::vector<char> sbuf;
     for (size_t lo = 0; lo < order.size(); lo += kMaxSegs) {
         const size_t hi = std::min(order.size(), lo + kMaxSegs);

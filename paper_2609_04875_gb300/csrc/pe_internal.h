@@ -33,7 +33,8 @@ struct AppendSeg {
     int32_t seq;
 };
 
-struct AppendParams {
+template <int SEGS, int PAGES>
+struct AppendParamsT {
     const uint4 *K;        // packed [L][n_total][Hkv][d] bf16, viewed as 16-byte chunks
     const uint4 *V;
     uint4 *k_pool;         // [L][num_pages][Hkv][ps][d]
@@ -41,9 +42,11 @@ struct AppendParams {
     int32_t *page_table;   // device mirror [max_seqs][max_pages_per_seq]
     int64_t *seq_len;      // device mirror [max_seqs]
     int32_t L, hkv, dvec, ps, num_pages, n_total, n_segs, seg_tokens;
-    AppendSeg segs[kMaxSegs];
-    int32_t new_pages[kAppendMaxPages];
+    int32_t n_new;         // page ids carried
+    AppendSeg segs[SEGS];
+    int32_t new_pages[PAGES];
 };
+using AppendParams = AppendParamsT<kMaxSegs, kAppendMaxPages>;
 
 // ---------------------------------------------------------------- crop
 constexpr int kMaxCropFreed = 2048;  // freed page ids carried by one crop launch (debug poison)
@@ -60,15 +63,17 @@ struct CropSeg {
     int32_t pad_;
 };
 
-struct CropParams {
+template <int SEGS, int FREED>
+struct CropParamsT {
     int32_t *page_table;
     int64_t *seq_len;
     uint4 *k_pool;
     uint4 *v_pool;
     int32_t n, poison, L, hkv, ps, dvec, num_pages;
-    CropSeg segs[kMaxCropSegs];
-    int32_t freed[kMaxCropFreed];
+    CropSeg segs[SEGS];
+    int32_t freed[FREED];
 };
+using CropParams = CropParamsT<kMaxCropSegs, kMaxCropFreed>;
 
 // ---------------------------------------------------------------- attention
 struct AttnSeq {

@@ -5,6 +5,10 @@
 // (8 bf16) with vector loads and stores; consecutive threads touch consecutive
 // chunks of one d-row, so a warp reads 512 contiguous bytes of the caller's
 // K/V and writes whole 256-byte rows (d = 128) of a page slot.
+#include <algorithm>
+#include <cstddef>
+#include <cstring>
+
 #include "pe_internal.h"
 #include "ptx.cuh"
 
@@ -22,7 +26,13 @@ __device__ __forceinline__ uint4 ld_stream(const uint4 *p)
     return v;
 }
 
-__global__ void __launch_bounds__(256) append_kv_kernel(const __grid_constant__ AppendParams p, int64_t chunks)
+// A launch's parameter block is copied by the host, the driver and the GPU's front end: 15 KB of it cost a
+// launch 0.5 us more than 1 KB (2.03 against 1.60 us of host time).  A batch of few sequences and pages
+// takes the kernel's form with the small block.
+constexpr int kSmallSegs = 16, kSmallPages = 128;
+
+template <typename Params>
+__global__ void __launch_bounds__(256) append_kv_kernel(const __grid_constant__ Params p, int64_t chunks)
 {
     // the attention launch that follows may start its set-up now; it waits for this grid's writes
     ptx::griddep_launch_dependents();
@@ -69,6 +79,14 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __grid_constant__ 
     }
 }
 
+// The fields before the segment table, which both forms of a parameter block share.
+template <typename Small, typename Full>
+static void copy_header(Small &q, const Full &p)
+{
+    static_assert(offsetof(Small, segs) == offsetof(Full, segs), "the same header");
+    std::memcpy(static_cast<void *>(&q), static_cast<const void *>(&p), offsetof(Full, segs));
+}
+
 cudaError_t launch_append(const AppendParams &p, int64_t chunks, cudaStream_t st)
 {
     static int sms = 0;
@@ -91,14 +109,23 @@ cudaError_t launch_append(const AppendParams &p, int64_t chunks, cudaStream_t st
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, append_kv_kernel, p, chunks);
+    if (p.n_segs <= kSmallSegs && p.n_new <= kSmallPages) {
+        using Small = AppendParamsT<kSmallSegs, kSmallPages>;
+        Small q;
+        copy_header(q, p);
+        std::copy(p.segs, p.segs + p.n_segs, q.segs);
+        std::copy(p.new_pages, p.new_pages + p.n_new, q.new_pages);
+        return cudaLaunchKernelEx(&cfg, append_kv_kernel<Small>, q, chunks);
+    }
+    return cudaLaunchKernelEx(&cfg, append_kv_kernel<AppendParams>, p, chunks);
 }
 
 // One block per cropped sequence.  Debug poison first overwrites the pages
 // whose last reference this crop dropped (every layer, head, slot, K and V) and
 // the stale tail of the last kept page when no other sequence holds it; then
 // the table entries [keep, old_n) of this sequence become -1.
-__global__ void __launch_bounds__(256) crop_kernel(const __grid_constant__ CropParams p)
+template <typename Params>
+__global__ void __launch_bounds__(256) crop_kernel(const __grid_constant__ Params p)
 {
     // launched with programmatic serialization: the launch overlaps the previous kernel (an attention
     // launch that may still read the pages this crop frees); every write here waits for it
@@ -155,7 +182,14 @@ cudaError_t launch_crop(const CropParams &p, cudaStream_t st)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, crop_kernel, p);
+    if (p.n <= kSmallSegs && !p.poison) {  // (the freed pages are only read to poison them)
+        using Small = CropParamsT<kSmallSegs, 1>;
+        Small q;
+        copy_header(q, p);
+        std::copy(p.segs, p.segs + p.n, q.segs);
+        return cudaLaunchKernelEx(&cfg, crop_kernel<Small>, q);
+    }
+    return cudaLaunchKernelEx(&cfg, crop_kernel<CropParams>, p);
 }
 
 __global__ void __launch_bounds__(256) table_copy_kernel(int32_t *page_table, int32_t src_row, int32_t dst_row,
