@@ -489,9 +489,35 @@ void settle_batch_cow(const pe_cache *c, std::vector<AppendPlan> &plans)
     }
 }
 
+// The copies-on-write of one append call that await their launch.
+struct CowList {
+    CowParams p;
+    CowList() { p.n = 0; }
+    pe_status flush(pe_cache *c, cudaStream_t st)
+    {
+        if (p.n == 0) return PE_OK;
+        p.k_pool = static_cast<uint4 *>(c->k_pool);
+        p.v_pool = static_cast<uint4 *>(c->v_pool);
+        p.page_table = c->d_table;
+        p.L = c->cfg.num_layers;
+        p.hkv = c->cfg.num_kv_heads;
+        p.ps = c->cfg.page_size;
+        p.dvec = c->cfg.head_dim / 8;
+        p.num_pages = c->cfg.num_pages;
+        cudaError_t e = launch_cow_copy(p, st);
+        p.n = 0;
+        if (e != cudaSuccess) return cuda_fail(e, "copy-on-write launch");
+        c->launches++;
+        return PE_OK;
+    }
+};
+
 // Copy-on-write of a sequence's shared, partially filled last page: pop a
-// fresh page, copy the valid slots on the device, drop one reference.
-pe_status apply_cow(pe_cache *c, int32_t seq, cudaStream_t st)
+// fresh page, copy the valid slots on the device, drop one reference.  The
+// copy goes into `cow`, launched before the call's next append launch: a page
+// that an append of the call writes has one holder by then, so no later copy
+// of the call reads it, and earlier copies of it were launched before.
+pe_status apply_cow(pe_cache *c, int32_t seq, CowList &cow, cudaStream_t st)
 {
     j_seq(c, seq, static_cast<int32_t>(c->table[seq].size()) - 1);
     std::vector<int32_t> &t = c->table[seq];
@@ -501,15 +527,16 @@ pe_status apply_cow(pe_cache *c, int32_t seq, cudaStream_t st)
     set_ref(c, src, c->refs[src] - 1);
     t.back() = dst;
     if (injected_failure(c)) return launch_fault("copy-on-write");
-    if (!c->host_only) {
-        const int32_t slots = static_cast<int32_t>(c->len[seq] % c->cfg.page_size);
-        int32_t *entry = c->d_table + static_cast<int64_t>(seq) * c->cfg.max_pages_per_seq + (t.size() - 1);
-        cudaError_t e = launch_cow_copy(static_cast<uint4 *>(c->k_pool), static_cast<uint4 *>(c->v_pool), src, dst,
-                                        slots, c->cfg.num_layers, c->cfg.num_kv_heads, c->cfg.page_size,
-                                        c->cfg.head_dim / 8, c->cfg.num_pages, entry, st);
-        if (e != cudaSuccess) return cuda_fail(e, "copy-on-write launch");
-        c->launches++;
+    if (c->host_only) return PE_OK;
+    if (cow.p.n == kMaxSegs) {
+        pe_status s = cow.flush(c, st);
+        if (s != PE_OK) return s;
     }
+    CowCopy &x = cow.p.copies[cow.p.n++];
+    x.src = src;
+    x.dst = dst;
+    x.slots = static_cast<int32_t>(c->len[seq] % c->cfg.page_size);
+    x.entry = static_cast<int32_t>(static_cast<int64_t>(seq) * c->cfg.max_pages_per_seq + static_cast<int64_t>(t.size()) - 1);
     return PE_OK;
 }
 
@@ -538,8 +565,11 @@ pe_status apply_appends(pe_cache *c, const std::vector<AppendPlan> &plans, const
         p->n_total = static_cast<int32_t>(n_total);
     }
     int32_t pages_in_launch = 0;
+    CowList cow;
     auto flush = [&]() -> pe_status {
         if (p->n_segs == 0) return PE_OK;
+        pe_status cs = cow.flush(c, st);
+        if (cs != PE_OK) return cs;
         p->n_new = pages_in_launch;
         p->seg_tokens = p->segs[p->n_segs - 1].cum0 + p->segs[p->n_segs - 1].n_tokens;
         const int64_t chunks = static_cast<int64_t>(p->L) * p->seg_tokens * p->hkv * p->dvec;
@@ -556,7 +586,7 @@ pe_status apply_appends(pe_cache *c, const std::vector<AppendPlan> &plans, const
         // decided now, on the current references (the planners' page counts agree: settle_batch_cow)
         const std::vector<int32_t> &tt = c->table[pl.seq];
         if (pl.n > 0 && c->len[pl.seq] % ps != 0 && c->refs[tt.back()] > 1) {
-            pe_status s = apply_cow(c, pl.seq, st);
+            pe_status s = apply_cow(c, pl.seq, cow, st);
             if (s != PE_OK) return s;
         }
         int32_t done = 0;

@@ -48,6 +48,21 @@ struct AppendParamsT {
 };
 using AppendParams = AppendParamsT<kMaxSegs, kAppendMaxPages>;
 
+// ---------------------------------------------------------------- copy-on-write
+struct CowCopy {
+    int32_t src, dst;      // pages
+    int32_t slots;         // valid slots of the shared page
+    int32_t entry;         // index of the device table entry to point at dst
+};
+
+struct CowParams {
+    uint4 *k_pool;
+    uint4 *v_pool;
+    int32_t *page_table;
+    int32_t n, L, hkv, ps, dvec, num_pages;
+    CowCopy copies[kMaxSegs];
+};
+
 // ---------------------------------------------------------------- crop
 constexpr int kMaxCropFreed = 2048;  // freed page ids carried by one crop launch (debug poison)
 
@@ -196,11 +211,9 @@ cudaError_t launch_crop(const CropParams &p, cudaStream_t st);
 // the new sequence's device length.
 cudaError_t launch_table_copy(int32_t *page_table, int32_t src_row, int32_t dst_row, int32_t n, int64_t *seq_len,
                               int32_t dst_seq, int64_t len, cudaStream_t st);
-// Copy-on-write: copies slots [0, slots) of page src to page dst (every layer
-// and kv-head, K and V) and points the device table entry at dst.
-cudaError_t launch_cow_copy(uint4 *k_pool, uint4 *v_pool, int32_t src, int32_t dst, int32_t slots, int32_t L,
-                            int32_t hkv, int32_t ps, int32_t dvec, int32_t num_pages, int32_t *table_entry,
-                            cudaStream_t st);
+// Copy-on-write: copies slots [0, slots) of each copy's page src to its page dst
+// (every layer and kv-head, K and V) and points its device table entry at dst.
+cudaError_t launch_cow_copy(const CowParams &p, cudaStream_t st);
 // tm_o: the output as a map of the same shape as tm_q (full q-tiles are stored by TMA); unused when split
 cudaError_t launch_replay_attn(int head_dim, bool split, const CUtensorMap &tm_q, const CUtensorMap &tm_k,
                                const CUtensorMap &tm_v, const CUtensorMap &tm_o, const AttnParams &p, cudaStream_t st);

@@ -195,6 +195,7 @@ cudaError_t launch_crop(const CropParams &p, cudaStream_t st)
 __global__ void __launch_bounds__(256) table_copy_kernel(int32_t *page_table, int32_t src_row, int32_t dst_row,
                                                          int32_t n, int64_t *seq_len, int32_t dst_seq, int64_t len)
 {
+    ptx::griddep_wait();  // launched with programmatic serialization: only the launch overlaps the kernel before
     for (int i = threadIdx.x; i < n; i += blockDim.x) page_table[dst_row + i] = page_table[src_row + i];
     if (threadIdx.x == 0) seq_len[dst_seq] = len;
 }
@@ -202,32 +203,50 @@ __global__ void __launch_bounds__(256) table_copy_kernel(int32_t *page_table, in
 cudaError_t launch_table_copy(int32_t *page_table, int32_t src_row, int32_t dst_row, int32_t n, int64_t *seq_len,
                               int32_t dst_seq, int64_t len, cudaStream_t st)
 {
-    table_copy_kernel<<<1, 256, 0, st>>>(page_table, src_row, dst_row, n, seq_len, dst_seq, len);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, table_copy_kernel, page_table, src_row, dst_row, n, seq_len, dst_seq, len);
 }
 
-// Grid: (layer x kv-head) blocks; each copies `slots` rows of d (16-byte chunks).
-__global__ void __launch_bounds__(256) cow_copy_kernel(uint4 *k_pool, uint4 *v_pool, int32_t src, int32_t dst,
-                                                       int32_t slots, int32_t hkv, int32_t ps, int32_t dvec,
-                                                       int32_t num_pages, int32_t *table_entry)
+// The copies of one append call, one launch before its append launch: grid (layer x kv-head, copy), each
+// block `slots` rows of d (16-byte chunks).  A few KB each, so a launch's own time is what they cost: one
+// launch per forked sequence (7 of 8 branches: 3.3 us each, one after another) made them a tenth of a
+// made a replay of 8 branches 205 us; with one launch, overlapped (and the table copies of the forks), 153.
+__global__ void __launch_bounds__(128) cow_copy_kernel(const __grid_constant__ CowParams p)
 {
-    const int l = blockIdx.x / hkv;
-    const int h = blockIdx.x % hkv;
-    const int64_t s_base = ((static_cast<int64_t>(l) * num_pages + src) * hkv + h) * ps * dvec;
-    const int64_t d_base = ((static_cast<int64_t>(l) * num_pages + dst) * hkv + h) * ps * dvec;
-    for (int i = threadIdx.x; i < slots * dvec; i += blockDim.x) {
-        k_pool[d_base + i] = k_pool[s_base + i];
-        v_pool[d_base + i] = v_pool[s_base + i];
+    ptx::griddep_wait();  // launched with programmatic serialization
+    const CowCopy &c = p.copies[blockIdx.y];
+    const int l = blockIdx.x / p.hkv;
+    const int h = blockIdx.x % p.hkv;
+    const int64_t s_base = ((static_cast<int64_t>(l) * p.num_pages + c.src) * p.hkv + h) * p.ps * p.dvec;
+    const int64_t d_base = ((static_cast<int64_t>(l) * p.num_pages + c.dst) * p.hkv + h) * p.ps * p.dvec;
+    for (int i = threadIdx.x; i < c.slots * p.dvec; i += blockDim.x) {
+        p.k_pool[d_base + i] = p.k_pool[s_base + i];
+        p.v_pool[d_base + i] = p.v_pool[s_base + i];
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *table_entry = dst;
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.page_table[c.entry] = c.dst;
 }
 
-cudaError_t launch_cow_copy(uint4 *k_pool, uint4 *v_pool, int32_t src, int32_t dst, int32_t slots, int32_t L,
-                            int32_t hkv, int32_t ps, int32_t dvec, int32_t num_pages, int32_t *table_entry,
-                            cudaStream_t st)
+cudaError_t launch_cow_copy(const CowParams &p, cudaStream_t st)
 {
-    cow_copy_kernel<<<L * hkv, 256, 0, st>>>(k_pool, v_pool, src, dst, slots, hkv, ps, dvec, num_pages, table_entry);
-    return cudaGetLastError();
+    if (p.n <= 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(p.L * p.hkv), static_cast<unsigned>(p.n));
+    cfg.blockDim = dim3(128);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, cow_copy_kernel, p);
 }
 
 }  // namespace pe
