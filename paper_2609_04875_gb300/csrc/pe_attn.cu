@@ -9,7 +9,7 @@
 // One CTA computes one work item: (sequence, kv-head, pair of q-tiles[, key
 // split]).  A q-tile packs 128 rows = (128/g queries) x (g q-heads of one
 // kv-head), so each K/V tile brought into shared memory serves 2 x 128 rows.
-// Roles (320 threads):
+// Roles (320 threads; 352 at d = 64):
 //   warps 0-3, 4-7  softmax of q-tile 0 / q-tile 1: thread r owns row r
 //                   (TMEM lane r); masks, online softmax in fp32 (exp2),
 //                   writes P (bf16) back into TMEM (d = 128: over its S
@@ -21,7 +21,8 @@
 //   warp 9          MMA: allocates TMEM; the converged warp issues tcgen05.mma
 //                   (through one elected lane) for S_t = Q_t K^T (A, B from
 //                   shared memory) and O_t += P_t V (A = P from TMEM, B = V
-//                   from shared memory).
+//                   from shared memory).  At d = 64 warp 9 serves q-tile 0,
+//                   warp 10 q-tile 1.
 // Tensor-core order per key tile j (d = 128):  PV_0(j), S_0(j+1), PV_1(j),
 // S_1(j+1), so one softmax group works while the tensor core runs the other
 // group's GEMMs; S_t(j+1) waits for PV_t(j), which reads P_t(j) over S_t.
@@ -55,7 +56,9 @@
 namespace pe {
 
 constexpr float kTileSumLimit = 1.8446744e19f;  // 2^64: larger tile sums move the reference
-constexpr int kThreads = 320;
+// 8 softmax warps, the producer, and the MMA warps: one per q-tile at d = 64
+template <int HD>
+constexpr int kThreads = HD == 64 ? 352 : 320;
 
 template <int HD>
 struct AttnCfg {
@@ -73,6 +76,7 @@ struct AttnCfg {
     // TMEM columns: S_0, S_1 (128 each), O_0, O_1 (HD each); for d = 64 the 128 left over hold P_0 and
     // P_1 (64 each), so S(j+1) need not wait for the P V GEMM of tile j (P(j) lives apart from S)
     static constexpr bool kSepP = HD == 64;
+    static constexpr int kMmaWarps = HD == 64 ? 2 : 1;
     static constexpr int kOffMisc = kOffBar + kNumBars * 8;  // tmem slot, abort flag
     static constexpr int kSmemBytes = kOffMisc + 16;
     static constexpr int kDynSmem = kSmemBytes + 1024;       // alignment slack
@@ -90,7 +94,7 @@ struct TileGeo {
 };
 
 template <int HD, bool SPLIT>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads<HD>, 1)
     replay_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
                        const __grid_constant__ AttnParams p)
@@ -219,9 +223,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             ptx::mbar_init(b_q_full, 1);
             for (int s = 0; s < C::kStages; ++s) {
                 ptx::mbar_init(b_k_full + 8 * s, 1);
-                ptx::mbar_init(b_k_empty + 8 * s, 1);
+                ptx::mbar_init(b_k_empty + 8 * s, C::kMmaWarps);
                 ptx::mbar_init(b_v_full + 8 * s, 1);
-                ptx::mbar_init(b_v_empty + 8 * s, 1);
+                ptx::mbar_init(b_v_empty + 8 * s, C::kMmaWarps);
             }
             for (int t = 0; t < 2; ++t) {
                 ptx::mbar_init(b_s_full + 8 * t, 1);
@@ -299,7 +303,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                        ptx::globaltimer() - t0 < 4000000ull) {}
             }
         }
-    } else if (warp == 9 && n_all > 0) {
+    } else if (C::kMmaWarps == 1 && warp == 9 && n_all > 0) {
         // =================================================== MMA issuer (the whole warp; one elected lane issues)
         constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
         constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
@@ -321,7 +325,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         };
         auto issue_pv = [&](int t, int s, bool acc) {
             const uint64_t vd = v_desc + s * (C::kTileBytes >> 4);
-            const uint32_t tp = C::kSepP ? tm + 256 + 2 * HD + 64 * t : tm + 128 * t;  // P_t
+            const uint32_t tp = tm + 128 * t;  // P_t over S_t
 #pragma unroll
             for (int kk = 0; kk < kBN / 16; ++kk)
                 mma_bf16_ts_warp(tm + 256 + HD * t, tp + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
@@ -335,33 +339,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (n1 > 0) issue_s(1, 0);
             if (n0 > 0 || n1 > 0) mma_commit_warp(b_k_empty);
         }
-        for (int j = 0; ok && C::kSepP && j < n_mma; ++j) {
-            // d = 64: S_t(j+1) once the softmax holds S_t(j) in registers, P V_t(j) once P_t(j) is in
-            const int s = j % C::kStages;
-            const int s1 = (j + 1) % C::kStages;
-            const bool more = j + 1 < n_mma;
-            if (more && !wait_bar_warp(b_k_full + 8 * s1, ((j + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                if (j + 1 >= (t ? n1 : n0)) continue;
-                if (!wait_bar_warp(b_s_free + 8 * t, j & 1, wctx)) { ok = false; break; }
-                ptx::tc_fence_after();
-                issue_s(t, s1);
-            }
-            if (!ok) break;
-            if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
-            if (!wait_bar_warp(b_v_full + 8 * s, (j / C::kStages) & 1, wctx)) { ok = false; break; }
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                if (j >= (t ? n1 : n0)) continue;
-                if (!wait_bar_warp(b_p_full + 8 * t, j & 1, wctx)) { ok = false; break; }
-                ptx::tc_fence_after();
-                issue_pv(t, s, j > 0);
-            }
-            if (!ok) break;
-            mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its PV GEMMs
-        }
-        for (int j = 0; ok && !C::kSepP && j < n_mma; ++j) {
+        for (int j = 0; ok && j < n_mma; ++j) {
             const int s = j % C::kStages;
             const int s1 = (j + 1) % C::kStages;
             const bool more = j + 1 < n_mma;
@@ -382,6 +360,74 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (j + 1 < n1) issue_s(1, s1);
             if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
             mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its PV GEMMs
+        }
+    } else if (C::kMmaWarps == 2 && warp >= 9 && n_all > 0) {
+        // =================================================== MMA issuers, d = 64 (whole warps; one elected lane issues)
+        // Warp 9 + t runs q-tile t's GEMMs, so that neither q-tile waits in the issue order for the other's
+        // softmax, which is what bounds d = 64 (6-agent batch, two layers: 392 -> 375 us).  At d = 128, where the tensor pipe is the
+        // bound, two interleaved streams of MMAs cost 18 % (agent batch 1.77 -> 2.10 ms).  Key tiles that the
+        // q-tile does not attend are passed on unread.
+        constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
+        constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
+        // warp-uniform copies (every lane holds the same values already)
+        const int t = __shfl_sync(0xffffffffu, warp - 9, 0);
+        const int n = __shfl_sync(0xffffffffu, t ? geo[1].ntiles : geo[0].ntiles, 0);
+        const int n_mma = __shfl_sync(0xffffffffu, n_all, 0);
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024) + t * (C::kTileBytes >> 4);
+        const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
+        const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
+        const uint32_t tp = tm + 256 + 2 * HD + 64 * t;  // P_t
+        auto issue_s = [&](int s) {
+            const uint64_t kd = k_desc + s * (C::kTileBytes >> 4);
+#pragma unroll
+            for (int kk = 0; kk < HD / 16; ++kk) {
+                const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
+                mma_bf16_warp(tm + 128 * t, q_desc + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
+            }
+            mma_commit_warp(b_s_full + 8 * t);
+            mma_commit_warp(b_k_empty + 8 * s);  // K consumed by this q-tile
+        };
+        auto full = [&](uint32_t bar, int j) {
+            return wait_bar_warp(bar + 8 * (j % C::kStages), (j / C::kStages) & 1, wctx);
+        };
+        auto pass = [&](uint32_t bar, int j) {  // this q-tile does not use tile j
+            if (lane == 0) ptx::mbar_arrive(bar + 8 * (j % C::kStages));
+            __syncwarp();
+        };
+        bool ok = (n == 0 || wait_bar_warp(b_q_full, 0, wctx)) && full(b_k_full, 0);
+        if (ok && n > 0) {
+            ptx::tc_fence_after();
+            issue_s(0);
+        } else if (ok) {
+            pass(b_k_empty, 0);
+        }
+        for (int j = 0; ok && j < n_mma; ++j) {
+            if (j + 1 < n_mma) {
+                // S_t(j+1) once the softmax holds S_t(j) in registers
+                if (!full(b_k_full, j + 1)) break;
+                if (j + 1 < n) {
+                    if (!wait_bar_warp(b_s_free + 8 * t, j & 1, wctx)) break;
+                    ptx::tc_fence_after();
+                    issue_s((j + 1) % C::kStages);
+                } else {
+                    pass(b_k_empty, j + 1);
+                }
+            }
+            if (!full(b_v_full, j)) break;
+            if (j >= n) {
+                pass(b_v_empty, j);
+                continue;
+            }
+            if (!wait_bar_warp(b_p_full + 8 * t, j & 1, wctx)) break;
+            ptx::tc_fence_after();
+            const uint64_t vd = v_desc + (j % C::kStages) * (C::kTileBytes >> 4);
+#pragma unroll
+            for (int kk = 0; kk < kBN / 16; ++kk)
+                mma_bf16_ts_warp(tm + 256 + HD * t, tp + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
+                                 (j > 0 || kk > 0) ? 1u : 0u);
+            mma_commit_warp(b_o_done + 8 * t);
+            mma_commit_warp(b_v_empty + 8 * (j % C::kStages));  // V consumed by this q-tile
         }
     } else if (warp < 8) {
         // =================================================== softmax / epilogue
@@ -741,7 +787,7 @@ static cudaError_t launch_attn_t(const CUtensorMap &q, const CUtensorMap &k, con
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(p.total_items));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kThreads<HD>);
     cfg.dynamicSmemBytes = C::kDynSmem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
