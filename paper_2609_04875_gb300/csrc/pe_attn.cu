@@ -212,11 +212,10 @@ __global__ void __launch_bounds__(kThreads<HD>, 1)
         return true;
     };
     // Launched with programmatic serialization: the next kernel in the stream may
-    // start its set-up once every CTA of this grid has started (it waits for this
-    // grid's completion before touching memory), and this grid's set-up overlaps
-    // the previous kernel; griddepcontrol.wait comes before the first read of
+    // start its set-up once every CTA of this grid has issued its loads (it waits
+    // for this grid's completion before touching memory), and this grid's set-up
+    // overlaps the previous kernel; griddepcontrol.wait comes before the first read of
     // memory an earlier kernel wrote (page table, pool, Q) and before any write.
-    ptx::griddep_launch_dependents();
     int page_next = -1;
     if (warp == 8) {
         if (lane == 0) {
@@ -277,6 +276,9 @@ __global__ void __launch_bounds__(kThreads<HD>, 1)
             if (i + 1 < n_all) page_next = page_of(i + 1);  // prefetch the next tile's page ids
             if (!issue_kv(i, page)) break;
         }
+        // The next kernel's set-up may start once every CTA has issued its loads; let in at this grid's start
+        // it cost launches of a few microseconds 2 % (133-token episode of 32 layers 460 -> 450 us).
+        ptx::griddep_launch_dependents();
         // With one CTA per SM, the CTA that starts on this SM next is about blockIdx.x + next_stride:
         // bring its Q tiles (read once, from DRAM) into L2 now, so that its first S GEMMs wait less.
         const int nxt = blockIdx.x + p.next_stride;

@@ -217,8 +217,8 @@ cudaError_t launch_table_copy(int32_t *page_table, int32_t src_row, int32_t dst_
 
 // The copies of one append call, one launch before its append launch: grid (layer x kv-head, copy), each
 // block `slots` rows of d (16-byte chunks).  A few KB each, so a launch's own time is what they cost: one
-// launch per forked sequence (7 of 8 branches: 3.3 us each, one after another) made them a tenth of a
-// made a replay of 8 branches 205 us; with one launch, overlapped (and the table copies of the forks), 153.
+// launch per forked sequence (7 of 8 branches, 3.3 us each, one after another) made a replay of 8 branches
+// 205 us; one launch, overlapped like the forks' table copies with the kernel before it, 153 us.
 __global__ void __launch_bounds__(128) cow_copy_kernel(const __grid_constant__ CowParams p)
 {
     ptx::griddep_wait();  // launched with programmatic serialization
