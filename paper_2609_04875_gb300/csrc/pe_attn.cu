@@ -9,15 +9,19 @@
 // One CTA computes one work item: (sequence, kv-head, pair of q-tiles[, key
 // split]).  A q-tile packs 128 rows = (128/g queries) x (g q-heads of one
 // kv-head), so each K/V tile brought into shared memory serves 2 x 128 rows.
-// Roles (320 threads; 352 at d = 64):
+// Roles (352 threads, 352 or 384 at d = 64):
 //   warps 0-3, 4-7  softmax of q-tile 0 / q-tile 1: thread r owns row r
 //                   (TMEM lane r); masks, online softmax in fp32 (exp2),
 //                   writes P (bf16) back into TMEM (d = 128: over its S
 //                   columns; d = 64: into its own P columns), rescales O in
 //                   TMEM when needed, epilogue (a full q-tile's O goes to
 //                   shared memory, then out by one TMA store per 64 columns).
-//   warp 8          producer: reads the page table; its lanes issue one TMA
-//                   box per (page, 64-column half) into K and V stage rings.
+//   warp 8, last    producers of K (and Q), of V (at d = 64 one for both from
+//                   16-token pages on): each reads the page table;
+//                   its lanes issue one TMA box per (page, 64-column half)
+//                   into its stage ring.  A warp issues a box in about 30 ns
+//                   whatever its size, so one warp for both held back small
+//                   pages (8-token pages: 64 boxes a tile, 1.9 us).
 //   warp 9          MMA: allocates TMEM; the converged warp issues tcgen05.mma
 //                   (through one elected lane) for S_t = Q_t K^T (A, B from
 //                   shared memory) and O_t += P_t V (A = P from TMEM, B = V
@@ -56,9 +60,14 @@
 namespace pe {
 
 constexpr float kTileSumLimit = 1.8446744e19f;  // 2^64: larger tile sums move the reference
-// 8 softmax warps, the producer, and the MMA warps: one per q-tile at d = 64
-template <int HD>
-constexpr int kThreads = HD == 64 ? 352 : 320;
+// 8 softmax warps, the K producer, the MMA warps (one per q-tile at d = 64) and the V producer, if apart
+template <int HD, bool VAPART>
+constexpr int kThreads = 32 * (9 + (HD == 64 ? 2 : 1) + (VAPART ? 1 : 0));
+
+// Whether V has a producer warp of its own.  At d = 64 a tile has half the boxes, and from 16-token pages on
+// one warp issues them in time (d = 64 batch: 375 against 380 us with 32-token pages, 448 against 412 with
+// 8-token ones).
+constexpr bool v_apart(int head_dim, int page_size) { return head_dim == 128 || page_size < 16; }
 
 template <int HD>
 struct AttnCfg {
@@ -93,8 +102,8 @@ struct TileGeo {
     int ntiles;      // key tiles this q-tile processes (from kt0)
 };
 
-template <int HD, bool SPLIT>
-__global__ void __launch_bounds__(kThreads<HD>, 1)
+template <int HD, bool SPLIT, bool VAPART>
+__global__ void __launch_bounds__(kThreads<HD, VAPART>, 1)
     replay_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
                        const __grid_constant__ AttnParams p)
@@ -196,20 +205,23 @@ __global__ void __launch_bounds__(kThreads<HD>, 1)
         const int lp = (kt0 + i) * ppt + lane;
         return (lane < ppt && lp < sq.n_pages) ? p.page_table[sq.table_row + lp] : -1;
     };
-    auto issue_kv = [&](int i, int page) {      // all lanes: TMA boxes of key tile i into stage i % S
+    // all lanes: TMA boxes of key tile i's K (or V) into stage i % S
+    auto issue = [&](const CUtensorMap *map, uint32_t smem0, uint32_t b_full, uint32_t b_empty, int i, int page) {
         const int s = i % C::kStages;
         const int pg = __shfl_sync(0xffffffffu, page, op_page & 31);
         // rows of pages past the sequence read as zeros (out-of-bounds box)
         const int y = pg >= 0 ? ((p.layer * p.num_pages + pg) * p.hkv + kvh) * p.ps : p.oob_row;
-        if (i >= C::kStages && !wait_bar_warp(b_k_empty + 8 * s, ((i / C::kStages) - 1) & 1, wctx)) return false;
-        if (lane == 0) ptx::mbar_arrive_expect_tx(b_k_full + 8 * s, C::kTileBytes);
+        if (i >= C::kStages && !wait_bar_warp(b_empty + 8 * s, ((i / C::kStages) - 1) & 1, wctx)) return false;
+        if (lane == 0) ptx::mbar_arrive_expect_tx(b_full + 8 * s, C::kTileBytes);
         __syncwarp();
-        if (op_on) ptx::tma_load_2d(k_smem0 + s * C::kTileBytes + op_off, &tm_k, op_reg * 64, y, b_k_full + 8 * s);
-        if (i >= C::kStages && !wait_bar_warp(b_v_empty + 8 * s, ((i / C::kStages) - 1) & 1, wctx)) return false;
-        if (lane == 0) ptx::mbar_arrive_expect_tx(b_v_full + 8 * s, C::kTileBytes);
-        __syncwarp();
-        if (op_on) ptx::tma_load_2d(v_smem0 + s * C::kTileBytes + op_off, &tm_v, op_reg * 64, y, b_v_full + 8 * s);
+        if (op_on) ptx::tma_load_2d(smem0 + s * C::kTileBytes + op_off, map, op_reg * 64, y, b_full + 8 * s);
         return true;
+    };
+    auto drain = [&](uint32_t b_full, int issued) {  // after an abort: a bounded chance for copies in flight to land
+        const uint64_t t0 = ptx::globaltimer();
+        for (int i = max(0, issued - C::kStages); i < issued; ++i)
+            while (!ptx::mbar_try_wait(b_full + 8 * (i % C::kStages), (i / C::kStages) & 1) &&
+                   ptx::globaltimer() - t0 < 4000000ull) {}
     };
     // Launched with programmatic serialization: the next kernel in the stream may
     // start its set-up once every CTA of this grid has issued its loads (it waits
@@ -257,7 +269,8 @@ __global__ void __launch_bounds__(kThreads<HD>, 1)
         if (n_all > 0) {
             const int page = page_next;
             if (n_all > 1) page_next = page_of(1);
-            issue_kv(0, page);  // tile 0 never waits (its stage is fresh)
+            issue(&tm_k, k_smem0, b_k_full, b_k_empty, 0, page);  // tile 0 never waits (its stage is fresh)
+            if (!VAPART) issue(&tm_v, v_smem0, b_v_full, b_v_empty, 0, page);
         }
     }
     if (warp == 9) {
@@ -269,12 +282,26 @@ __global__ void __launch_bounds__(kThreads<HD>, 1)
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 8 && n_all > 0) {
-        // =================================================== producer (TMA), tiles 1..
-        for (int i = 1; i < n_all; ++i) {
+    constexpr int kWarpV = 9 + C::kMmaWarps;
+    if (VAPART && warp == kWarpV && n_all > 0) {
+        // =================================================== V producer (TMA)
+        ptx::griddep_wait();
+        int page = page_of(0), i = 0;
+        for (; i < n_all; ++i) {
+            const int next = i + 1 < n_all ? page_of(i + 1) : -1;
+            if (!issue(&tm_v, v_smem0, b_v_full, b_v_empty, i, page)) break;
+            page = next;
+        }
+        __syncwarp();
+        if (*abort_flag && lane == 0) drain(b_v_full, i);
+    } else if (warp == 8 && n_all > 0) {
+        // =================================================== K producer (TMA), tiles 1.. (and V's)
+        int i = 1, iv = 0;
+        for (; i < n_all; ++i) {
             const int page = page_next;
             if (i + 1 < n_all) page_next = page_of(i + 1);  // prefetch the next tile's page ids
-            if (!issue_kv(i, page)) break;
+            if (!issue(&tm_k, k_smem0, b_k_full, b_k_empty, i, page)) break;
+            if (!VAPART && !issue(&tm_v, v_smem0, b_v_full, b_v_empty, iv = i, page)) break;
         }
         // The next kernel's set-up may start once every CTA has issued its loads; let in at this grid's start
         // it cost launches of a few microseconds 2 % (133-token episode of 32 layers 460 -> 450 us).
@@ -295,15 +322,8 @@ __global__ void __launch_bounds__(kThreads<HD>, 1)
         }
         __syncwarp();
         if (*abort_flag && lane == 0) {
-            // give copies in flight a bounded chance to land before the CTA exits
-            const uint64_t t0 = ptx::globaltimer();
-            for (int i = max(0, n_all - C::kStages); i < n_all; ++i) {
-                const int s = i % C::kStages;
-                while (!ptx::mbar_try_wait(b_k_full + 8 * s, (i / C::kStages) & 1) &&
-                       ptx::globaltimer() - t0 < 2000000ull) {}
-                while (!ptx::mbar_try_wait(b_v_full + 8 * s, (i / C::kStages) & 1) &&
-                       ptx::globaltimer() - t0 < 4000000ull) {}
-            }
+            drain(b_k_full, i);
+            if (!VAPART) drain(b_v_full, iv + 1);
         }
     } else if (C::kMmaWarps == 1 && warp == 9 && n_all > 0) {
         // =================================================== MMA issuer (the whole warp; one elected lane issues)
@@ -363,7 +383,7 @@ __global__ void __launch_bounds__(kThreads<HD>, 1)
             if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
             mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its PV GEMMs
         }
-    } else if (C::kMmaWarps == 2 && warp >= 9 && n_all > 0) {
+    } else if (C::kMmaWarps == 2 && (warp == 9 || warp == 10) && n_all > 0) {
         // =================================================== MMA issuers, d = 64 (whole warps; one elected lane issues)
         // Warp 9 + t runs q-tile t's GEMMs, so that neither q-tile waits in the issue order for the other's
         // softmax, which is what bounds d = 64 (6-agent batch, two layers: 392 -> 375 us).  At d = 128, where the tensor pipe is the
@@ -779,17 +799,17 @@ cudaError_t static_scratch(float **ptr)
     return cudaSuccess;
 }
 
-template <int HD, bool SPLIT>
+template <int HD, bool SPLIT, bool VAPART>
 static cudaError_t launch_attn_t(const CUtensorMap &q, const CUtensorMap &k, const CUtensorMap &v,
                                  const CUtensorMap &o, const AttnParams &p, cudaStream_t st)
 {
     using C = AttnCfg<HD>;
     static std::atomic<uint64_t> configured{0};
-    cudaError_t e = set_dyn_smem_once(replay_attn_kernel<HD, SPLIT>, C::kDynSmem, configured);
+    cudaError_t e = set_dyn_smem_once(replay_attn_kernel<HD, SPLIT, VAPART>, C::kDynSmem, configured);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(p.total_items));
-    cfg.blockDim = dim3(kThreads<HD>);
+    cfg.blockDim = dim3(kThreads<HD, VAPART>);
     cfg.dynamicSmemBytes = C::kDynSmem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -797,7 +817,7 @@ static cudaError_t launch_attn_t(const CUtensorMap &q, const CUtensorMap &k, con
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, replay_attn_kernel<HD, SPLIT>, q, k, v, o, p);
+    return cudaLaunchKernelEx(&cfg, replay_attn_kernel<HD, SPLIT, VAPART>, q, k, v, o, p);
 }
 
 cudaError_t launch_replay_attn(int head_dim, bool split, const CUtensorMap &tm_q, const CUtensorMap &tm_k,
@@ -805,11 +825,14 @@ cudaError_t launch_replay_attn(int head_dim, bool split, const CUtensorMap &tm_q
 {
     if (p.total_items <= 0) return cudaSuccess;
     if (head_dim == 128)
-        return split ? launch_attn_t<128, true>(tm_q, tm_k, tm_v, tm_o, p, st)
-                     : launch_attn_t<128, false>(tm_q, tm_k, tm_v, tm_o, p, st);
+        return split ? launch_attn_t<128, true, true>(tm_q, tm_k, tm_v, tm_o, p, st)
+                     : launch_attn_t<128, false, true>(tm_q, tm_k, tm_v, tm_o, p, st);
+    if (head_dim == 64 && v_apart(64, p.ps))
+        return split ? launch_attn_t<64, true, true>(tm_q, tm_k, tm_v, tm_o, p, st)
+                     : launch_attn_t<64, false, true>(tm_q, tm_k, tm_v, tm_o, p, st);
     if (head_dim == 64)
-        return split ? launch_attn_t<64, true>(tm_q, tm_k, tm_v, tm_o, p, st)
-                     : launch_attn_t<64, false>(tm_q, tm_k, tm_v, tm_o, p, st);
+        return split ? launch_attn_t<64, true, false>(tm_q, tm_k, tm_v, tm_o, p, st)
+                     : launch_attn_t<64, false, false>(tm_q, tm_k, tm_v, tm_o, p, st);
     return cudaErrorInvalidValue;
 }
 

@@ -19,10 +19,10 @@
 // tile and epilogue run (no CTA launch, TMEM allocation or barrier set-up
 // between units).
 //
-// Roles (320 threads) as in replay_attn_kernel: softmax warpgroups 0 and 1
-// (one per q-tile, thread r owns row r), producer warp 8 (page table -> TMA
-// boxes), MMA warp 9 (converged; one elected lane issues tcgen05.mma).  Every role walks the
-// same sequence of pieces, computed from the kernel parameters; barrier phases
+// Roles (352 threads) as in replay_attn_kernel: softmax warpgroups 0 and 1
+// (one per q-tile, thread r owns row r), producer warps 8 (Q, K) and 10 (V)
+// (page table -> TMA boxes), MMA warp 9 (converged; one elected lane issues
+// tcgen05.mma).  Every role walks the same sequence of pieces, computed from the kernel parameters; barrier phases
 // run on across pieces (per q-tile tile counts for S / P / O, a global key
 // tile count for the K and V rings, a piece count for Q).  Two more barriers
 // than the one-unit kernel: q_empty (the piece's last S GEMMs are done, so the
@@ -44,7 +44,7 @@ namespace pe {
 namespace {
 
 constexpr float kTileSumLimit = 1.8446744e19f;  // 2^64: larger tile sums move the reference
-constexpr int kThreads = 320;
+constexpr int kThreads = 352;
 
 template <int HD>
 struct SkCfg {
@@ -359,17 +359,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 8) {
-        // =================================================== producer (TMA)
+    if (warp == 8 || warp == 10) {
+        // =================================================== producers (TMA): warp 8 Q and K, warp 10 V.  A warp
+        // issues a box in about 30 ns whatever its size, so one warp for both held back small pages (8-token
+        // pages: 64 boxes a tile).
         ptx::griddep_wait();  // page table, pool and Q were written by earlier kernels
+        const bool is_v = warp == 10;
+        const CUtensorMap *map = is_v ? &tm_v : &tm_k;
+        const uint32_t smem0 = is_v ? v_smem0 : k_smem0;
+        const uint32_t b_full = is_v ? b_v_full : b_k_full, b_empty = is_v ? b_v_empty : b_k_empty;
         const int ppt = kBN / p.ps;                 // pages per key tile
         const int n_ops = ppt * C::kRegions;        // TMA boxes per K (or V) tile, <= 32
         const int op_page = lane / C::kRegions;     // this lane's box: page index and half
         const int op_reg = lane % C::kRegions;
         const bool op_on = lane < n_ops;
         const uint32_t op_off = op_reg * C::kRegionBytes + op_page * p.ps * 128;
-        int gk = 0;        // key tiles issued so far (K / V ring position)
-        int q_issued = 0;  // Q loads issued so far
+        int gk = 0;        // key tiles issued so far (ring position)
+        int q_issued = 0;  // pieces so far (Q loads issued)
         bool ok = true;
         Piece pc;
         UnitGeo U;
@@ -381,17 +387,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                 return (lane < ppt && lp < sq.n_pages) ? p.page_table[sq.table_row + lp] : -1;
             };
             int page_next = page_of(pc.lo);  // read while the previous piece's last S GEMMs run
-            // Q of this piece once the previous piece's S GEMMs have read theirs
-            if (q_issued > 0 && !wait_bar_warp(b_q_empty, (q_issued - 1) & 1, wctx)) { ok = false; break; }
-            if (lane == 0) {
-                const int nq = two ? 2 : 1;
-                ptx::mbar_arrive_expect_tx(b_q_full, nq * C::kTileBytes);
-                for (int t = 0; t < nq; ++t)
-                    for (int r = 0; r < C::kRegions; ++r)
-                        ptx::tma_load_3d(q_smem + t * C::kTileBytes + r * C::kRegionBytes, &tm_q, r * 64,
-                                         U.kvh * g, sq.q_row0 + (2 * U.pair + t) * (kBM / g), b_q_full);
+            if (!is_v) {
+                // Q of this piece once the previous piece's S GEMMs have read theirs
+                if (q_issued > 0 && !wait_bar_warp(b_q_empty, (q_issued - 1) & 1, wctx)) { ok = false; break; }
+                if (lane == 0) {
+                    const int nq = two ? 2 : 1;
+                    ptx::mbar_arrive_expect_tx(b_q_full, nq * C::kTileBytes);
+                    for (int t = 0; t < nq; ++t)
+                        for (int r = 0; r < C::kRegions; ++r)
+                            ptx::tma_load_3d(q_smem + t * C::kTileBytes + r * C::kRegionBytes, &tm_q, r * 64,
+                                             U.kvh * g, sq.q_row0 + (2 * U.pair + t) * (kBM / g), b_q_full);
+                }
+                __syncwarp();
             }
-            __syncwarp();
             ++q_issued;
             for (int kt = pc.lo; kt < pc.hi; ++kt, ++gk) {
                 const int page = page_next;
@@ -400,37 +408,24 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int pg = __shfl_sync(0xffffffffu, page, op_page & 31);
                 // rows of pages past the sequence read as zeros (out-of-bounds box)
                 const int y = pg >= 0 ? ((p.layer * p.num_pages + pg) * p.hkv + U.kvh) * p.ps : p.oob_row;
-                if (gk >= C::kStages && !wait_bar_warp(b_k_empty + 8 * s, ((gk / C::kStages) - 1) & 1, wctx)) {
+                if (gk >= C::kStages && !wait_bar_warp(b_empty + 8 * s, ((gk / C::kStages) - 1) & 1, wctx)) {
                     ok = false;
                     break;
                 }
-                if (lane == 0) ptx::mbar_arrive_expect_tx(b_k_full + 8 * s, C::kTileBytes);
+                if (lane == 0) ptx::mbar_arrive_expect_tx(b_full + 8 * s, C::kTileBytes);
                 __syncwarp();
-                if (op_on)
-                    ptx::tma_load_2d(k_smem0 + s * C::kTileBytes + op_off, &tm_k, op_reg * 64, y, b_k_full + 8 * s);
-                if (gk >= C::kStages && !wait_bar_warp(b_v_empty + 8 * s, ((gk / C::kStages) - 1) & 1, wctx)) {
-                    ok = false;
-                    break;
-                }
-                if (lane == 0) ptx::mbar_arrive_expect_tx(b_v_full + 8 * s, C::kTileBytes);
-                __syncwarp();
-                if (op_on)
-                    ptx::tma_load_2d(v_smem0 + s * C::kTileBytes + op_off, &tm_v, op_reg * 64, y, b_v_full + 8 * s);
+                if (op_on) ptx::tma_load_2d(smem0 + s * C::kTileBytes + op_off, map, op_reg * 64, y, b_full + 8 * s);
             }
         }
         __syncwarp();
         if (!ok && lane == 0) {
             // give copies in flight a bounded chance to land before the CTA exits
             const uint64_t t0 = ptx::globaltimer();
-            if (q_issued > 0)
+            if (!is_v && q_issued > 0)
                 while (!ptx::mbar_try_wait(b_q_full, (q_issued - 1) & 1) && ptx::globaltimer() - t0 < 2000000ull) {}
-            for (int i = max(0, gk - C::kStages); i <= gk && i >= 0; ++i) {
-                const int s = i % C::kStages;
-                while (!ptx::mbar_try_wait(b_k_full + 8 * s, (i / C::kStages) & 1) &&
+            for (int i = max(0, gk - C::kStages); i < gk; ++i)
+                while (!ptx::mbar_try_wait(b_full + 8 * (i % C::kStages), (i / C::kStages) & 1) &&
                        ptx::globaltimer() - t0 < 4000000ull) {}
-                while (!ptx::mbar_try_wait(b_v_full + 8 * s, (i / C::kStages) & 1) &&
-                       ptx::globaltimer() - t0 < 6000000ull) {}
-            }
         }
     } else if (warp == 9) {
         // =================================================== MMA issuer (the whole warp; one elected lane issues)
