@@ -46,14 +46,14 @@ namespace {
 constexpr float kTileSumLimit = 1.8446744e19f;  // 2^64: larger tile sums move the reference
 constexpr int kThreads = 352;
 
-template <int HD>
+template <int HD, bool ONE>
 struct SkCfg {
     static constexpr int kRegions = HD / 64;            // 128-byte swizzle atoms along d
     static constexpr int kTileBytes = kBM * HD * 2;     // one Q, K or V tile (128 rows)
     static constexpr int kRegionBytes = kBM * 128;      // 128 rows x 128 bytes
-    static constexpr int kStages = (HD == 128) ? 2 : 3; // K ring and V ring depth
-    static constexpr int kOffQ = 0;                     // Q_0, Q_1
-    static constexpr int kOffK = kOffQ + 2 * kTileBytes;
+    static constexpr int kStages = (HD == 128) ? 2 : 3; // K ring and V ring depth (ONE: 3 of 32 KB: 1 % slower)
+    static constexpr int kOffQ = 0;                     // Q_0, Q_1 (ONE: Q_0)
+    static constexpr int kOffK = kOffQ + (ONE ? 1 : 2) * kTileBytes;
     static constexpr int kOffV = kOffK + kStages * kTileBytes;
     static constexpr int kOffBar = kOffV + kStages * kTileBytes;
     // q_full, q_empty, k_full[S], k_empty[S], v_full[S], v_empty[S], s_full[2], p_full[2], o_done[2], o_free[2]
@@ -288,12 +288,16 @@ __device__ __noinline__ void merge_own_row(const SkParams &P, int slot, int t, i
     }
 }
 
-template <int HD>
+// ONE: every unit of the launch is one q-tile (suffixes of at most 128 rows per kv-head): its key tiles
+// alternate between the two S buffers, so that S(j+1) runs during the softmax of tile j.  A kernel of its
+// own, because both forms in one cost the two-q-tile launches 1 % (d = 64: 7 %).  Short suffix (8 x 16 tokens
+// on 32k, HBM-bound) 181 -> 175 us, at d = 64 133 -> 104 us.
+template <int HD, bool ONE>
 __global__ void __launch_bounds__(kThreads, 1)
     replay_attn_sk_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                           const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ SkParams P)
 {
-    using C = SkCfg<HD>;
+    using C = SkCfg<HD, ONE>;
     const AttnParams &p = P.a;
     const SkCta &cw = P.cta[blockIdx.x];
     extern __shared__ uint8_t smem_raw[];
@@ -435,25 +439,27 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024);
         const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
         const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
-        auto issue_s = [&](int t, int s) {
+        // q-tile t, S (and P) buffer b
+        auto issue_s = [&](int t, int b, int s) {
             const uint64_t qd = q_desc + t * (C::kTileBytes >> 4), kd = k_desc + s * (C::kTileBytes >> 4);
 #pragma unroll
             for (int kk = 0; kk < HD / 16; ++kk) {
                 const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
-                mma_bf16_warp(tm + 128 * t, qd + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
+                mma_bf16_warp(tm + 128 * b, qd + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
             }
-            mma_commit_warp(b_s_full + 8 * t);
+            mma_commit_warp(b_s_full + 8 * b);
         };
-        auto issue_pv = [&](int t, int s, bool acc) {
+        auto issue_pv = [&](int t, int b, int s, bool acc) {
             const uint64_t vd = v_desc + s * (C::kTileBytes >> 4);
 #pragma unroll
             for (int kk = 0; kk < kBN / 16; ++kk)
-                mma_bf16_ts_warp(tm + 256 + HD * t, tm + 128 * t + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
+                mma_bf16_ts_warp(tm + 256 + HD * t, tm + 128 * b + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
                                  (acc || kk > 0) ? 1u : 0u);
-            mma_commit_warp(b_o_done + 8 * t);
+            mma_commit_warp(b_o_done + 8 * (ONE ? b : t));
         };
         int gk = 0;              // key tiles consumed so far (ring position)
-        int cnt0 = 0, cnt1 = 0;  // tiles of q-tile 0 / 1 in earlier pieces (S, P, O phases)
+        int cnt0 = 0, cnt1 = 0;  // tiles of q-tile 0 / 1 in earlier pieces (S and P phases)
+        uint32_t ph = 0;         // (ONE) bit b: parity of the uses of S buffer b in earlier pieces
         int seg0 = 0, seg1 = 0;  // earlier pieces in which q-tile 0 / 1 had tiles (o_free phase)
         bool ok = true;
         Piece pc;
@@ -470,9 +476,45 @@ __global__ void __launch_bounds__(kThreads, 1)
                 break;
             }
             ptx::tc_fence_after();
+            if (ONE) {
+                // S(j+1) runs during the softmax of tile j, in the other buffer; S(j+2) goes behind P V(j), which
+                // reads P(j) over S(j)
+                auto k_full = [&](int j) {
+                    return wait_bar_warp(b_k_full + 8 * ((gk + j) % C::kStages), ((gk + j) / C::kStages) & 1, wctx);
+                };
+                auto s_tile = [&](int j) {
+                    issue_s(0, j & 1, (gk + j) % C::kStages);
+                    mma_commit_warp(b_k_empty + 8 * ((gk + j) % C::kStages));
+                    if (j + 1 == n_all) mma_commit_warp(b_q_empty);
+                };
+                s_tile(0);
+                if (n_all > 1) {
+                    if (!k_full(1)) { ok = false; break; }
+                    ptx::tc_fence_after();
+                    s_tile(1);
+                }
+                for (int j = 0; j < n_all; ++j) {
+                    const int s = (gk + j) % C::kStages;
+                    if (!wait_bar_warp(b_v_full + 8 * s, ((gk + j) / C::kStages) & 1, wctx)) { ok = false; break; }
+                    if (j == 0 && seg0 > 0 && !wait_bar_warp(b_o_free, (seg0 - 1) & 1, wctx)) { ok = false; break; }
+                    if (!wait_bar_warp(b_p_full + 8 * (j & 1), ((ph >> (j & 1)) + (j >> 1)) & 1, wctx)) { ok = false; break; }
+                    ptx::tc_fence_after();
+                    issue_pv(0, j & 1, s, j > 0);
+                    mma_commit_warp(b_v_empty + 8 * s);
+                    if (j + 2 < n_all) {
+                        if (!k_full(j + 2)) { ok = false; break; }
+                        ptx::tc_fence_after();
+                        s_tile(j + 2);
+                    }
+                }
+                gk += n_all;
+                ph ^= (((n_all + 1) / 2) & 1) | ((n_all / 2 & 1) << 1);
+                seg0 += 1;
+                continue;
+            }
             const int n_s = max(n0, n1);  // key tiles with S GEMMs; Q is free after the last one
-            if (n0 > 0) issue_s(0, gk % C::kStages);
-            if (n1 > 0) issue_s(1, gk % C::kStages);
+            if (n0 > 0) issue_s(0, 0, gk % C::kStages);
+            if (n1 > 0) issue_s(1, 1, gk % C::kStages);
             mma_commit_warp(b_k_empty + 8 * (gk % C::kStages));
             if (n_s <= 1) mma_commit_warp(b_q_empty);
             for (int j = 0; j < n_all; ++j) {
@@ -486,18 +528,18 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (j == 0 && seg0 > 0 && !wait_bar_warp(b_o_free, (seg0 - 1) & 1, wctx)) { ok = false; break; }
                     if (!wait_bar_warp(b_p_full, (cnt0 + j) & 1, wctx)) { ok = false; break; }
                     ptx::tc_fence_after();
-                    issue_pv(0, s, j > 0);
+                    issue_pv(0, 0, s, j > 0);
                 }
                 if (more && !wait_bar_warp(b_k_full + 8 * s1, ((gj + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
                 ptx::tc_fence_after();
-                if (j + 1 < n0) issue_s(0, s1);
+                if (j + 1 < n0) issue_s(0, 0, s1);
                 if (j < n1) {
                     if (j == 0 && seg1 > 0 && !wait_bar_warp(b_o_free + 8, (seg1 - 1) & 1, wctx)) { ok = false; break; }
                     if (!wait_bar_warp(b_p_full + 8, (cnt1 + j) & 1, wctx)) { ok = false; break; }
                     ptx::tc_fence_after();
-                    issue_pv(1, s, j > 0);
+                    issue_pv(1, 1, s, j > 0);
                 }
-                if (j + 1 < n1) issue_s(1, s1);
+                if (j + 1 < n1) issue_s(1, 1, s1);
                 if (j + 2 == n_s) mma_commit_warp(b_q_empty);    // the piece's last S GEMMs read Q
                 if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
                 mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its P V GEMMs
@@ -514,13 +556,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int t = warp >> 2;                 // q-tile of this warpgroup
         const int row = threadIdx.x & 127;       // TMEM lane
         const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
-        const uint32_t tS = tmem + 128 * t + lane_off;
         const uint32_t tO = tmem + 256 + HD * t + lane_off;
-        const uint32_t b_s = b_s_full + 8 * t, b_p = b_p_full + 8 * t, b_o = b_o_done + 8 * t;
         const uint32_t b_f = b_o_free + 8 * t;
         const float sl2 = p.scale_log2;
         const float2 sl2x2 = make_float2(sl2, sl2);
-        int cnt = 0;  // tiles of this q-tile in earlier pieces (S, P, O phases)
+        int cnt = 0;             // tiles of this q-tile in earlier pieces (O phases, and S, P unless ONE)
+        uint32_t ph = 0;         // (ONE) bit b: parity of the uses of S buffer b in earlier pieces
         bool ok = true;
         Piece pc;
         UnitGeo U;
@@ -530,11 +571,20 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int qi = G.q_first + row / g;
             const bool valid = G.qt >= 0 && qi <= G.q_last;
             const int pos = sq.n_keys - sq.n_q + qi;
+            // P V of tile j (ONE: a barrier per buffer, or with the softmax up to two tiles ahead of P V the parity
+            // of a wait could be that of an earlier phase; S(j + 2) is behind P V(j))
+            auto pv_done = [&](int j) {
+                return ONE ? wait_bar_warp(b_o_done + 8 * (j & 1), ((ph >> (j & 1)) + (j >> 1)) & 1, wctx)
+                           : wait_bar_warp(b_o_done + 8 * t, (cnt + j) & 1, wctx);
+            };
             float m_ref = -INFINITY;
             float l = 0.f;
             for (int j = 0; j < G.ntiles; ++j) {
                 const int kbase = (pc.lo + j) * kBN;
-                if (!wait_bar_warp(b_s, (cnt + j) & 1, wctx)) { ok = false; break; }
+                // S buffer: the q-tile's own, or by tile parity
+                const uint32_t tS = ONE ? tmem + 128 * (j & 1) + lane_off : tmem + 128 * t + lane_off;
+                const uint32_t b_s = ONE ? b_s_full + 8 * (j & 1) : b_s_full + 8 * t;
+                if (!wait_bar_warp(b_s, (ONE ? (ph >> (j & 1)) + (j >> 1) : cnt + j) & 1, wctx)) { ok = false; break; }
                 ptx::tc_fence_after();
                 float s[kBN];
                 {
@@ -596,7 +646,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         m_ref = (m_new == -INFINITY) ? 0.f : m_new;
                     } else {
                         // O holds P V of this piece's tiles < j once P V(j-1) completed
-                        if (!wait_bar_warp(b_o, (cnt + j - 1) & 1, wctx)) { ok = false; break; }
+                        if (!pv_done(j - 1)) { ok = false; break; }
                         ptx::tc_fence_after();
                         const float alpha = need ? ex2(m_ref - m_new) : 1.0f;
 #pragma unroll 1
@@ -619,7 +669,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 l += rs;
                 ptx::tmem_wait_st();
                 ptx::tc_fence_before();
-                ptx::mbar_arrive(b_p);
+                ptx::mbar_arrive(ONE ? b_p_full + 8 * (j & 1) : b_p_full + 8 * t);
             }
             if (!ok) break;
             if (pc.slot >= P.n_slots || pc.part >= P.max_parts) {  // a plan outside the workspace: never write
@@ -655,7 +705,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             if (G.ntiles > 0) {
                 // ---- epilogue: O / l, bf16 output or fp32 partial
-                if (!wait_bar_warp(b_o, (cnt + G.ntiles - 1) & 1, wctx)) { ok = false; break; }
+                if (!pv_done(G.ntiles - 1)) { ok = false; break; }
                 ptx::tc_fence_after();
                 const float inv = l > 0.f ? 1.0f / l : 0.f;
                 if (pc.slot == -1) {
@@ -723,6 +773,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
             cnt += G.ntiles;
+            if (ONE) ph ^= (((G.ntiles + 1) / 2) & 1) | ((G.ntiles / 2 & 1) << 1);
         }
     }
 
@@ -734,13 +785,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-template <int HD>
+template <int HD, bool ONE>
 cudaError_t launch_sk_t(const CUtensorMap &q, const CUtensorMap &k, const CUtensorMap &v, const SkParams &p,
                         cudaStream_t st)
 {
-    using C = SkCfg<HD>;
+    using C = SkCfg<HD, ONE>;
     static std::atomic<uint64_t> configured{0};
-    cudaError_t e = set_dyn_smem_once(replay_attn_sk_kernel<HD>, C::kDynSmem, configured);
+    cudaError_t e = set_dyn_smem_once(replay_attn_sk_kernel<HD, ONE>, C::kDynSmem, configured);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(p.n_ctas));
@@ -752,7 +803,7 @@ cudaError_t launch_sk_t(const CUtensorMap &q, const CUtensorMap &k, const CUtens
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, replay_attn_sk_kernel<HD>, q, k, v, p);
+    return cudaLaunchKernelEx(&cfg, replay_attn_sk_kernel<HD, ONE>, q, k, v, p);
 }
 
 }  // namespace
@@ -762,8 +813,12 @@ cudaError_t launch_replay_attn_sk(int head_dim, const CUtensorMap &tm_q, const C
 {
     if (p.n_ctas <= 0) return cudaSuccess;
     if (p.n_ctas > kMaxSkCtas) return cudaErrorInvalidValue;
-    if (head_dim == 128) return launch_sk_t<128>(tm_q, tm_k, tm_v, p, st);
-    if (head_dim == 64) return launch_sk_t<64>(tm_q, tm_k, tm_v, p, st);
+    bool one = true;  // every unit is one q-tile
+    for (int32_t i = 0; i < p.a.n_seqs; ++i) one = one && p.a.seqs[i].n_qtiles == 1;
+    if (head_dim == 128)
+        return one ? launch_sk_t<128, true>(tm_q, tm_k, tm_v, p, st) : launch_sk_t<128, false>(tm_q, tm_k, tm_v, p, st);
+    if (head_dim == 64)
+        return one ? launch_sk_t<64, true>(tm_q, tm_k, tm_v, p, st) : launch_sk_t<64, false>(tm_q, tm_k, tm_v, p, st);
     return cudaErrorInvalidValue;
 }
 
