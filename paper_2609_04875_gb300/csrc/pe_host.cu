@@ -1147,6 +1147,9 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
 
     // split-KV decision over the whole launch group; plan_est: the cost model's time of the plan
     double plan_est = 0.0;
+    // the group's units (pairs of q-tiles x kv-heads), their key tiles, and whether every unit is one q-tile
+    int64_t grp_units = 0, grp_tiles = 0;
+    bool grp_lone = false;
     // time of one key tile per CTA in the cost models: about 1.5 us, compute- or HBM-bound alike; 1 us at
     // d = 64, whose next S GEMM overlaps the softmax
     const double tile_s = d == 64 ? 1.0e-6 : 1.5e-6;
@@ -1196,6 +1199,9 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         }
         if (splitkv != 0 && c->num_splits > 0) best = c->num_splits;
         plan_est = cost(best);
+        grp_units = C;
+        grp_tiles = tiles;
+        grp_lone = rows == C * kBM;
         int split_tiles = static_cast<int>(max_tiles);
         split = best > 1 || splitkv == 1;
         if (split) split_tiles = static_cast<int>(std::max<int64_t>(1, ceil_div(max_tiles, std::max<int64_t>(best, 1))));
@@ -1267,6 +1273,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
     // waves.  Chosen by the same cost model, when it beats the group's plan by 5 %.
     struct TailPlan {
         int64_t pairs = 0, splits = 0, split_tiles = 0, qtiles = 0;
+        double est = 0.0;  // estimated time of both launches
     };
     auto plan_tail = [&](const AttnItem &it, TailPlan &tp) -> bool {
         const int64_t len = c->len[it.seq];
@@ -1300,6 +1307,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
             }
         }
         if (tp.splits == 0 || best_t > 0.95 * plan_est) return false;
+        tp.est = best_t;
         tp.pairs = cut;
         tp.qtiles = qt_b;
         tp.split_tiles = ceil_div(ktiles, tp.splits);
@@ -1315,22 +1323,36 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         if (s != PE_OK) return s;
         TailPlan tp;
         const bool tail = hi - lo == 1 && c->splitkv == -1 && c->num_splits == 0 && plan_tail(order[lo], tp);
-        // The persistent stream-K kernel where the one-item plan leaves SMs idle (it needs key splits
-        // or a tail launch) and its units fill between a quarter of the SMs and two waves: one CTA
-        // per SM, whole units in rounds, the rest cut into equal stretches.  Elsewhere the one-item
-        // kernel, whose tile loop runs a little faster (measured: short suffix 195 -> 184 us and
-        // tau/T 0.9 311 -> 303 us with the persistent kernel; tau/T 0.7 716 -> 749 us and the
-        // 8-unit tiny launch 14 -> 16 us without it).
-        int64_t units = 0;
-        for (size_t i = lo; i < hi; ++i)
-            units += ceil_div(ceil_div(static_cast<int64_t>(order[i].n_q) * g, kBM), 2) * hkv;
-        const bool sk_fits = 4 * units >= c->num_sms && units < 2 * static_cast<int64_t>(c->num_sms);
-        const bool sk = c->num_splits == 0 &&
-                        (c->attn_kernel == 2 || (c->attn_kernel == 1 && (split || tail) && sk_fits));
+        // The persistent stream-K kernel where it should beat the one-item plan, among launches whose units
+        // fill between a quarter of the SMs and two waves.  One CTA per SM takes an equal stretch of key
+        // tiles, at a slightly longer tile and a longer start and end (the parts of cut units are merged by
+        // single warps, about 2 us a part), so it wins where the one-item plan leaves SMs idle for long:
+        // its estimate is linear in the key tiles per SM.  Measured, d = 128, one-item / persistent us a
+        // layer: 64 units of one q-tile 21 / 27 at 7 tiles per SM, 51 / 58 at 27, 174 / 171 at 108; 64
+        // pairs 36 / 42 at 13, 182 / 174 at 108; 168 pairs 152 / 124 at 70 (key splits).  d = 64, whose pair
+        // tiles the one-item kernel runs 20 % faster: 64 units of one q-tile 23 / 27 at 13, 114 / 100 at
+        // 108; 64 pairs 27 / 33 at 13, 137 / 149 at 108; 256 pairs 492 / 536 at 419 (tail launch).  A plan
+        // in one pass is left only for a clear gain, a last wave nearly empty: 168 pairs of 32 tiles 93 / 72
+        // (d = 64: 68 / 59).
+        const bool sk_fits = 4 * grp_units >= c->num_sms && grp_units < 2 * static_cast<int64_t>(c->num_sms);
+        const double sk_tile = d == 64 ? (grp_lone ? 0.77e-6 : 1.23e-6) : (grp_lone ? 1.38e-6 : 1.45e-6);
+        const double sk_fixed =
+            d == 64 ? 17e-6 : 1e-6 + 5e-6 * std::max(4.0, 1.0 + static_cast<double>(c->num_sms) / std::max<int64_t>(grp_units, 1));
+        const double sk_est = sk_fixed + sk_tile * static_cast<double>(grp_tiles) / c->num_sms;
+        // (the cost model's estimates of these launches come out 3 to 8 % high at d = 128)
+        const double one_est = (tail ? tp.est : plan_est) * (d == 64 ? 1.0 : 0.95);
+        const bool one_pass = !split && !tail;
+        const bool sk_wins = sk_fits && !(one_pass && c->splitkv == 0) && sk_est <= (one_pass ? 0.9 : 1.0) * one_est;
+        bool sk = c->num_splits == 0 && (c->attn_kernel == 2 || (c->attn_kernel == 1 && sk_wins));
         if (sk) {
             if (sbuf.empty()) sbuf.resize(sizeof(SkParams));
             SkParams &P = *reinterpret_cast<SkParams *>(sbuf.data());
             if ((s = plan_sk(c, order, lo, hi, layer, out, hq, scale, P)) != PE_OK) return s;
+            // no unit cut (the workspace is too small for the parts): nothing gained over the one pass
+            if (c->attn_kernel == 1 && one_pass && P.n_slots == 0) sk = false;
+        }
+        if (sk) {
+            SkParams &P = *reinterpret_cast<SkParams *>(sbuf.data());
             c->last_split = P.n_slots > 0 ? 1 : 0;
             c->last_splits = P.max_parts;
             c->last_ctas = P.n_ctas;
