@@ -51,6 +51,7 @@
 // all roles leave their loops, and TMEM is freed before exit.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "dev_common.cuh"
@@ -744,15 +745,21 @@ cudaError_t launch_bounded_wait_selftest(int32_t *status, uint64_t limit_ns, cud
     return cudaGetLastError();
 }
 
-// LSE-weighted merge of the split partials: one warp per 32 rows (a row block of the partials) and 32
+// LSE-weighted merge of the split partials: one warp per 32 rows (a row block of the partials) and kCombCols
 // columns, lane i on row 32 w + i, so every load of a split's chunk is 512 contiguous bytes.  For each
 // row, in split order: w_s = 2^(lse_s - max lse), den += w_s, acc += w_s O_s.
-template <int HD>
+// Bound by the latency of its round trips -- batches of kCombBatch splits, every load of a batch in flight at
+// once, against a running maximum -- and by what one SM takes from L2 (a warp's batch is 16 KB), so the work is
+// spread over every SM (launch_combine_t).  Up to 4 splits 32 columns a warp, else 16 columns and batches of 8:
+// one agent's 30 tokens on 5.3k, 14 splits, 16.3 -> 12.4 us a layer with its attention, 133 on 12k, 6 splits,
+// 34.0 -> 31.1; with 16 columns, 3 splits of 2 agents x 133 tokens took 17.2 us a layer, with 32 15.5.
+template <int HD, int kCombCols, int kCombBatch>
 __global__ void __launch_bounds__(256) splitkv_combine_kernel(const __grid_constant__ AttnParams p)
 {
     // launched with programmatic serialization after the attention grid: the item is found before the
     // wait for its partials, and the next kernel may start its own set-up during the merge
-    constexpr int kGroups = HD / 32;  // column groups of 32 (8 chunks of 16 bytes)
+    constexpr int kGroups = HD / kCombCols;  // column groups
+    constexpr int kChunks = kCombCols / 4;   // 16-byte chunks of one
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int blk = gw / kGroups, cg = gw % kGroups;
@@ -772,58 +779,60 @@ __global__ void __launch_bounds__(256) splitkv_combine_kernel(const __grid_const
     const int ns = sq.n_splits;
     ptx::griddep_wait();
     ptx::griddep_launch_dependents();
-    // Bound by the latency of its round trips: batches of kB splits, every load of a batch in flight at
-    // once, against a running maximum.  (Taking the maximum first and then the splits two at a time, a
-    // 4-split merge of 532 rows x 8 kv-heads cost 2 us more: 32 layers of it 530 -> 458 us.)
-    constexpr int kB = 4;
+    if (qi >= sq.n_q) return;
     float mx = -INFINITY, den = 0.f;
-    float acc[32];
+    float4 acc[kChunks];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-    for (int s0 = 0; s0 < ns; s0 += kB) {
-        float lse[kB];
-        float4 v[kB][8];
+    for (int k = 0; k < kChunks; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < ns; s0 += kCombBatch) {
+        float lse[kCombBatch];
+        float4 v[kCombBatch][kChunks];
 #pragma unroll
-        for (int u = 0; u < kB; ++u) {
-            const int64_t r = base + static_cast<int64_t>(min(s0 + u, ns - 1)) * kBM;
-            lse[u] = s0 + u < ns ? __ldcg(p.part_lse + r) : -INFINITY;
+        for (int u = 0; u < kCombBatch; ++u) {
+            const int64_t r = base + static_cast<int64_t>(s0 + u) * kBM;
+            const bool in = s0 + u < ns;
+            lse[u] = in ? __ldcg(p.part_lse + r) : -INFINITY;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) v[u][k] = __ldcg(part_chunk<HD>(p.part_o, r, cg * 8 + k));
+            for (int k = 0; k < kChunks; ++k)
+                v[u][k] = in ? __ldcg(part_chunk<HD>(p.part_o, r, cg * kChunks + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         float bmx = mx;
 #pragma unroll
-        for (int u = 0; u < kB; ++u) bmx = fmaxf(bmx, lse[u]);
+        for (int u = 0; u < kCombBatch; ++u) bmx = fmaxf(bmx, lse[u]);
         if (bmx == -INFINITY) continue;  // no visible key so far
         const float f = mx == -INFINITY ? 0.f : ex2(mx - bmx);
         den *= f;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) acc[i] *= f;
+        for (int k = 0; k < kChunks; ++k) {
+            acc[k].x *= f;
+            acc[k].y *= f;
+            acc[k].z *= f;
+            acc[k].w *= f;
+        }
         mx = bmx;
 #pragma unroll
-        for (int u = 0; u < kB; ++u) {
+        for (int u = 0; u < kCombBatch; ++u) {
             if (lse[u] == -INFINITY) continue;  // (its rows may hold anything)
             const float w = ex2(lse[u] - mx);
             den += w;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                acc[4 * k + 0] += w * v[u][k].x;
-                acc[4 * k + 1] += w * v[u][k].y;
-                acc[4 * k + 2] += w * v[u][k].z;
-                acc[4 * k + 3] += w * v[u][k].w;
+            for (int k = 0; k < kChunks; ++k) {
+                acc[k].x += w * v[u][k].x;
+                acc[k].y += w * v[u][k].y;
+                acc[k].z += w * v[u][k].z;
+                acc[k].w += w * v[u][k].w;
             }
         }
     }
-    if (qi >= sq.n_q) return;
     const float inv = den > 0.f ? 1.0f / den : 0.f;
     const int head = kvh * g + (row % g);
     uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.out) +
-                                           (static_cast<int64_t>(sq.q_row0 + qi) * p.hq + head) * HD + cg * 32);
+                                           (static_cast<int64_t>(sq.q_row0 + qi) * p.hq + head) * HD + cg * kCombCols);
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        dst[k] = make_uint4(pack_bf16(acc[8 * k + 0] * inv, acc[8 * k + 1] * inv),
-                            pack_bf16(acc[8 * k + 2] * inv, acc[8 * k + 3] * inv),
-                            pack_bf16(acc[8 * k + 4] * inv, acc[8 * k + 5] * inv),
-                            pack_bf16(acc[8 * k + 6] * inv, acc[8 * k + 7] * inv));
+    for (int k = 0; k < kChunks; k += 2)
+        dst[k / 2] = make_uint4(pack_bf16(acc[k].x * inv, acc[k].y * inv), pack_bf16(acc[k].z * inv, acc[k].w * inv),
+                                pack_bf16(acc[k + 1].x * inv, acc[k + 1].y * inv),
+                                pack_bf16(acc[k + 1].z * inv, acc[k + 1].w * inv));
 }
 
 // Split-KV partials of pe_replay_attn_static_scratch: a fixed 16 MiB array that
@@ -894,25 +903,44 @@ cudaError_t launch_replay_attn(int head_dim, bool split, const CUtensorMap &tm_q
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_splitkv_combine(int head_dim, const AttnParams &p, cudaStream_t st)
+template <int HD, int COLS, int BATCH>
+static cudaError_t launch_combine_t(const AttnParams &p, int ns, cudaStream_t st)
 {
-    if (p.total_comb <= 0) return cudaSuccess;
-    if (head_dim != 64 && head_dim != 128) return cudaErrorInvalidValue;
-    const int warps_per_block = 8;
-    const int64_t warps = static_cast<int64_t>(p.total_comb + 31) / 32 * (head_dim / 32);  // row blocks x column groups
-    const int blocks = static_cast<int>((warps + warps_per_block - 1) / warps_per_block);
+    constexpr int kCombSmSmem = 226 * 1024;  // shared memory of an SM, nearly
+    const int64_t warps = static_cast<int64_t>(p.total_comb + 31) / 32 * (HD / COLS);  // row blocks x column groups
+    // Blocks let in while attention CTAs still run all land on the SMs that are idle then, as many as fit,
+    // and the merge runs on those alone.  So, from 8 MB of partials on, a block an SM (up to 8 warps each), kept
+    // to that many an SM by its shared memory: 2 agents x 133 tokens on 1.3k, 3 splits, 17.8 -> 15.5 us a layer,
+    // attention included (d = 128).  Below, blocks of one warp, waiting early: 5.2 MB 10.7 us against 11.2.
+    const int64_t sms = p.next_stride > 0 ? p.next_stride : 152;
+    const bool small = static_cast<int64_t>(p.total_comb) * ns * HD * 4 < (8 << 20);
+    const int per_block = small ? 1 : static_cast<int>(std::min<int64_t>(8, (warps + sms - 1) / sms));
+    const int64_t blocks = (warps + per_block - 1) / per_block;
+    const int64_t per_sm = (blocks + sms - 1) / sms;
+    const int smem = small || per_sm > 4 ? 0 : static_cast<int>(kCombSmSmem / per_sm) - 1024;  // (1 KB a block is reserved)
+    static std::atomic<uint64_t> configured{0};
+    cudaError_t e = set_dyn_smem_once(splitkv_combine_kernel<HD, COLS, BATCH>, kCombSmSmem - 1024, configured);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(blocks));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
+    cfg.blockDim = dim3(static_cast<unsigned>(32 * per_block));
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (head_dim == 128) return cudaLaunchKernelEx(&cfg, splitkv_combine_kernel<128>, p);
-    if (head_dim == 64) return cudaLaunchKernelEx(&cfg, splitkv_combine_kernel<64>, p);
+    return cudaLaunchKernelEx(&cfg, splitkv_combine_kernel<HD, COLS, BATCH>, p);
+}
+
+cudaError_t launch_splitkv_combine(int head_dim, const AttnParams &p, cudaStream_t st)
+{
+    if (p.total_comb <= 0) return cudaSuccess;
+    int ns = 0;
+    for (int i = 0; i < p.n_seqs; ++i) ns = std::max(ns, static_cast<int>(p.seqs[i].n_splits));
+    if (head_dim == 128) return ns <= 4 ? launch_combine_t<128, 32, 4>(p, ns, st) : launch_combine_t<128, 16, 8>(p, ns, st);
+    if (head_dim == 64) return ns <= 4 ? launch_combine_t<64, 32, 4>(p, ns, st) : launch_combine_t<64, 16, 8>(p, ns, st);
     return cudaErrorInvalidValue;
 }
 
