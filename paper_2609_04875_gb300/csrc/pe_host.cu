@@ -1172,16 +1172,18 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         }
         // Estimated time with s key splits: the CTAs run in ceil(C s / N) waves of
         // (W/s + 2) tile times, and never faster than the longest CTA
-        // (max_tiles/s + 2); splits add their fp32 partials' HBM round trip and
-        // a combine launch.
+        // (max_tiles/s + 2); splits add a combine launch: 2.5 us, 1 us per batch of 8 splits, and the round
+        // trip of their fp32 partials, twice as fast while they are few (measured at d = 64, 64 CTAs of 12
+        // tiles: one pass 17.9 us, 2 splits 14.8; 32 CTAs of 11: 16.5, 4 splits 11.9).
         const double W = C > 0 ? static_cast<double>(tiles) / C : 0.0;
         const int64_t row_bytes = static_cast<int64_t>(d) * 4 + 4;
-        // (the combine kernel is a programmatic dependent of the attention grid: about 5 us more, measured
-        // on the 1-agent d = 64 launch: 5 splits + combine 14.0 us, one pass 13.0 us)
         auto cost = [&](int64_t sp) {
             const double waves = std::ceil(static_cast<double>(C * sp) / c->num_sms);
             double t = std::max(waves * (W / sp + 2.0), static_cast<double>(max_tiles) / sp + 2.0) * tile_s;
-            if (sp > 1) t += static_cast<double>(valid_rows * sp * row_bytes * 2) / 6.0e12 + 5e-6;
+            if (sp > 1) {
+                const double bytes = static_cast<double>(valid_rows * sp * row_bytes);
+                t += bytes * 2.0 / (bytes < 20e6 ? 12.0e12 : 6.0e12) + 2.5e-6 + 1e-6 * static_cast<double>(ceil_div(sp, 8));
+            }
             return t;
         };
         int64_t best = 1;
@@ -1195,7 +1197,8 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
                 const double t = cost(sp);
                 if (t < best_t) { best_t = t; best = sp; }
             }
-            if (splitkv == -1 && best > 1 && best_t > 0.95 * cost(1)) best = 1;  // keep the single pass unless clearly faster
+            // keep the single pass unless clearly faster, by more than a launch costs the host
+            if (splitkv == -1 && best > 1 && best_t > std::min(0.95 * cost(1), cost(1) - 1.0e-6)) best = 1;
         }
         if (splitkv != 0 && c->num_splits > 0) best = c->num_splits;
         plan_est = cost(best);
