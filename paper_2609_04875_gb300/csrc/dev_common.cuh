@@ -157,6 +157,16 @@ __device__ __forceinline__ void mma_commit_warp(uint32_t bar)
         : "memory");
 }
 
+// Registers of the prefill kernels' three warpgroups (384 threads, launched with 168 each): the two softmax
+// warpgroups, whose threads hold a row of 128 scores, take from the third (producers, MMA), so more of their
+// exponentials are in flight and less spills.  The three may sum to what the launch holds.  One-item kernel,
+// 16 agents of 2k to 8k keys 1745 -> 1665 us, 16k suffixes of 20k 16.0 -> 15.5 ms, the d = 64 batch 375 -> 370;
+// with 208 + 88 the d = 64 batch lost 1 %, with 224 + 56 the MMA warp spills and every launch lost.
+constexpr int kPrefillThreads = 384;
+constexpr int kSoftmaxRegs = 192;
+constexpr int kOtherRegs = 120;
+static_assert(2 * kSoftmaxRegs + kOtherRegs <= 3 * 168, "more registers than the launch holds");
+
 // Split partials (O / l, fp32, HD columns a row) are stored in blocks of 32 rows, 16-byte chunk major:
 // chunk k of row r at [r & ~31][k][r & 31].  Row blocks start at multiples of 32 rows, so a warp whose
 // lane i holds row 32 w + i writes or reads one chunk of its 32 rows as 512 contiguous bytes.

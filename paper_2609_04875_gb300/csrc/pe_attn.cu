@@ -9,7 +9,7 @@
 // One CTA computes one work item: (sequence, kv-head, pair of q-tiles[, key
 // split]).  A q-tile packs 128 rows = (128/g queries) x (g q-heads of one
 // kv-head), so each K/V tile brought into shared memory serves 2 x 128 rows.
-// Roles (352 threads, 352 or 384 at d = 64):
+// Roles (384 threads; those left over idle):
 //   warps 0-3, 4-7  softmax of q-tile 0 / q-tile 1: thread r owns row r
 //                   (TMEM lane r); masks, online softmax in fp32 (exp2),
 //                   writes P (bf16) back into TMEM (d = 128: over its S
@@ -61,9 +61,6 @@
 namespace pe {
 
 constexpr float kTileSumLimit = 1.8446744e19f;  // 2^64: larger tile sums move the reference
-// 8 softmax warps, the K producer, the MMA warps (one per q-tile at d = 64) and the V producer, if apart
-template <int HD, bool VAPART>
-constexpr int kThreads = 32 * (9 + (HD == 64 ? 2 : 1) + (VAPART ? 1 : 0));
 
 // Whether V has a producer warp of its own.  At d = 64 a tile has half the boxes, and from 16-token pages on
 // one warp issues them in time (d = 64 batch: 375 against 380 us with 32-token pages, 448 against 412 with
@@ -108,7 +105,7 @@ struct TileGeo {
 // a tile is its softmax alone (at d = 64 S(j+1) overlaps it anyway).  16 agents of 30 tokens on 4k: 55.8 -> 52.1
 // us a layer; 64 MHA agents of 60 tokens on 1.5k: 100.6 -> 93.8.
 template <int HD, bool SPLIT, bool VAPART, bool ONE>
-__global__ void __launch_bounds__(kThreads<HD, VAPART>, 1)
+__global__ void __launch_bounds__(kPrefillThreads, 1)
     replay_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
                        const __grid_constant__ AttnParams p)
@@ -288,218 +285,222 @@ __global__ void __launch_bounds__(kThreads<HD, VAPART>, 1)
     const uint32_t tmem = *tmem_slot;
 
     constexpr int kWarpV = 9 + C::kMmaWarps;
-    if (VAPART && warp == kWarpV && n_all > 0) {
-        // =================================================== V producer (TMA)
-        ptx::griddep_wait();
-        int page = page_of(0), i = 0;
-        for (; i < n_all; ++i) {
-            const int next = i + 1 < n_all ? page_of(i + 1) : -1;
-            if (!issue(&tm_v, v_smem0, b_v_full, b_v_empty, i, page)) break;
-            page = next;
-        }
-        __syncwarp();
-        if (*abort_flag && lane == 0) drain(b_v_full, i);
-    } else if (warp == 8 && n_all > 0) {
-        // =================================================== K producer (TMA), tiles 1.. (and V's)
-        int i = 1, iv = 0;
-        for (; i < n_all; ++i) {
-            const int page = page_next;
-            if (i + 1 < n_all) page_next = page_of(i + 1);  // prefetch the next tile's page ids
-            if (!issue(&tm_k, k_smem0, b_k_full, b_k_empty, i, page)) break;
-            if (!VAPART && !issue(&tm_v, v_smem0, b_v_full, b_v_empty, iv = i, page)) break;
-        }
-        // The next kernel's set-up may start once every CTA has issued its loads; let in at this grid's start
-        // it cost launches of a few microseconds 2 % (133-token episode of 32 layers 460 -> 450 us).
-        ptx::griddep_launch_dependents();
-        // With one CTA per SM, the CTA that starts on this SM next is about blockIdx.x + next_stride:
-        // bring its Q tiles (read once, from DRAM) into L2 now, so that its first S GEMMs wait less.
-        const int nxt = blockIdx.x + p.next_stride;
-        if (p.next_stride > 0 && nxt < p.total_items && lane == 0 && !*abort_flag) {
-            int nsi, nkvh, nsplit, npair;
-            decode_item(nxt, nsi, nkvh, nsplit, npair);
-            const AttnSeq &nq = p.seqs[nsi];
-            for (int t = 0; t < 2; ++t) {
-                const int qt = 2 * npair + t;
-                if (qt >= nq.n_qtiles) break;
-                for (int r = 0; r < C::kRegions; ++r)
-                    ptx::tma_prefetch_3d(&tm_q, r * 64, nkvh * g, nq.q_row0 + qt * (kBM / g));
+    if (warp >= 8) {
+        ptx::regs_dec<kOtherRegs>();
+        if (VAPART && warp == kWarpV && n_all > 0) {
+            // =================================================== V producer (TMA)
+            ptx::griddep_wait();
+            int page = page_of(0), i = 0;
+            for (; i < n_all; ++i) {
+                const int next = i + 1 < n_all ? page_of(i + 1) : -1;
+                if (!issue(&tm_v, v_smem0, b_v_full, b_v_empty, i, page)) break;
+                page = next;
             }
-        }
-        __syncwarp();
-        if (*abort_flag && lane == 0) {
-            drain(b_k_full, i);
-            if (!VAPART) drain(b_v_full, iv + 1);
-        }
-    } else if (C::kMmaWarps == 1 && warp == 9 && n_all > 0) {
-        // =================================================== MMA issuer (the whole warp; one elected lane issues)
-        constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
-        constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
-        // warp-uniform copies (every lane holds the same values already)
-        const int n0 = __shfl_sync(0xffffffffu, geo[0].ntiles, 0), n1 = __shfl_sync(0xffffffffu, geo[1].ntiles, 0);
-        const int n_mma = max(n0, n1);
-        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-        const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024);
-        const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
-        const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
-        auto issue_s = [&](int t, int s) {
-            const uint64_t qd = q_desc + t * (C::kTileBytes >> 4), kd = k_desc + s * (C::kTileBytes >> 4);
-#pragma unroll
-            for (int kk = 0; kk < HD / 16; ++kk) {
-                const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
-                mma_bf16_warp(tm + 128 * t, qd + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
+            __syncwarp();
+            if (*abort_flag && lane == 0) drain(b_v_full, i);
+        } else if (warp == 8 && n_all > 0) {
+            // =================================================== K producer (TMA), tiles 1.. (and V's)
+            int i = 1, iv = 0;
+            for (; i < n_all; ++i) {
+                const int page = page_next;
+                if (i + 1 < n_all) page_next = page_of(i + 1);  // prefetch the next tile's page ids
+                if (!issue(&tm_k, k_smem0, b_k_full, b_k_empty, i, page)) break;
+                if (!VAPART && !issue(&tm_v, v_smem0, b_v_full, b_v_empty, iv = i, page)) break;
             }
-            mma_commit_warp(b_s_full + 8 * t);
-        };
-        auto issue_pv = [&](int t, int s, bool acc) {
-            const uint64_t vd = v_desc + s * (C::kTileBytes >> 4);
-            const uint32_t tp = tm + 128 * t;  // P_t over S_t
-#pragma unroll
-            for (int kk = 0; kk < kBN / 16; ++kk)
-                mma_bf16_ts_warp(tm + 256 + HD * t, tp + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
-                                 (acc || kk > 0) ? 1u : 0u);
-            mma_commit_warp(b_o_done + 8 * t);
-        };
-        bool ok = wait_bar_warp(b_q_full, 0, wctx) && wait_bar_warp(b_k_full, 0, wctx);
-        if (ONE) {
-            // S(j) into buffer j % 2; S(j+2) goes behind P V(j), which reads P(j) over S(j)
-            auto s_tile = [&](int j) {
-                const uint64_t kd = k_desc + (j % C::kStages) * (C::kTileBytes >> 4);
+            // The next kernel's set-up may start once every CTA has issued its loads; let in at this grid's start
+            // it cost launches of a few microseconds 2 % (133-token episode of 32 layers 460 -> 450 us).
+            ptx::griddep_launch_dependents();
+            // With one CTA per SM, the CTA that starts on this SM next is about blockIdx.x + next_stride:
+            // bring its Q tiles (read once, from DRAM) into L2 now, so that its first S GEMMs wait less.
+            const int nxt = blockIdx.x + p.next_stride;
+            if (p.next_stride > 0 && nxt < p.total_items && lane == 0 && !*abort_flag) {
+                int nsi, nkvh, nsplit, npair;
+                decode_item(nxt, nsi, nkvh, nsplit, npair);
+                const AttnSeq &nq = p.seqs[nsi];
+                for (int t = 0; t < 2; ++t) {
+                    const int qt = 2 * npair + t;
+                    if (qt >= nq.n_qtiles) break;
+                    for (int r = 0; r < C::kRegions; ++r)
+                        ptx::tma_prefetch_3d(&tm_q, r * 64, nkvh * g, nq.q_row0 + qt * (kBM / g));
+                }
+            }
+            __syncwarp();
+            if (*abort_flag && lane == 0) {
+                drain(b_k_full, i);
+                if (!VAPART) drain(b_v_full, iv + 1);
+            }
+        } else if (C::kMmaWarps == 1 && warp == 9 && n_all > 0) {
+            // =================================================== MMA issuer (the whole warp; one elected lane issues)
+            constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
+            constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
+            // warp-uniform copies (every lane holds the same values already)
+            const int n0 = __shfl_sync(0xffffffffu, geo[0].ntiles, 0), n1 = __shfl_sync(0xffffffffu, geo[1].ntiles, 0);
+            const int n_mma = max(n0, n1);
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+            const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024);
+            const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
+            const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
+            auto issue_s = [&](int t, int s) {
+                const uint64_t qd = q_desc + t * (C::kTileBytes >> 4), kd = k_desc + s * (C::kTileBytes >> 4);
 #pragma unroll
                 for (int kk = 0; kk < HD / 16; ++kk) {
                     const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
-                    mma_bf16_warp(tm + 128 * (j & 1), q_desc + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
+                    mma_bf16_warp(tm + 128 * t, qd + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
                 }
-                mma_commit_warp(b_s_full + 8 * (j & 1));
-                mma_commit_warp(b_k_empty + 8 * (j % C::kStages));
+                mma_commit_warp(b_s_full + 8 * t);
+            };
+            auto issue_pv = [&](int t, int s, bool acc) {
+                const uint64_t vd = v_desc + s * (C::kTileBytes >> 4);
+                const uint32_t tp = tm + 128 * t;  // P_t over S_t
+#pragma unroll
+                for (int kk = 0; kk < kBN / 16; ++kk)
+                    mma_bf16_ts_warp(tm + 256 + HD * t, tp + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
+                                     (acc || kk > 0) ? 1u : 0u);
+                mma_commit_warp(b_o_done + 8 * t);
+            };
+            bool ok = wait_bar_warp(b_q_full, 0, wctx) && wait_bar_warp(b_k_full, 0, wctx);
+            if (ONE) {
+                // S(j) into buffer j % 2; S(j+2) goes behind P V(j), which reads P(j) over S(j)
+                auto s_tile = [&](int j) {
+                    const uint64_t kd = k_desc + (j % C::kStages) * (C::kTileBytes >> 4);
+#pragma unroll
+                    for (int kk = 0; kk < HD / 16; ++kk) {
+                        const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
+                        mma_bf16_warp(tm + 128 * (j & 1), q_desc + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
+                    }
+                    mma_commit_warp(b_s_full + 8 * (j & 1));
+                    mma_commit_warp(b_k_empty + 8 * (j % C::kStages));
+                };
+                auto full = [&](uint32_t bar, int j) {
+                    return wait_bar_warp(bar + 8 * (j % C::kStages), (j / C::kStages) & 1, wctx);
+                };
+                if (ok) {
+                    ptx::tc_fence_after();
+                    s_tile(0);
+                    if (n0 > 1 && (ok = full(b_k_full, 1))) {
+                        ptx::tc_fence_after();
+                        s_tile(1);
+                    }
+                }
+                for (int j = 0; ok && j < n0; ++j) {
+                    if (!full(b_v_full, j) || !wait_bar_warp(b_p_full + 8 * (j & 1), (j >> 1) & 1, wctx)) break;
+                    ptx::tc_fence_after();
+                    const uint64_t vd = v_desc + (j % C::kStages) * (C::kTileBytes >> 4);
+#pragma unroll
+                    for (int kk = 0; kk < kBN / 16; ++kk)
+                        mma_bf16_ts_warp(tm + 256, tm + 128 * (j & 1) + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
+                                         (j > 0 || kk > 0) ? 1u : 0u);
+                    // (a barrier per buffer: with the softmax up to two tiles ahead of P V the parity of a wait on one
+                    // barrier could be that of an earlier phase)
+                    mma_commit_warp(b_o_done + 8 * (j & 1));
+                    mma_commit_warp(b_v_empty + 8 * (j % C::kStages));
+                    if (j + 2 < n0) {
+                        if (!full(b_k_full, j + 2)) break;
+                        ptx::tc_fence_after();
+                        s_tile(j + 2);
+                    }
+                }
+                ok = false;  // (the loop below is the two-q-tile form)
+            }
+            if (ok) {
+                ptx::tc_fence_after();
+                if (n0 > 0) issue_s(0, 0);
+                if (n1 > 0) issue_s(1, 0);
+                if (n0 > 0 || n1 > 0) mma_commit_warp(b_k_empty);
+            }
+            for (int j = 0; ok && j < n_mma; ++j) {
+                const int s = j % C::kStages;
+                const int s1 = (j + 1) % C::kStages;
+                const bool more = j + 1 < n_mma;
+                if (!wait_bar_warp(b_v_full + 8 * s, (j / C::kStages) & 1, wctx)) { ok = false; break; }
+                if (j < n0) {
+                    if (!wait_bar_warp(b_p_full, j & 1, wctx)) { ok = false; break; }
+                    ptx::tc_fence_after();
+                    issue_pv(0, s, j > 0);
+                }
+                if (more && !wait_bar_warp(b_k_full + 8 * s1, ((j + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
+                ptx::tc_fence_after();
+                if (j + 1 < n0) issue_s(0, s1);
+                if (j < n1) {
+                    if (!wait_bar_warp(b_p_full + 8, j & 1, wctx)) { ok = false; break; }
+                    ptx::tc_fence_after();
+                    issue_pv(1, s, j > 0);
+                }
+                if (j + 1 < n1) issue_s(1, s1);
+                if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
+                mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its PV GEMMs
+            }
+        } else if (C::kMmaWarps == 2 && (warp == 9 || warp == 10) && n_all > 0) {
+            // =================================================== MMA issuers, d = 64 (converged warps)
+            // Warp 9 + t runs q-tile t's GEMMs, so that neither q-tile waits in the issue order for the
+            // other's softmax, which is what bounds d = 64 (6-agent batch, two layers: 392 -> 375 us).  At
+            // d = 128, where the tensor pipe is the bound, two interleaved streams of MMAs cost 18 % (agent
+            // batch 1.77 -> 2.10 ms).  Key tiles that the q-tile does not attend are passed on unread.
+            constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
+            constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
+            // warp-uniform copies (every lane holds the same values already)
+            const int t = __shfl_sync(0xffffffffu, warp - 9, 0);
+            const int n = __shfl_sync(0xffffffffu, t ? geo[1].ntiles : geo[0].ntiles, 0);
+            const int n_mma = __shfl_sync(0xffffffffu, n_all, 0);
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+            const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024) + t * (C::kTileBytes >> 4);
+            const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
+            const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
+            const uint32_t tp = tm + 256 + 2 * HD + 64 * t;  // P_t
+            auto issue_s = [&](int s) {
+                const uint64_t kd = k_desc + s * (C::kTileBytes >> 4);
+#pragma unroll
+                for (int kk = 0; kk < HD / 16; ++kk) {
+                    const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
+                    mma_bf16_warp(tm + 128 * t, q_desc + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
+                }
+                mma_commit_warp(b_s_full + 8 * t);
+                mma_commit_warp(b_k_empty + 8 * s);  // K consumed by this q-tile
             };
             auto full = [&](uint32_t bar, int j) {
                 return wait_bar_warp(bar + 8 * (j % C::kStages), (j / C::kStages) & 1, wctx);
             };
-            if (ok) {
+            auto pass = [&](uint32_t bar, int j) {  // this q-tile does not use tile j
+                if (lane == 0) ptx::mbar_arrive(bar + 8 * (j % C::kStages));
+                __syncwarp();
+            };
+            bool ok = (n == 0 || wait_bar_warp(b_q_full, 0, wctx)) && full(b_k_full, 0);
+            if (ok && n > 0) {
                 ptx::tc_fence_after();
-                s_tile(0);
-                if (n0 > 1 && (ok = full(b_k_full, 1))) {
-                    ptx::tc_fence_after();
-                    s_tile(1);
-                }
+                issue_s(0);
+            } else if (ok) {
+                pass(b_k_empty, 0);
             }
-            for (int j = 0; ok && j < n0; ++j) {
-                if (!full(b_v_full, j) || !wait_bar_warp(b_p_full + 8 * (j & 1), (j >> 1) & 1, wctx)) break;
+            for (int j = 0; ok && j < n_mma; ++j) {
+                if (j + 1 < n_mma) {
+                    // S_t(j+1) once the softmax holds S_t(j) in registers
+                    if (!full(b_k_full, j + 1)) break;
+                    if (j + 1 < n) {
+                        if (!wait_bar_warp(b_s_free + 8 * t, j & 1, wctx)) break;
+                        ptx::tc_fence_after();
+                        issue_s((j + 1) % C::kStages);
+                    } else {
+                        pass(b_k_empty, j + 1);
+                    }
+                }
+                if (!full(b_v_full, j)) break;
+                if (j >= n) {
+                    pass(b_v_empty, j);
+                    continue;
+                }
+                if (!wait_bar_warp(b_p_full + 8 * t, j & 1, wctx)) break;
                 ptx::tc_fence_after();
                 const uint64_t vd = v_desc + (j % C::kStages) * (C::kTileBytes >> 4);
 #pragma unroll
                 for (int kk = 0; kk < kBN / 16; ++kk)
-                    mma_bf16_ts_warp(tm + 256, tm + 128 * (j & 1) + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
+                    mma_bf16_ts_warp(tm + 256 + HD * t, tp + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
                                      (j > 0 || kk > 0) ? 1u : 0u);
-                // (a barrier per buffer: with the softmax up to two tiles ahead of P V the parity of a wait on one
-                // barrier could be that of an earlier phase)
-                mma_commit_warp(b_o_done + 8 * (j & 1));
-                mma_commit_warp(b_v_empty + 8 * (j % C::kStages));
-                if (j + 2 < n0) {
-                    if (!full(b_k_full, j + 2)) break;
-                    ptx::tc_fence_after();
-                    s_tile(j + 2);
-                }
+                mma_commit_warp(b_o_done + 8 * t);
+                mma_commit_warp(b_v_empty + 8 * (j % C::kStages));  // V consumed by this q-tile
             }
-            ok = false;  // (the loop below is the two-q-tile form)
         }
-        if (ok) {
-            ptx::tc_fence_after();
-            if (n0 > 0) issue_s(0, 0);
-            if (n1 > 0) issue_s(1, 0);
-            if (n0 > 0 || n1 > 0) mma_commit_warp(b_k_empty);
-        }
-        for (int j = 0; ok && j < n_mma; ++j) {
-            const int s = j % C::kStages;
-            const int s1 = (j + 1) % C::kStages;
-            const bool more = j + 1 < n_mma;
-            if (!wait_bar_warp(b_v_full + 8 * s, (j / C::kStages) & 1, wctx)) { ok = false; break; }
-            if (j < n0) {
-                if (!wait_bar_warp(b_p_full, j & 1, wctx)) { ok = false; break; }
-                ptx::tc_fence_after();
-                issue_pv(0, s, j > 0);
-            }
-            if (more && !wait_bar_warp(b_k_full + 8 * s1, ((j + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
-            ptx::tc_fence_after();
-            if (j + 1 < n0) issue_s(0, s1);
-            if (j < n1) {
-                if (!wait_bar_warp(b_p_full + 8, j & 1, wctx)) { ok = false; break; }
-                ptx::tc_fence_after();
-                issue_pv(1, s, j > 0);
-            }
-            if (j + 1 < n1) issue_s(1, s1);
-            if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
-            mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its PV GEMMs
-        }
-    } else if (C::kMmaWarps == 2 && (warp == 9 || warp == 10) && n_all > 0) {
-        // =================================================== MMA issuers, d = 64 (whole warps; one elected lane issues)
-        // Warp 9 + t runs q-tile t's GEMMs, so that neither q-tile waits in the issue order for the other's
-        // softmax, which is what bounds d = 64 (6-agent batch, two layers: 392 -> 375 us).  At d = 128, where the tensor pipe is the
-        // bound, two interleaved streams of MMAs cost 18 % (agent batch 1.77 -> 2.10 ms).  Key tiles that the
-        // q-tile does not attend are passed on unread.
-        constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
-        constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
-        // warp-uniform copies (every lane holds the same values already)
-        const int t = __shfl_sync(0xffffffffu, warp - 9, 0);
-        const int n = __shfl_sync(0xffffffffu, t ? geo[1].ntiles : geo[0].ntiles, 0);
-        const int n_mma = __shfl_sync(0xffffffffu, n_all, 0);
-        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-        const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024) + t * (C::kTileBytes >> 4);
-        const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
-        const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
-        const uint32_t tp = tm + 256 + 2 * HD + 64 * t;  // P_t
-        auto issue_s = [&](int s) {
-            const uint64_t kd = k_desc + s * (C::kTileBytes >> 4);
-#pragma unroll
-            for (int kk = 0; kk < HD / 16; ++kk) {
-                const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
-                mma_bf16_warp(tm + 128 * t, q_desc + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
-            }
-            mma_commit_warp(b_s_full + 8 * t);
-            mma_commit_warp(b_k_empty + 8 * s);  // K consumed by this q-tile
-        };
-        auto full = [&](uint32_t bar, int j) {
-            return wait_bar_warp(bar + 8 * (j % C::kStages), (j / C::kStages) & 1, wctx);
-        };
-        auto pass = [&](uint32_t bar, int j) {  // this q-tile does not use tile j
-            if (lane == 0) ptx::mbar_arrive(bar + 8 * (j % C::kStages));
-            __syncwarp();
-        };
-        bool ok = (n == 0 || wait_bar_warp(b_q_full, 0, wctx)) && full(b_k_full, 0);
-        if (ok && n > 0) {
-            ptx::tc_fence_after();
-            issue_s(0);
-        } else if (ok) {
-            pass(b_k_empty, 0);
-        }
-        for (int j = 0; ok && j < n_mma; ++j) {
-            if (j + 1 < n_mma) {
-                // S_t(j+1) once the softmax holds S_t(j) in registers
-                if (!full(b_k_full, j + 1)) break;
-                if (j + 1 < n) {
-                    if (!wait_bar_warp(b_s_free + 8 * t, j & 1, wctx)) break;
-                    ptx::tc_fence_after();
-                    issue_s((j + 1) % C::kStages);
-                } else {
-                    pass(b_k_empty, j + 1);
-                }
-            }
-            if (!full(b_v_full, j)) break;
-            if (j >= n) {
-                pass(b_v_empty, j);
-                continue;
-            }
-            if (!wait_bar_warp(b_p_full + 8 * t, j & 1, wctx)) break;
-            ptx::tc_fence_after();
-            const uint64_t vd = v_desc + (j % C::kStages) * (C::kTileBytes >> 4);
-#pragma unroll
-            for (int kk = 0; kk < kBN / 16; ++kk)
-                mma_bf16_ts_warp(tm + 256 + HD * t, tp + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
-                                 (j > 0 || kk > 0) ? 1u : 0u);
-            mma_commit_warp(b_o_done + 8 * t);
-            mma_commit_warp(b_v_empty + 8 * (j % C::kStages));  // V consumed by this q-tile
-        }
-    } else if (warp < 8) {
+    } else {
+        ptx::regs_inc<kSoftmaxRegs>();
         // =================================================== softmax / epilogue
         ptx::griddep_wait();                     // before this role's first global write
         const int t = warp >> 2;                 // q-tile of this warpgroup
@@ -871,7 +872,7 @@ static cudaError_t launch_attn_t(const CUtensorMap &q, const CUtensorMap &k, con
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(p.total_items));
-    cfg.blockDim = dim3(kThreads<HD, VAPART>);
+    cfg.blockDim = dim3(kPrefillThreads);
     cfg.dynamicSmemBytes = C::kDynSmem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -917,7 +918,8 @@ static cudaError_t launch_combine_t(const AttnParams &p, int ns, cudaStream_t st
     const int per_block = small ? 1 : static_cast<int>(std::min<int64_t>(8, (warps + sms - 1) / sms));
     const int64_t blocks = (warps + per_block - 1) / per_block;
     const int64_t per_sm = (blocks + sms - 1) / sms;
-    const int smem = small || per_sm > 4 ? 0 : static_cast<int>(kCombSmSmem / per_sm) - 1024;  // (1 KB a block is reserved)
+    // (1 KB a block is reserved)
+    const int smem = small || per_sm > 4 ? 0 : static_cast<int>(kCombSmSmem / per_sm) - 1024;
     static std::atomic<uint64_t> configured{0};
     cudaError_t e = set_dyn_smem_once(splitkv_combine_kernel<HD, COLS, BATCH>, kCombSmSmem - 1024, configured);
     if (e != cudaSuccess) return e;
