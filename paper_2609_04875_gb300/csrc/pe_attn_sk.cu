@@ -19,7 +19,7 @@
 // tile and epilogue run (no CTA launch, TMEM allocation or barrier set-up
 // between units).
 //
-// Roles (352 threads) as in replay_attn_kernel: softmax warpgroups 0 and 1
+// Roles (384 threads, warp 11 idle) as in replay_attn_kernel: softmax warpgroups 0 and 1
 // (one per q-tile, thread r owns row r), producer warps 8 (Q, K) and 10 (V)
 // (page table -> TMA boxes), MMA warp 9 (converged; one elected lane issues
 // tcgen05.mma).  Every role walks the same sequence of pieces, computed from the kernel parameters; barrier phases
@@ -44,8 +44,6 @@ namespace pe {
 namespace {
 
 constexpr float kTileSumLimit = 1.8446744e19f;  // 2^64: larger tile sums move the reference
-constexpr int kThreads = 352;
-
 template <int HD, bool ONE>
 struct SkCfg {
     static constexpr int kRegions = HD / 64;            // 128-byte swizzle atoms along d
@@ -293,7 +291,7 @@ __device__ __noinline__ void merge_own_row(const SkParams &P, int slot, int t, i
 // own, because both forms in one cost the two-q-tile launches 1 % (d = 64: 7 %).  Short suffix (8 x 16 tokens
 // on 32k, HBM-bound) 181 -> 175 us, at d = 64 133 -> 104 us.
 template <int HD, bool ONE>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kPrefillThreads, 1)
     replay_attn_sk_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                           const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ SkParams P)
 {
@@ -363,194 +361,198 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 8 || warp == 10) {
-        // =================================================== producers (TMA): warp 8 Q and K, warp 10 V.  A warp
-        // issues a box in about 30 ns whatever its size, so one warp for both held back small pages (8-token
-        // pages: 64 boxes a tile).
-        ptx::griddep_wait();  // page table, pool and Q were written by earlier kernels
-        const bool is_v = warp == 10;
-        const CUtensorMap *map = is_v ? &tm_v : &tm_k;
-        const uint32_t smem0 = is_v ? v_smem0 : k_smem0;
-        const uint32_t b_full = is_v ? b_v_full : b_k_full, b_empty = is_v ? b_v_empty : b_k_empty;
-        const int ppt = kBN / p.ps;                 // pages per key tile
-        const int n_ops = ppt * C::kRegions;        // TMA boxes per K (or V) tile, <= 32
-        const int op_page = lane / C::kRegions;     // this lane's box: page index and half
-        const int op_reg = lane % C::kRegions;
-        const bool op_on = lane < n_ops;
-        const uint32_t op_off = op_reg * C::kRegionBytes + op_page * p.ps * 128;
-        int gk = 0;        // key tiles issued so far (ring position)
-        int q_issued = 0;  // pieces so far (Q loads issued)
-        bool ok = true;
-        Piece pc;
-        UnitGeo U;
-        for (int k = 0; ok && piece_of(P, cw, k, pc, U); ++k) {
-            const AttnSeq &sq = p.seqs[U.si];
-            const bool two = 2 * U.pair + 1 < sq.n_qtiles;
-            auto page_of = [&](int kt) -> int {  // this lane's page id of key tile kt (or -1)
-                const int lp = kt * ppt + lane;
-                return (lane < ppt && lp < sq.n_pages) ? p.page_table[sq.table_row + lp] : -1;
-            };
-            int page_next = page_of(pc.lo);  // read while the previous piece's last S GEMMs run
-            if (!is_v) {
-                // Q of this piece once the previous piece's S GEMMs have read theirs
-                if (q_issued > 0 && !wait_bar_warp(b_q_empty, (q_issued - 1) & 1, wctx)) { ok = false; break; }
-                if (lane == 0) {
-                    const int nq = two ? 2 : 1;
-                    ptx::mbar_arrive_expect_tx(b_q_full, nq * C::kTileBytes);
-                    for (int t = 0; t < nq; ++t)
-                        for (int r = 0; r < C::kRegions; ++r)
-                            ptx::tma_load_3d(q_smem + t * C::kTileBytes + r * C::kRegionBytes, &tm_q, r * 64,
-                                             U.kvh * g, sq.q_row0 + (2 * U.pair + t) * (kBM / g), b_q_full);
+    if (warp >= 8) {
+        ptx::regs_dec<kOtherRegs>();
+        if (warp == 8 || warp == 10) {
+            // =================================================== producers (TMA): warp 8 Q and K, warp 10 V.  A warp
+            // issues a box in about 30 ns whatever its size, so one warp for both held back small pages (8-token
+            // pages: 64 boxes a tile).
+            ptx::griddep_wait();  // page table, pool and Q were written by earlier kernels
+            const bool is_v = warp == 10;
+            const CUtensorMap *map = is_v ? &tm_v : &tm_k;
+            const uint32_t smem0 = is_v ? v_smem0 : k_smem0;
+            const uint32_t b_full = is_v ? b_v_full : b_k_full, b_empty = is_v ? b_v_empty : b_k_empty;
+            const int ppt = kBN / p.ps;                 // pages per key tile
+            const int n_ops = ppt * C::kRegions;        // TMA boxes per K (or V) tile, <= 32
+            const int op_page = lane / C::kRegions;     // this lane's box: page index and half
+            const int op_reg = lane % C::kRegions;
+            const bool op_on = lane < n_ops;
+            const uint32_t op_off = op_reg * C::kRegionBytes + op_page * p.ps * 128;
+            int gk = 0;        // key tiles issued so far (ring position)
+            int q_issued = 0;  // pieces so far (Q loads issued)
+            bool ok = true;
+            Piece pc;
+            UnitGeo U;
+            for (int k = 0; ok && piece_of(P, cw, k, pc, U); ++k) {
+                const AttnSeq &sq = p.seqs[U.si];
+                const bool two = 2 * U.pair + 1 < sq.n_qtiles;
+                auto page_of = [&](int kt) -> int {  // this lane's page id of key tile kt (or -1)
+                    const int lp = kt * ppt + lane;
+                    return (lane < ppt && lp < sq.n_pages) ? p.page_table[sq.table_row + lp] : -1;
+                };
+                int page_next = page_of(pc.lo);  // read while the previous piece's last S GEMMs run
+                if (!is_v) {
+                    // Q of this piece once the previous piece's S GEMMs have read theirs
+                    if (q_issued > 0 && !wait_bar_warp(b_q_empty, (q_issued - 1) & 1, wctx)) { ok = false; break; }
+                    if (lane == 0) {
+                        const int nq = two ? 2 : 1;
+                        ptx::mbar_arrive_expect_tx(b_q_full, nq * C::kTileBytes);
+                        for (int t = 0; t < nq; ++t)
+                            for (int r = 0; r < C::kRegions; ++r)
+                                ptx::tma_load_3d(q_smem + t * C::kTileBytes + r * C::kRegionBytes, &tm_q, r * 64,
+                                                 U.kvh * g, sq.q_row0 + (2 * U.pair + t) * (kBM / g), b_q_full);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
+                ++q_issued;
+                for (int kt = pc.lo; kt < pc.hi; ++kt, ++gk) {
+                    const int page = page_next;
+                    if (kt + 1 < pc.hi) page_next = page_of(kt + 1);
+                    const int s = gk % C::kStages;
+                    const int pg = __shfl_sync(0xffffffffu, page, op_page & 31);
+                    // rows of pages past the sequence read as zeros (out-of-bounds box)
+                    const int y = pg >= 0 ? ((p.layer * p.num_pages + pg) * p.hkv + U.kvh) * p.ps : p.oob_row;
+                    if (gk >= C::kStages && !wait_bar_warp(b_empty + 8 * s, ((gk / C::kStages) - 1) & 1, wctx)) {
+                        ok = false;
+                        break;
+                    }
+                    if (lane == 0) ptx::mbar_arrive_expect_tx(b_full + 8 * s, C::kTileBytes);
+                    __syncwarp();
+                    if (op_on) ptx::tma_load_2d(smem0 + s * C::kTileBytes + op_off, map, op_reg * 64, y, b_full + 8 * s);
+                }
             }
-            ++q_issued;
-            for (int kt = pc.lo; kt < pc.hi; ++kt, ++gk) {
-                const int page = page_next;
-                if (kt + 1 < pc.hi) page_next = page_of(kt + 1);
-                const int s = gk % C::kStages;
-                const int pg = __shfl_sync(0xffffffffu, page, op_page & 31);
-                // rows of pages past the sequence read as zeros (out-of-bounds box)
-                const int y = pg >= 0 ? ((p.layer * p.num_pages + pg) * p.hkv + U.kvh) * p.ps : p.oob_row;
-                if (gk >= C::kStages && !wait_bar_warp(b_empty + 8 * s, ((gk / C::kStages) - 1) & 1, wctx)) {
+            __syncwarp();
+            if (!ok && lane == 0) {
+                // give copies in flight a bounded chance to land before the CTA exits
+                const uint64_t t0 = ptx::globaltimer();
+                if (!is_v && q_issued > 0)
+                    while (!ptx::mbar_try_wait(b_q_full, (q_issued - 1) & 1) && ptx::globaltimer() - t0 < 2000000ull) {}
+                for (int i = max(0, gk - C::kStages); i < gk; ++i)
+                    while (!ptx::mbar_try_wait(b_full + 8 * (i % C::kStages), (i / C::kStages) & 1) &&
+                           ptx::globaltimer() - t0 < 4000000ull) {}
+            }
+        } else if (warp == 9) {
+            // =================================================== MMA issuer (the whole warp; one elected lane issues)
+            constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
+            constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+            const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024);
+            const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
+            const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
+            // q-tile t, S (and P) buffer b
+            auto issue_s = [&](int t, int b, int s) {
+                const uint64_t qd = q_desc + t * (C::kTileBytes >> 4), kd = k_desc + s * (C::kTileBytes >> 4);
+#pragma unroll
+                for (int kk = 0; kk < HD / 16; ++kk) {
+                    const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
+                    mma_bf16_warp(tm + 128 * b, qd + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
+                }
+                mma_commit_warp(b_s_full + 8 * b);
+            };
+            auto issue_pv = [&](int t, int b, int s, bool acc) {
+                const uint64_t vd = v_desc + s * (C::kTileBytes >> 4);
+#pragma unroll
+                for (int kk = 0; kk < kBN / 16; ++kk)
+                    mma_bf16_ts_warp(tm + 256 + HD * t, tm + 128 * b + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
+                                     (acc || kk > 0) ? 1u : 0u);
+                mma_commit_warp(b_o_done + 8 * (ONE ? b : t));
+            };
+            int gk = 0;              // key tiles consumed so far (ring position)
+            int cnt0 = 0, cnt1 = 0;  // tiles of q-tile 0 / 1 in earlier pieces (S and P phases)
+            uint32_t ph = 0;         // (ONE) bit b: parity of the uses of S buffer b in earlier pieces
+            int seg0 = 0, seg1 = 0;  // earlier pieces in which q-tile 0 / 1 had tiles (o_free phase)
+            bool ok = true;
+            Piece pc;
+            UnitGeo U;
+            for (int k = 0; ok && piece_of(P, cw, k, pc, U); ++k) {
+                const AttnSeq &sq = p.seqs[U.si];
+                // warp-uniform copies (every lane holds the same values already)
+                const int n0 = __shfl_sync(0xffffffffu, q_geo(p, sq, U.pair, 0, pc.lo, pc.hi).ntiles, 0);
+                const int n1 = __shfl_sync(0xffffffffu, q_geo(p, sq, U.pair, 1, pc.lo, pc.hi).ntiles, 0);
+                const int n_all = __shfl_sync(0xffffffffu, pc.hi - pc.lo, 0);
+                if (!wait_bar_warp(b_q_full, k & 1, wctx) || !wait_bar_warp(b_k_full + 8 * (gk % C::kStages),
+                                                                 (gk / C::kStages) & 1, wctx)) {
                     ok = false;
                     break;
                 }
-                if (lane == 0) ptx::mbar_arrive_expect_tx(b_full + 8 * s, C::kTileBytes);
-                __syncwarp();
-                if (op_on) ptx::tma_load_2d(smem0 + s * C::kTileBytes + op_off, map, op_reg * 64, y, b_full + 8 * s);
-            }
-        }
-        __syncwarp();
-        if (!ok && lane == 0) {
-            // give copies in flight a bounded chance to land before the CTA exits
-            const uint64_t t0 = ptx::globaltimer();
-            if (!is_v && q_issued > 0)
-                while (!ptx::mbar_try_wait(b_q_full, (q_issued - 1) & 1) && ptx::globaltimer() - t0 < 2000000ull) {}
-            for (int i = max(0, gk - C::kStages); i < gk; ++i)
-                while (!ptx::mbar_try_wait(b_full + 8 * (i % C::kStages), (i / C::kStages) & 1) &&
-                       ptx::globaltimer() - t0 < 4000000ull) {}
-        }
-    } else if (warp == 9) {
-        // =================================================== MMA issuer (the whole warp; one elected lane issues)
-        constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
-        constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
-        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-        const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024);
-        const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
-        const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
-        // q-tile t, S (and P) buffer b
-        auto issue_s = [&](int t, int b, int s) {
-            const uint64_t qd = q_desc + t * (C::kTileBytes >> 4), kd = k_desc + s * (C::kTileBytes >> 4);
-#pragma unroll
-            for (int kk = 0; kk < HD / 16; ++kk) {
-                const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
-                mma_bf16_warp(tm + 128 * b, qd + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
-            }
-            mma_commit_warp(b_s_full + 8 * b);
-        };
-        auto issue_pv = [&](int t, int b, int s, bool acc) {
-            const uint64_t vd = v_desc + s * (C::kTileBytes >> 4);
-#pragma unroll
-            for (int kk = 0; kk < kBN / 16; ++kk)
-                mma_bf16_ts_warp(tm + 256 + HD * t, tm + 128 * b + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
-                                 (acc || kk > 0) ? 1u : 0u);
-            mma_commit_warp(b_o_done + 8 * (ONE ? b : t));
-        };
-        int gk = 0;              // key tiles consumed so far (ring position)
-        int cnt0 = 0, cnt1 = 0;  // tiles of q-tile 0 / 1 in earlier pieces (S and P phases)
-        uint32_t ph = 0;         // (ONE) bit b: parity of the uses of S buffer b in earlier pieces
-        int seg0 = 0, seg1 = 0;  // earlier pieces in which q-tile 0 / 1 had tiles (o_free phase)
-        bool ok = true;
-        Piece pc;
-        UnitGeo U;
-        for (int k = 0; ok && piece_of(P, cw, k, pc, U); ++k) {
-            const AttnSeq &sq = p.seqs[U.si];
-            // warp-uniform copies (every lane holds the same values already)
-            const int n0 = __shfl_sync(0xffffffffu, q_geo(p, sq, U.pair, 0, pc.lo, pc.hi).ntiles, 0);
-            const int n1 = __shfl_sync(0xffffffffu, q_geo(p, sq, U.pair, 1, pc.lo, pc.hi).ntiles, 0);
-            const int n_all = __shfl_sync(0xffffffffu, pc.hi - pc.lo, 0);
-            if (!wait_bar_warp(b_q_full, k & 1, wctx) || !wait_bar_warp(b_k_full + 8 * (gk % C::kStages),
-                                                             (gk / C::kStages) & 1, wctx)) {
-                ok = false;
-                break;
-            }
-            ptx::tc_fence_after();
-            if (ONE) {
-                // S(j+1) runs during the softmax of tile j, in the other buffer; S(j+2) goes behind P V(j), which
-                // reads P(j) over S(j)
-                auto k_full = [&](int j) {
-                    return wait_bar_warp(b_k_full + 8 * ((gk + j) % C::kStages), ((gk + j) / C::kStages) & 1, wctx);
-                };
-                auto s_tile = [&](int j) {
-                    issue_s(0, j & 1, (gk + j) % C::kStages);
-                    mma_commit_warp(b_k_empty + 8 * ((gk + j) % C::kStages));
-                    if (j + 1 == n_all) mma_commit_warp(b_q_empty);
-                };
-                s_tile(0);
-                if (n_all > 1) {
-                    if (!k_full(1)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    s_tile(1);
-                }
-                for (int j = 0; j < n_all; ++j) {
-                    const int s = (gk + j) % C::kStages;
-                    if (!wait_bar_warp(b_v_full + 8 * s, ((gk + j) / C::kStages) & 1, wctx)) { ok = false; break; }
-                    if (j == 0 && seg0 > 0 && !wait_bar_warp(b_o_free, (seg0 - 1) & 1, wctx)) { ok = false; break; }
-                    if (!wait_bar_warp(b_p_full + 8 * (j & 1), ((ph >> (j & 1)) + (j >> 1)) & 1, wctx)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    issue_pv(0, j & 1, s, j > 0);
-                    mma_commit_warp(b_v_empty + 8 * s);
-                    if (j + 2 < n_all) {
-                        if (!k_full(j + 2)) { ok = false; break; }
+                ptx::tc_fence_after();
+                if (ONE) {
+                    // S(j+1) runs during the softmax of tile j, in the other buffer; S(j+2) goes behind P V(j), which
+                    // reads P(j) over S(j)
+                    auto k_full = [&](int j) {
+                        return wait_bar_warp(b_k_full + 8 * ((gk + j) % C::kStages), ((gk + j) / C::kStages) & 1, wctx);
+                    };
+                    auto s_tile = [&](int j) {
+                        issue_s(0, j & 1, (gk + j) % C::kStages);
+                        mma_commit_warp(b_k_empty + 8 * ((gk + j) % C::kStages));
+                        if (j + 1 == n_all) mma_commit_warp(b_q_empty);
+                    };
+                    s_tile(0);
+                    if (n_all > 1) {
+                        if (!k_full(1)) { ok = false; break; }
                         ptx::tc_fence_after();
-                        s_tile(j + 2);
+                        s_tile(1);
                     }
+                    for (int j = 0; j < n_all; ++j) {
+                        const int s = (gk + j) % C::kStages;
+                        if (!wait_bar_warp(b_v_full + 8 * s, ((gk + j) / C::kStages) & 1, wctx)) { ok = false; break; }
+                        if (j == 0 && seg0 > 0 && !wait_bar_warp(b_o_free, (seg0 - 1) & 1, wctx)) { ok = false; break; }
+                        if (!wait_bar_warp(b_p_full + 8 * (j & 1), ((ph >> (j & 1)) + (j >> 1)) & 1, wctx)) { ok = false; break; }
+                        ptx::tc_fence_after();
+                        issue_pv(0, j & 1, s, j > 0);
+                        mma_commit_warp(b_v_empty + 8 * s);
+                        if (j + 2 < n_all) {
+                            if (!k_full(j + 2)) { ok = false; break; }
+                            ptx::tc_fence_after();
+                            s_tile(j + 2);
+                        }
+                    }
+                    gk += n_all;
+                    ph ^= (((n_all + 1) / 2) & 1) | ((n_all / 2 & 1) << 1);
+                    seg0 += 1;
+                    continue;
+                }
+                const int n_s = max(n0, n1);  // key tiles with S GEMMs; Q is free after the last one
+                if (n0 > 0) issue_s(0, 0, gk % C::kStages);
+                if (n1 > 0) issue_s(1, 1, gk % C::kStages);
+                mma_commit_warp(b_k_empty + 8 * (gk % C::kStages));
+                if (n_s <= 1) mma_commit_warp(b_q_empty);
+                for (int j = 0; j < n_all; ++j) {
+                    const int gj = gk + j;
+                    const int s = gj % C::kStages;
+                    const int s1 = (gj + 1) % C::kStages;
+                    const bool more = j + 1 < n_all;
+                    if (!wait_bar_warp(b_v_full + 8 * s, (gj / C::kStages) & 1, wctx)) { ok = false; break; }
+                    if (j < n0) {
+                        // the first P V GEMM of a piece overwrites O_0: the previous piece's epilogue read it
+                        if (j == 0 && seg0 > 0 && !wait_bar_warp(b_o_free, (seg0 - 1) & 1, wctx)) { ok = false; break; }
+                        if (!wait_bar_warp(b_p_full, (cnt0 + j) & 1, wctx)) { ok = false; break; }
+                        ptx::tc_fence_after();
+                        issue_pv(0, 0, s, j > 0);
+                    }
+                    if (more && !wait_bar_warp(b_k_full + 8 * s1, ((gj + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
+                    ptx::tc_fence_after();
+                    if (j + 1 < n0) issue_s(0, 0, s1);
+                    if (j < n1) {
+                        if (j == 0 && seg1 > 0 && !wait_bar_warp(b_o_free + 8, (seg1 - 1) & 1, wctx)) { ok = false; break; }
+                        if (!wait_bar_warp(b_p_full + 8, (cnt1 + j) & 1, wctx)) { ok = false; break; }
+                        ptx::tc_fence_after();
+                        issue_pv(1, 1, s, j > 0);
+                    }
+                    if (j + 1 < n1) issue_s(1, 1, s1);
+                    if (j + 2 == n_s) mma_commit_warp(b_q_empty);    // the piece's last S GEMMs read Q
+                    if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
+                    mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its P V GEMMs
                 }
                 gk += n_all;
-                ph ^= (((n_all + 1) / 2) & 1) | ((n_all / 2 & 1) << 1);
-                seg0 += 1;
-                continue;
+                cnt0 += n0;
+                cnt1 += n1;
+                seg0 += n0 > 0 ? 1 : 0;
+                seg1 += n1 > 0 ? 1 : 0;
             }
-            const int n_s = max(n0, n1);  // key tiles with S GEMMs; Q is free after the last one
-            if (n0 > 0) issue_s(0, 0, gk % C::kStages);
-            if (n1 > 0) issue_s(1, 1, gk % C::kStages);
-            mma_commit_warp(b_k_empty + 8 * (gk % C::kStages));
-            if (n_s <= 1) mma_commit_warp(b_q_empty);
-            for (int j = 0; j < n_all; ++j) {
-                const int gj = gk + j;
-                const int s = gj % C::kStages;
-                const int s1 = (gj + 1) % C::kStages;
-                const bool more = j + 1 < n_all;
-                if (!wait_bar_warp(b_v_full + 8 * s, (gj / C::kStages) & 1, wctx)) { ok = false; break; }
-                if (j < n0) {
-                    // the first P V GEMM of a piece overwrites O_0: the previous piece's epilogue read it
-                    if (j == 0 && seg0 > 0 && !wait_bar_warp(b_o_free, (seg0 - 1) & 1, wctx)) { ok = false; break; }
-                    if (!wait_bar_warp(b_p_full, (cnt0 + j) & 1, wctx)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    issue_pv(0, 0, s, j > 0);
-                }
-                if (more && !wait_bar_warp(b_k_full + 8 * s1, ((gj + 1) / C::kStages) & 1, wctx)) { ok = false; break; }
-                ptx::tc_fence_after();
-                if (j + 1 < n0) issue_s(0, 0, s1);
-                if (j < n1) {
-                    if (j == 0 && seg1 > 0 && !wait_bar_warp(b_o_free + 8, (seg1 - 1) & 1, wctx)) { ok = false; break; }
-                    if (!wait_bar_warp(b_p_full + 8, (cnt1 + j) & 1, wctx)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    issue_pv(1, 1, s, j > 0);
-                }
-                if (j + 1 < n1) issue_s(1, 1, s1);
-                if (j + 2 == n_s) mma_commit_warp(b_q_empty);    // the piece's last S GEMMs read Q
-                if (more) mma_commit_warp(b_k_empty + 8 * s1);  // K of tile j+1 consumed by its S GEMMs
-                mma_commit_warp(b_v_empty + 8 * s);              // V of tile j consumed by its P V GEMMs
-            }
-            gk += n_all;
-            cnt0 += n0;
-            cnt1 += n1;
-            seg0 += n0 > 0 ? 1 : 0;
-            seg1 += n1 > 0 ? 1 : 0;
         }
     } else {
+        ptx::regs_inc<kSoftmaxRegs>();
         // =================================================== softmax / epilogue (warps 0-7)
         ptx::griddep_wait();                     // before this role's first global write
         const int t = warp >> 2;                 // q-tile of this warpgroup
@@ -795,7 +797,7 @@ cudaError_t launch_sk_t(const CUtensorMap &q, const CUtensorMap &k, const CUtens
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(p.n_ctas));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kPrefillThreads);
     cfg.dynamicSmemBytes = C::kDynSmem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
