@@ -1147,9 +1147,8 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
 
     // split-KV decision over the whole launch group; plan_est: the cost model's time of the plan
     double plan_est = 0.0;
-    // the group's units (pairs of q-tiles x kv-heads), their key tiles, and whether every unit is one q-tile
-    int64_t grp_units = 0, grp_tiles = 0;
-    bool grp_lone = false;
+    // the group's units (pairs of q-tiles x kv-heads), their key tiles, and how many units are one q-tile
+    int64_t grp_units = 0, grp_tiles = 0, grp_lone = 0;
     // time of one key tile per CTA in the cost models: about 1.5 us, compute- or HBM-bound alike; 1 us at
     // d = 64, whose next S GEMM overlaps the softmax
     const double tile_s = d == 64 ? 1.0e-6 : 1.5e-6;
@@ -1204,7 +1203,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         plan_est = cost(best);
         grp_units = C;
         grp_tiles = tiles;
-        grp_lone = rows == C * kBM;
+        grp_lone = 2 * C - rows / kBM;
         int split_tiles = static_cast<int>(max_tiles);
         split = best > 1 || splitkv == 1;
         if (split) split_tiles = static_cast<int>(std::max<int64_t>(1, ceil_div(max_tiles, std::max<int64_t>(best, 1))));
@@ -1328,24 +1327,31 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         const bool tail = hi - lo == 1 && c->splitkv == -1 && c->num_splits == 0 && plan_tail(order[lo], tp);
         // The persistent stream-K kernel where it should beat the one-item plan, among launches whose units
         // fill between a quarter of the SMs and two waves.  One CTA per SM takes an equal stretch of key
-        // tiles, at a slightly longer tile and a longer start and end (the parts of cut units are merged by
-        // single warps, about 2 us a part), so it wins where the one-item plan leaves SMs idle for long:
-        // its estimate is linear in the key tiles per SM.  Measured, d = 128, one-item / persistent us a
-        // layer: 64 units of one q-tile 21 / 27 at 7 tiles per SM, 51 / 58 at 27, 174 / 171 at 108; 64
-        // pairs 36 / 42 at 13, 182 / 174 at 108; 168 pairs 152 / 124 at 70 (key splits).  d = 64, whose pair
-        // tiles the one-item kernel runs 20 % faster: 64 units of one q-tile 23 / 27 at 13, 114 / 100 at
-        // 108; 64 pairs 27 / 33 at 13, 137 / 149 at 108; 256 pairs 492 / 536 at 419 (tail launch).  A plan
-        // in one pass is left only for a clear gain, a last wave nearly empty: 168 pairs of 32 tiles 93 / 72
-        // (d = 64: 68 / 59).
+        // tiles; its longer start and end (the parts of cut units are merged by single warps, about 2 us a
+        // part) pay where the one-item plan leaves SMs idle for long.  Its estimate is linear in the key
+        // tiles per SM.  Measured, one-item / persistent us a layer, d = 128: 64 units of one q-tile 20 / 27 at
+        // 7 tiles per SM, 50 / 57 at 27, 172 / 169 at 108; 64 pairs 34 / 41 at 13, 178 / 166 at 107; 168 pairs
+        // 143 / 120 at 70; 256 pairs 319 / 297 at 204, but 337 / 362 where a quarter of them are one q-tile,
+        // which only the one-item kernel is done with sooner.  d = 64: 64 units of one q-tile 22 / 26 at 13,
+        // 115 / 95 at 108; 64 pairs 26 / 31 at 13, 136 / 139 at 108; 168 pairs 109 / 96 at 70.  A plan in one pass
+        // is left for a clear gain only: a last wave nearly empty, 168 pairs of 32 tiles 88 / 69 (d = 64: 67 / 56).
         const bool sk_fits = 4 * grp_units >= c->num_sms && grp_units < 2 * static_cast<int64_t>(c->num_sms);
-        const double sk_tile = d == 64 ? (grp_lone ? 0.77e-6 : 1.23e-6) : (grp_lone ? 1.38e-6 : 1.45e-6);
-        const double sk_fixed =
-            d == 64 ? 17e-6 : 1e-6 + 5e-6 * std::max(4.0, 1.0 + static_cast<double>(c->num_sms) / std::max<int64_t>(grp_units, 1));
-        const double sk_est = sk_fixed + sk_tile * static_cast<double>(grp_tiles) / c->num_sms;
-        // (the cost model's estimates of these launches come out 3 to 8 % high at d = 128)
-        const double one_est = (tail ? tp.est : plan_est) * (d == 64 ? 1.0 : 0.95);
         const bool one_pass = !split && !tail;
-        const bool sk_wins = sk_fits && !(one_pass && c->splitkv == 0) && sk_est <= (one_pass ? 0.9 : 1.0) * one_est;
+        const bool all_lone = grp_lone == grp_units;
+        const double lone = all_lone || grp_units == 0 ? 0.0 : static_cast<double>(grp_lone) / grp_units;
+        double sk_tile, sk_fixed, one_scale;  // us a key tile per SM, us; measured over estimated time of the one-item plan
+        if (d == 64) {
+            sk_tile = all_lone ? 0.74 : 1.135;
+            sk_fixed = all_lone && one_pass ? 10.0 : 17.0;
+            one_scale = all_lone ? 0.95 : 1.04;
+        } else {
+            sk_tile = all_lone ? 1.37 : 1.36;
+            sk_fixed = 21.0 + 8.0 * std::max(0.0, static_cast<double>(c->num_sms) / std::max<int64_t>(grp_units, 1) - 3.0);
+            one_scale = all_lone ? (one_pass ? 0.85 : 0.95) : 0.90 - 0.36 * lone;
+        }
+        const double sk_est = (sk_fixed + sk_tile * static_cast<double>(grp_tiles) / c->num_sms) * 1e-6;
+        const double one_est = (tail ? tp.est : plan_est) * one_scale * (!one_pass ? 1.0 : d == 64 ? 0.95 : 0.9);
+        const bool sk_wins = sk_fits && !(one_pass && c->splitkv == 0) && sk_est <= one_est;
         bool sk = c->num_splits == 0 && (c->attn_kernel == 2 || (c->attn_kernel == 1 && sk_wins));
         if (sk) {
             if (sbuf.empty()) sbuf.resize(sizeof(SkParams));
