@@ -19,10 +19,11 @@
 // tile and epilogue run (no CTA launch, TMEM allocation or barrier set-up
 // between units).
 //
-// Roles (384 threads, warp 11 idle) as in replay_attn_kernel: softmax warpgroups 0 and 1
+// Roles (384 threads) as in replay_attn_kernel: softmax warpgroups 0 and 1
 // (one per q-tile, thread r owns row r), producer warps 8 (Q, K) and 10 (V)
 // (page table -> TMA boxes), MMA warp 9 (converged; one elected lane issues
-// tcgen05.mma).  Every role walks the same sequence of pieces, computed from the kernel parameters; barrier phases
+// tcgen05.mma), at d = 64 with two q-tiles warp 9 for the first and warp 11
+// for the second, else warp 11 idles.  Every role walks the same sequence of pieces, computed from the kernel parameters; barrier phases
 // run on across pieces (per q-tile tile counts for S / P / O, a global key
 // tile count for the K and V rings, a piece count for Q).  Two more barriers
 // than the one-unit kernel: q_empty (the piece's last S GEMMs are done, so the
@@ -54,8 +55,14 @@ struct SkCfg {
     static constexpr int kOffK = kOffQ + (ONE ? 1 : 2) * kTileBytes;
     static constexpr int kOffV = kOffK + kStages * kTileBytes;
     static constexpr int kOffBar = kOffV + kStages * kTileBytes;
-    // q_full, q_empty, k_full[S], k_empty[S], v_full[S], v_empty[S], s_full[2], p_full[2], o_done[2], o_free[2]
-    static constexpr int kNumBars = 2 + 4 * kStages + 8;
+    // q_full, q_empty, k_full[S], k_empty[S], v_full[S], v_empty[S], s_full[2], p_full[2], o_done[2], o_free[2],
+    // s_free[2]
+    static constexpr int kNumBars = 2 + 4 * kStages + 10;
+    // d = 64, two q-tiles: P_0 and P_1 in the 128 TMEM columns O leaves free, so that S_t(j+1) need not wait for
+    // P V_t(j), and an MMA warp per q-tile, as in the one-item kernel.  With P over S and one MMA warp, 1638
+    // tokens on 16k took 207.3 us a layer, now 190.3; the 6-agent batch, forced here, 404 -> 364 (one-item 370)
+    static constexpr bool kSepP = HD == 64 && !ONE;
+    static constexpr int kMmaWarps = kSepP ? 2 : 1;
     static constexpr int kOffMisc = kOffBar + kNumBars * 8;  // tmem slot, abort flag
     static constexpr int kSmemBytes = kOffMisc + 16;
     static constexpr int kDynSmem = kSmemBytes + 1024;       // alignment slack
@@ -321,6 +328,7 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
     const uint32_t b_p_full = b_s_full + 16;               // [2]
     const uint32_t b_o_done = b_p_full + 16;               // [2]
     const uint32_t b_o_free = b_o_done + 16;               // [2]
+    const uint32_t b_s_free = b_o_free + 16;               // [2] (kSepP) S_t has been read into registers
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + C::kOffMisc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + C::kOffMisc + 4);
     const WaitCtx wctx{abort_flag, p.status};
@@ -330,18 +338,19 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
     if (warp == 8) {
         if (lane == 0) {
             ptx::mbar_init(b_q_full, 1);
-            ptx::mbar_init(b_q_empty, 1);
+            ptx::mbar_init(b_q_empty, C::kMmaWarps);
             for (int s = 0; s < C::kStages; ++s) {
                 ptx::mbar_init(b_k_full + 8 * s, 1);
-                ptx::mbar_init(b_k_empty + 8 * s, 1);
+                ptx::mbar_init(b_k_empty + 8 * s, C::kMmaWarps);
                 ptx::mbar_init(b_v_full + 8 * s, 1);
-                ptx::mbar_init(b_v_empty + 8 * s, 1);
+                ptx::mbar_init(b_v_empty + 8 * s, C::kMmaWarps);
             }
             for (int t = 0; t < 2; ++t) {
                 ptx::mbar_init(b_s_full + 8 * t, 1);
                 ptx::mbar_init(b_p_full + 8 * t, 128);
                 ptx::mbar_init(b_o_done + 8 * t, 1);
                 ptx::mbar_init(b_o_free + 8 * t, 128);
+                ptx::mbar_init(b_s_free + 8 * t, 128);
             }
             *abort_flag = 0;
             ptx::fence_barrier_init();
@@ -431,7 +440,81 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
                     while (!ptx::mbar_try_wait(b_full + 8 * (i % C::kStages), (i / C::kStages) & 1) &&
                            ptx::globaltimer() - t0 < 4000000ull) {}
             }
-        } else if (warp == 9) {
+        } else if (C::kMmaWarps == 2 && (warp == 9 || warp == 11)) {
+            // =================================================== MMA issuers, d = 64 (converged warps)
+            // Warp 9 runs q-tile 0's GEMMs, warp 11 q-tile 1's.  Both pass through every key tile and piece; a
+            // tile or piece that the q-tile does not attend is passed on unread.
+            constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
+            constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
+            // warp-uniform copies (every lane holds the same values already)
+            const int t = __shfl_sync(0xffffffffu, warp == 11 ? 1 : 0, 0);
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+            const uint64_t q_desc = ptx::smem_desc_sw128(q_smem, 16, 1024) + t * (C::kTileBytes >> 4);
+            const uint64_t k_desc = ptx::smem_desc_sw128(k_smem0, 16, 1024);
+            const uint64_t v_desc = ptx::smem_desc_sw128(v_smem0, C::kRegionBytes, 1024);
+            const uint32_t tp = tm + 256 + 2 * HD + 64 * t;  // P_t
+            auto pass = [&](uint32_t bar) {
+                if (lane == 0) ptx::mbar_arrive(bar);
+                __syncwarp();
+            };
+            int gk = 0;   // key tiles passed so far (ring position)
+            int cnt = 0;  // tiles of this q-tile in earlier pieces (S, P and O phases)
+            int seg = 0;  // earlier pieces in which it had tiles (o_free phase)
+            bool ok = true;
+            Piece pc;
+            UnitGeo U;
+            for (int k = 0; ok && piece_of(P, cw, k, pc, U); ++k) {
+                const int n = __shfl_sync(0xffffffffu, q_geo(p, p.seqs[U.si], U.pair, t, pc.lo, pc.hi).ntiles, 0);
+                const int n_all = __shfl_sync(0xffffffffu, pc.hi - pc.lo, 0);
+                // S_t of the piece's tile j: its K has landed and the softmax holds the S_t before it in registers
+                auto s_tile = [&](int j) -> bool {
+                    const int s = (gk + j) % C::kStages;
+                    if (!wait_bar_warp(b_k_full + 8 * s, ((gk + j) / C::kStages) & 1, wctx)) return false;
+                    if (j >= n) {
+                        pass(b_k_empty + 8 * s);
+                        return true;
+                    }
+                    if (cnt + j > 0 && !wait_bar_warp(b_s_free + 8 * t, (cnt + j - 1) & 1, wctx)) return false;
+                    ptx::tc_fence_after();
+                    const uint64_t kd = k_desc + s * (C::kTileBytes >> 4);
+#pragma unroll
+                    for (int kk = 0; kk < HD / 16; ++kk) {
+                        const uint32_t off = ((kk >> 2) * C::kRegionBytes + (kk & 3) * 32) >> 4;
+                        mma_bf16_warp(tm + 128 * t, q_desc + off, kd + off, kIdescQK, kk > 0 ? 1u : 0u);
+                    }
+                    mma_commit_warp(b_s_full + 8 * t);
+                    mma_commit_warp(b_k_empty + 8 * s);         // K consumed by this q-tile
+                    if (j + 1 == n) mma_commit_warp(b_q_empty);  // the piece's last S GEMM reads Q
+                    return true;
+                };
+                if (!wait_bar_warp(b_q_full, k & 1, wctx)) break;
+                if (n == 0) pass(b_q_empty);
+                if (!s_tile(0)) break;
+                for (int j = 0; j < n_all; ++j) {
+                    if (j + 1 < n_all && !s_tile(j + 1)) { ok = false; break; }
+                    const int s = (gk + j) % C::kStages;
+                    if (!wait_bar_warp(b_v_full + 8 * s, ((gk + j) / C::kStages) & 1, wctx)) { ok = false; break; }
+                    if (j >= n) {
+                        pass(b_v_empty + 8 * s);
+                        continue;
+                    }
+                    // the first P V GEMM of a piece overwrites O_t: the previous piece's epilogue read it
+                    if (j == 0 && seg > 0 && !wait_bar_warp(b_o_free + 8 * t, (seg - 1) & 1, wctx)) { ok = false; break; }
+                    if (!wait_bar_warp(b_p_full + 8 * t, (cnt + j) & 1, wctx)) { ok = false; break; }
+                    ptx::tc_fence_after();
+                    const uint64_t vd = v_desc + s * (C::kTileBytes >> 4);
+#pragma unroll
+                    for (int kk = 0; kk < kBN / 16; ++kk)
+                        mma_bf16_ts_warp(tm + 256 + HD * t, tp + kk * 8, vd + (kk * 16 * 128 >> 4), kIdescPV,
+                                         (j > 0 || kk > 0) ? 1u : 0u);
+                    mma_commit_warp(b_o_done + 8 * t);
+                    mma_commit_warp(b_v_empty + 8 * s);  // V consumed by this q-tile
+                }
+                gk += n_all;
+                cnt += n;
+                seg += n > 0 ? 1 : 0;
+            }
+        } else if (C::kMmaWarps == 1 && warp == 9) {
             // =================================================== MMA issuer (the whole warp; one elected lane issues)
             constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(kBM, kBN, false);
             constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(kBM, HD, true);
@@ -585,6 +668,7 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
                 const int kbase = (pc.lo + j) * kBN;
                 // S buffer: the q-tile's own, or by tile parity
                 const uint32_t tS = ONE ? tmem + 128 * (j & 1) + lane_off : tmem + 128 * t + lane_off;
+                const uint32_t tP = C::kSepP ? tmem + 256 + 2 * HD + 64 * t + lane_off : tS;
                 const uint32_t b_s = ONE ? b_s_full + 8 * (j & 1) : b_s_full + 8 * t;
                 if (!wait_bar_warp(b_s, (ONE ? (ph >> (j & 1)) + (j >> 1) : cnt + j) & 1, wctx)) { ok = false; break; }
                 ptx::tc_fence_after();
@@ -599,6 +683,11 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
                     ptx::tmem_ld32(tS + 64, s2);
                     ptx::tmem_ld32(tS + 96, s3);
                     ptx::tmem_wait_ld();
+                }
+                if (C::kSepP) {
+                    // S_t(j) is in registers: the next S GEMM may overwrite it
+                    ptx::tc_fence_before();
+                    ptx::mbar_arrive(b_s_free + 8 * t);
                 }
                 if (kbase + kBN - 1 > G.pos_first) {  // tile crosses the causal diagonal of some row
 #pragma unroll
@@ -622,7 +711,12 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
                             acc[q & 3] = add2(acc[q & 3], e);
                             pk[q] = pack_bf16(e.x, e.y);
                         }
-                        tmem_st16(tS + ch * 16, pk);
+                        if (C::kSepP && ch == 0 && j > 0) {
+                            // P_t(j) goes to P_t's own columns once P V_t(j-1) has read P_t(j-1)
+                            if (!pv_done(j - 1)) ok = false;
+                            ptx::tc_fence_after();
+                        }
+                        tmem_st16(tP + ch * 16, pk);
                     }
                     const float2 a = add2(add2(acc[0], acc[1]), add2(acc[2], acc[3]));
                     return a.x + a.y;
@@ -631,6 +725,7 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
                 bool need = j == 0;
                 if (j > 0) {
                     rs = exp_tile(m_ref);
+                    if (!ok) break;
                     need = !(rs <= kTileSumLimit);
                 }
                 if (__any_sync(0xffffffffu, need)) {
@@ -667,6 +762,7 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
                     }
                     ptx::tmem_wait_st();
                     rs = exp_tile(m_ref);
+                    if (!ok) break;
                 }
                 l += rs;
                 ptx::tmem_wait_st();

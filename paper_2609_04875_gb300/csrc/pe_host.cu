@@ -1333,16 +1333,16 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         // 7 tiles per SM, 50 / 57 at 27, 172 / 169 at 108; 64 pairs 34 / 41 at 13, 178 / 166 at 107; 168 pairs
         // 143 / 120 at 70; 256 pairs 319 / 297 at 204, but 337 / 362 where a quarter of them are one q-tile,
         // which only the one-item kernel is done with sooner.  d = 64: 64 units of one q-tile 22 / 26 at 13,
-        // 115 / 95 at 108; 64 pairs 26 / 31 at 13, 136 / 139 at 108; 168 pairs 109 / 96 at 70.  A plan in one pass
-        // is left for a clear gain only: a last wave nearly empty, 168 pairs of 32 tiles 88 / 69 (d = 64: 67 / 56).
+        // 115 / 95 at 108; 64 pairs 26 / 29 at 13, 136 / 129 at 108; 168 pairs 109 / 90 at 70.  A plan in one pass
+        // is left for a clear gain only: a last wave nearly empty, 168 pairs of 32 tiles 88 / 69 (d = 64: 67 / 52).
         const bool sk_fits = 4 * grp_units >= c->num_sms && grp_units < 2 * static_cast<int64_t>(c->num_sms);
         const bool one_pass = !split && !tail;
         const bool all_lone = grp_lone == grp_units;
         const double lone = all_lone || grp_units == 0 ? 0.0 : static_cast<double>(grp_lone) / grp_units;
         double sk_tile, sk_fixed, one_scale;  // us a key tile per SM, us; measured over estimated time of the one-item plan
         if (d == 64) {
-            sk_tile = all_lone ? 0.74 : 1.135;
-            sk_fixed = all_lone && one_pass ? 10.0 : 17.0;
+            sk_tile = all_lone ? 0.74 : 1.06;
+            sk_fixed = !all_lone ? 15.0 : one_pass ? 10.0 : 17.0;
             one_scale = all_lone ? 0.95 : 1.04;
         } else {
             sk_tile = all_lone ? 1.37 : 1.36;
