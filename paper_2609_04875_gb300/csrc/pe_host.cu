@@ -874,7 +874,7 @@ pe_status run_decode(pe_cache *c, const std::vector<AttnItem> &items, int32_t la
 // ---- persistent stream-K plan of one launch group (replay_attn_sk_kernel)
 // Units are (sequence, kv-head, q-tile pair) in the kernel's order: sequences
 // as given (longest first), kv-head fastest, pairs heaviest first.  A unit
-// costs its key tiles plus kSkUnitCost for loading Q and writing the output;
+// costs its key tiles (sk_lone_cost each when it is one q-tile among pairs) plus kSkUnitCost for loading Q and writing the output;
 // CTA c takes the work between boundaries c and c + 1 at c / P of the total.
 // With cuts allowed a boundary falls inside a unit (at a key tile, each piece
 // at least kSkMinPiece tiles), else at the unit boundary nearest to it; cuts
@@ -883,6 +883,9 @@ pe_status run_decode(pe_cache *c, const std::vector<AttnItem> &items, int32_t la
 // "splitkv" = 1.
 constexpr double kSkUnitCost = 2.0;
 constexpr int kSkMinPiece = 2;
+// A key tile of a unit of one q-tile against one of two, in launches that mix them: 8 agents x 200 tokens (one unit
+// in four) on 8k 200.5 -> 180.6 us a layer, at d = 64 133.6 -> 125.4; 0.1 more or less costs 2 to 9 %.
+constexpr double sk_lone_cost(int head_dim) { return head_dim == 64 ? 0.75 : 0.85; }
 
 struct SkBound {
     int32_t u, t;  // unit and key tile (t = 0: the start of unit u)
@@ -908,7 +911,11 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
     p.oob_row = static_cast<int32_t>(c->pool_rows);
     p.scale_log2 = scale * 1.4426950408889634f;
     std::vector<int32_t> n_all;   // key tiles per unit
+    std::vector<double> wt;        // cost of one of its key tiles
     std::vector<double> cum{0.0};  // cost before each unit
+    bool pairs = false;            // some unit has two q-tiles
+    for (size_t i = lo; i < hi; ++i) pairs = pairs || static_cast<int64_t>(order[i].n_q) * g > kBM;
+    const double lone_cost = pairs ? sk_lone_cost(d) : 1.0;
     for (size_t i = lo; i < hi; ++i) {
         const AttnItem &it = order[i];
         AttnSeq &q = p.seqs[p.n_seqs++];
@@ -927,10 +934,12 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
             const int64_t q_last = std::min<int64_t>((qt_last + 1) * static_cast<int64_t>(bmq), it.n_q) - 1;
             const int32_t n = static_cast<int32_t>(ceil_div(c->len[it.seq] - it.n_q + q_last + 1, kBN));
             n_all.push_back(n);
-            cum.push_back(cum.back() + n + kSkUnitCost);
+            wt.push_back(2 * pair + 1 < q.n_qtiles ? 1.0 : lone_cost);
+            cum.push_back(cum.back() + n * wt.back() + kSkUnitCost);
         }
     }
     const int32_t U = static_cast<int32_t>(n_all.size());
+    auto unit_cost = [&](int32_t u) { return n_all[u] * wt[u] + kSkUnitCost; };
     auto unit_at = [&](double x) {  // the unit whose cost range holds x
         return static_cast<int32_t>(std::upper_bound(cum.begin(), cum.end(), x) - cum.begin()) - 1;
     };
@@ -952,7 +961,7 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
         pl.own.assign(nc, 0.0);
         for (int32_t r = 0; r < pl.R; ++r)
             for (int32_t k = 0; k < nc; ++k)
-                pl.own[k] += n_all[r * nc + ((r & 1) ? nc - 1 - k : k)] + kSkUnitCost;
+                pl.own[k] += unit_cost(r * nc + ((r & 1) ? nc - 1 - k : k));
         const double W = cum.back() - cum[T0];
         const double mean = cum.back() / nc;
         std::vector<double> want(nc), pos(nc + 1, 0.0);
@@ -967,10 +976,10 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
             if (x < cum.back()) {
                 const int32_t u = std::min(unit_at(x), U - 1);
                 const double off = x - cum[u];
-                const int32_t t = static_cast<int32_t>(std::lround(off - kSkUnitCost));
+                const int32_t t = static_cast<int32_t>(std::lround((off - kSkUnitCost) / wt[u]));
                 bd = SkBound{u, 0};
                 if (cuts && t >= kSkMinPiece && n_all[u] - t >= kSkMinPiece) bd.t = t;
-                else if (off > 0.5 * (n_all[u] + kSkUnitCost)) bd = SkBound{u + 1, 0};
+                else if (off > 0.5 * unit_cost(u)) bd = SkBound{u + 1, 0};
             }
             const SkBound &prev = pl.b[k - 1];
             if (bd.u < prev.u || (bd.u == prev.u && bd.t < prev.t)) bd = prev;  // an empty stretch
@@ -980,7 +989,7 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
     // the busiest CTA: its rounds plus its tail stretch (a cut piece pays its own set-up)
     auto busiest = [&](const Plan &pl) {
         auto at = [&](const SkBound &x) {
-            return (x.u < U ? cum[x.u] : cum.back()) + (x.t > 0 ? kSkUnitCost + x.t : 0.0);
+            return (x.u < U ? cum[x.u] : cum.back()) + (x.t > 0 ? kSkUnitCost + x.t * wt[x.u] : 0.0);
         };
         double worst = 0.0;
         for (int32_t k = 0; k < pl.nc; ++k) {
@@ -1147,22 +1156,24 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
 
     // split-KV decision over the whole launch group; plan_est: the cost model's time of the plan
     double plan_est = 0.0;
-    // the group's units (pairs of q-tiles x kv-heads), their key tiles, and how many units are one q-tile
-    int64_t grp_units = 0, grp_tiles = 0, grp_lone = 0;
+    // the group's units (pairs of q-tiles x kv-heads) and their key tiles, and those of units of one q-tile
+    int64_t grp_units = 0, grp_tiles = 0, grp_lone = 0, grp_lone_tiles = 0;
     // time of one key tile per CTA in the cost models: about 1.5 us, compute- or HBM-bound alike; 1 us at
     // d = 64, whose next S GEMM overlaps the softmax
     const double tile_s = d == 64 ? 1.0e-6 : 1.5e-6;
     // splitkv: the "splitkv" option's value for this plan (-1 auto, 0 never, 1 always)
     auto plan_group = [&](size_t lo, size_t hi, AttnParams &p, bool &split, int splitkv) -> pe_status {
         // C CTAs (pairs of q-tiles x kv-heads), W key tiles per CTA on average.
-        int64_t C = 0, tiles = 0, rows = 0, valid_rows = 0, max_tiles = 0;
+        int64_t C = 0, tiles = 0, lone_tiles = 0, rows = 0, valid_rows = 0, max_tiles = 0;
         for (size_t i = lo; i < hi; ++i) {
             const AttnItem &it = order[i];
             const int64_t len = c->len[it.seq];
             const int64_t nqt = ceil_div(static_cast<int64_t>(it.n_q) * g, kBM);
             for (int64_t pp = 0; pp < ceil_div(nqt, 2); ++pp) {
                 const int64_t q_last = std::min<int64_t>((std::min(2 * pp + 1, nqt - 1) + 1) * bmq, it.n_q) - 1;
-                tiles += ceil_div(len - it.n_q + q_last + 1, kBN) * hkv;
+                const int64_t n = ceil_div(len - it.n_q + q_last + 1, kBN) * hkv;
+                tiles += n;
+                if (2 * pp + 1 >= nqt) lone_tiles += n;
             }
             C += ceil_div(nqt, 2) * hkv;
             rows += nqt * hkv * kBM;                               // workspace slots (whole tiles)
@@ -1203,6 +1214,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         plan_est = cost(best);
         grp_units = C;
         grp_tiles = tiles;
+        grp_lone_tiles = lone_tiles;
         grp_lone = 2 * C - rows / kBM;
         int split_tiles = static_cast<int>(max_tiles);
         split = best > 1 || splitkv == 1;
@@ -1325,40 +1337,52 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         if (s != PE_OK) return s;
         TailPlan tp;
         const bool tail = hi - lo == 1 && c->splitkv == -1 && c->num_splits == 0 && plan_tail(order[lo], tp);
-        // The persistent stream-K kernel where it should beat the one-item plan, among launches whose units
-        // fill between a quarter of the SMs and two waves.  One CTA per SM takes an equal stretch of key
-        // tiles; its longer start and end (the parts of cut units are merged by single warps, about 2 us a
-        // part) pay where the one-item plan leaves SMs idle for long.  Its estimate is linear in the key
-        // tiles per SM.  Measured, one-item / persistent us a layer, d = 128: 64 units of one q-tile 20 / 27 at
-        // 7 tiles per SM, 50 / 57 at 27, 172 / 169 at 108; 64 pairs 34 / 41 at 13, 178 / 166 at 107; 168 pairs
-        // 143 / 120 at 70; 256 pairs 319 / 297 at 204, but 337 / 362 where a quarter of them are one q-tile,
-        // which only the one-item kernel is done with sooner.  d = 64: 64 units of one q-tile 22 / 26 at 13,
-        // 115 / 95 at 108; 64 pairs 26 / 29 at 13, 136 / 129 at 108; 168 pairs 109 / 90 at 70.  A plan in one pass
-        // is left for a clear gain only: a last wave nearly empty, 168 pairs of 32 tiles 88 / 69 (d = 64: 67 / 52).
-        const bool sk_fits = 4 * grp_units >= c->num_sms && grp_units < 2 * static_cast<int64_t>(c->num_sms);
-        const bool one_pass = !split && !tail;
-        const bool all_lone = grp_lone == grp_units;
-        const double lone = all_lone || grp_units == 0 ? 0.0 : static_cast<double>(grp_lone) / grp_units;
-        double sk_tile, sk_fixed, one_scale;  // us a key tile per SM, us; measured over estimated time of the one-item plan
-        if (d == 64) {
-            sk_tile = all_lone ? 0.74 : 1.06;
-            sk_fixed = !all_lone ? 15.0 : one_pass ? 10.0 : 17.0;
-            one_scale = all_lone ? 0.95 : 1.04;
+        // The persistent stream-K kernel where it should beat the one-item plan.  One CTA per SM takes an equal
+        // stretch of key tiles and goes from unit to unit without a gap; its longer start and end (the parts
+        // of cut units are merged by single warps, about 2 us a part) pay where the one-item plan leaves SMs
+        // idle for long, and at d = 64, where the gaps between CTAs weigh more.  Measured, one-item / persistent
+        // us a layer, d = 128: 64 units of one q-tile 20 / 27 at 7 key tiles per SM, 50 / 57 at 27, 172 / 169 at
+        // 108; 64 pairs 34 / 41 at 13, 178 / 166 at 107; 168 pairs 143 / 120 at 70; 312 pairs 254 / 203 at 129; 5016
+        // pairs (the 16-agent batch) 1670 / 1805.  d = 64: 64 units of one q-tile 22 / 26 at 13, 115 / 95 at 108;
+        // 64 pairs 26 / 29 at 13, 136 / 129 at 108; 168 pairs 109 / 90 at 70; 768 pairs 136 / 118 at 81; 1584 pairs
+        // 355 / 343 at 286; 1440 pairs 877 / 883 at 796.
+        const double n_sm = c->num_sms, units = static_cast<double>(std::max<int64_t>(grp_units, 1));
+        const bool one_pass = !split && !tail, all_lone = grp_lone == grp_units;
+        const bool many = grp_units >= 2 * static_cast<int64_t>(c->num_sms);
+        const double x = grp_tiles / n_sm;                                                  // key tiles per SM
+        const double xw = all_lone ? x : x - (1.0 - sk_lone_cost(d)) * grp_lone_tiles / n_sm;  // as plan_sk weighs them
+        // One pass of a launch with pairs: its waves, the last one counted for most of what it lacks of a full
+        // one (less where one sequence's heaviest-first items end it with the light ones).
+        const double waves = units / n_sm;
+        const double wave_us = (d == 64 ? 1.05 : 1.38) * x / waves + (d == 64 ? 5.0 : 6.0);
+        const double last = waves <= 1.0 ? 1.0 : (hi - lo == 1 && waves > 3.0 ? 0.4 : 0.8);
+        const double pass_us = wave_us * (waves + last * (std::ceil(waves) - waves));
+        const double plan_us = (tail ? tp.est : plan_est) * 1e6;
+        double sk_us, one_us;
+        if (all_lone) {
+            sk_us = d == 64 ? 0.74 * x + (one_pass ? 8.0 + 3.0 * waves : 17.0)
+                            : 1.37 * x + 21.0 + 8.0 * std::max(0.0, 1.0 / waves - 3.0);
+            one_us = plan_us * (one_pass ? (d == 64 ? 0.9 : 0.77) : 0.95);
+        } else if (d == 64) {
+            sk_us = 13.0 + 1.05 * xw + 2.7 * waves;
+            one_us = one_pass ? 0.97 * pass_us : 1.04 * plan_us;
+        } else if (many) {
+            sk_us = 13.0 + 1.5 * xw + 4.5 * waves;
+            one_us = one_pass ? 0.95 * pass_us : tail ? 0.0 : 0.9 * plan_us;
         } else {
-            sk_tile = all_lone ? 1.37 : 1.36;
-            sk_fixed = 21.0 + 8.0 * std::max(0.0, static_cast<double>(c->num_sms) / std::max<int64_t>(grp_units, 1) - 3.0);
-            one_scale = all_lone ? (one_pass ? 0.85 : 0.95) : 0.90 - 0.36 * lone;
+            sk_us = 21.0 + 1.36 * xw + 8.0 * std::max(0.0, 1.0 / waves - 3.0);
+            // (a unit of one q-tile among pairs is less work than the cost model counts)
+            one_us = plan_us * (0.90 - 0.15 * grp_lone / units) * (one_pass ? 0.9 : 1.0);
         }
-        const double sk_est = (sk_fixed + sk_tile * static_cast<double>(grp_tiles) / c->num_sms) * 1e-6;
-        const double one_est = (tail ? tp.est : plan_est) * one_scale * (!one_pass ? 1.0 : d == 64 ? 0.95 : 0.9);
-        const bool sk_wins = sk_fits && !(one_pass && c->splitkv == 0) && sk_est <= one_est;
+        const bool sk_fits = 4 * grp_units >= c->num_sms && grp_units <= 16384 && !(all_lone && d != 64 && many);
+        const bool sk_wins = sk_fits && !(one_pass && c->splitkv == 0) && sk_us <= one_us;
         bool sk = c->num_splits == 0 && (c->attn_kernel == 2 || (c->attn_kernel == 1 && sk_wins));
         if (sk) {
             if (sbuf.empty()) sbuf.resize(sizeof(SkParams));
             SkParams &P = *reinterpret_cast<SkParams *>(sbuf.data());
             if ((s = plan_sk(c, order, lo, hi, layer, out, hq, scale, P)) != PE_OK) return s;
             // no unit cut (the workspace is too small for the parts): nothing gained over the one pass
-            if (c->attn_kernel == 1 && one_pass && P.n_slots == 0) sk = false;
+            if (c->attn_kernel == 1 && one_pass && d != 64 && !many && P.n_slots == 0) sk = false;
         }
         if (sk) {
             SkParams &P = *reinterpret_cast<SkParams *>(sbuf.data());
