@@ -1,0 +1,147 @@
+"""The prefill, merge, decode and copy kernels' forms at the sizes where one
+gives way to the next: one-q-tile launches of a few key tiles, pairs whose
+q-tiles end at different key tiles (with V's producer apart or not), split
+merges around their batch of splits and their block shapes, persistent pieces of
+one or two q-tiles, decode merges of one and of many chunks, and appends, crops
+and copy-on-write around the limits of their parameter blocks.  Attention is held
+to the gate of tests/parity.py against the fp64 oracle; everything that moves
+bytes is compared exactly."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from gpu_common import Pair, assert_close, dev, requires_cuda
+from test_gpu_fork import _check_pools
+
+pytestmark = [pytest.mark.gpu, requires_cuda]
+
+
+def _batch(d, hq, hkv, ps, lens, nqs, options, seed):
+    """One launch over sequences of `lens` keys and `nqs` queries against the oracle; returns the plan."""
+    npg = sum(-(-n // ps) for n in lens) + 4
+    pair = Pair(1, hkv, d, ps, npg, len(lens), max(-(-n // ps) for n in lens) + 1, seed=seed)
+    for key, value in options.items():
+        pair.gpu.set_option(key, value)
+    g = synth.rng(seed, 71)
+    seqs = []
+    for n in lens:
+        s = pair.seq()
+        pair.append(s, synth.normal_bf16(g, (1, n, hkv, d)), synth.normal_bf16(g, (1, n, hkv, d)))
+        seqs.append(s)
+    cu = [0] + [int(x) for x in np.cumsum(nqs)]
+    q = synth.normal_bf16(g, (cu[-1], hq, d))
+    out = pair.gpu.replay_attn_batch(seqs, 0, dev(q), cu)
+    torch.cuda.synchronize()
+    for i, s in enumerate(seqs):
+        ref = oracle.replay_attention(pair.orc, s, 0, q[cu[i]:cu[i + 1]], 1 / math.sqrt(d))
+        assert_close(out[cu[i]:cu[i + 1]], ref, f"d={d} ps={ps} lens={lens} nqs={nqs} {options} seq {i}")
+    assert pair.gpu.device_status() == 0
+    return pair.gpu.last_attn_plan()
+
+
+@pytest.mark.parametrize("kernel", [0, 2])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("split", [0, 1])
+def test_one_q_tile_launches_of_few_key_tiles(kernel, d, split):
+    """Every unit one q-tile, 1 to 5 key tiles (the last ragged), whole or cut into pieces of 1 to 4."""
+    lens = [40, 128, 129, 256, 300, 511, 640]
+    opts = {"attn_kernel": kernel, "splitkv": split}
+    if split and kernel == 0:
+        opts["num_splits"] = 2
+    if split and kernel == 2:
+        opts["attn_ctas"] = 11
+    _batch(d, 8, 2, 16, lens, [32, 20, 17, 32, 31, 9, 32], opts, seed=3 + d)
+
+
+@pytest.mark.parametrize("kernel", [0, 2])
+@pytest.mark.parametrize("d,ps", [(64, 8), (64, 16), (64, 32), (128, 8), (128, 64)])
+def test_pairs_whose_q_tiles_end_apart(kernel, d, ps):
+    """g = 16: 8 queries a q-tile, so a pair's second q-tile reaches one key tile further where the first
+    ends on a tile's edge; odd q-tile counts leave a lone one; 1 to 3 key tiles exercise every ring slot."""
+    _batch(d, 16, 1, ps, [128, 136, 264, 390, 1000], [16, 24, 136, 7, 100], {"attn_kernel": kernel}, seed=d + ps)
+    _batch(d, 16, 1, ps, [264, 900], [136, 300], {"attn_kernel": kernel, "splitkv": 1, "attn_ctas": 7 if kernel else 0,
+                                                  "num_splits": 0 if kernel else 3}, seed=d + ps + 1)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("splits", [2, 4, 5, 8, 9, 17])
+@pytest.mark.parametrize("wide", [False, True])
+def test_split_merge_shapes(d, splits, wide):
+    """Split counts around the merge's batches (4, then 8), with few partial rows (blocks of one warp) and
+    with more than 8 MB of them (a block an SM)."""
+    hq, hkv = (64, 8) if wide else (8, 2)
+    nqs = [130, 70, 1] if wide else [30, 5]
+    lens = [2176, 900, 70] if wide else [2176, 500]
+    plan = _batch(d, hq, hkv, 16, lens, nqs, {"attn_kernel": 0, "splitkv": 1, "num_splits": splits, "decode_kernel": 0},
+                  seed=splits)
+    assert plan[1] == -(-17 // -(-17 // splits)), plan
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_default_plans_of_mixed_launches(d):
+    """The plan's own choice over launches of few and of many units, with units of one q-tile among pairs."""
+    kinds = set()
+    for i, (lens, nqs, hq, hkv) in enumerate([
+            ([1500, 900, 2000, 700], [200, 33, 129, 60], 32, 8), ([600] * 24, [40] * 24, 16, 8),
+            ([3000], [700], 32, 8), ([900] * 3, [300] * 3, 64, 8), ([2500, 2600], [20, 20], 32, 8)]):
+        split, _, ctas = _batch(d, hq, hkv, 16, lens, nqs, {}, seed=40 + i)
+        kinds.add((split, ctas == 152))
+    assert len(kinds) > 1, kinds
+
+
+@pytest.mark.parametrize("d,hq,hkv", [(128, 8, 2), (64, 16, 1), (128, 32, 8)])
+@pytest.mark.parametrize("chunks_per_sm", [None, 1, 64])
+def test_decode_merges_of_one_and_many_chunks(d, hq, hkv, chunks_per_sm):
+    """Items of 1 chunk (no merge) to 71 one-tile chunks (more than one round trip of the merge) in one launch."""
+    options = {} if chunks_per_sm is None else {"decode_chunks_per_sm": chunks_per_sm}
+    _batch(d, hq, hkv, 16, [100, 128, 1025, 9000, 4097], [1] * 5, options, seed=d + hq)
+
+
+@pytest.mark.parametrize("n", [1, 16, 17, 40])
+def test_append_and_crop_around_the_small_parameter_blocks(n):
+    """n sequences appended and cropped in one call each, the first append of 8 pages a sequence: 16 sequences
+    make 128 pages, and 17 leave the small blocks by both counts."""
+    hkv, d, ps, L = 2, 64, 16, 2
+    pair = Pair(L, hkv, d, ps, 9 * n + 8, n, 10, seed=n)
+    g = synth.rng(n, 72)
+    seqs = [pair.seq() for _ in range(n)]
+    for lens in ([128] * n, [1 + (7 * i) % 15 for i in range(n)]):
+        cu = [0] + [int(x) for x in np.cumsum(lens)]
+        k, v = (synth.normal_bf16(g, (L, cu[-1], hkv, d)) for _ in range(2))
+        pair.gpu.append_kv_batch(seqs, dev(k), dev(v), cu)
+        for i, s in enumerate(seqs):
+            pair.orc.append(s, k[:, cu[i]:cu[i + 1]], v[:, cu[i]:cu[i + 1]])
+        pair.check_state(seqs)
+    _check_pools(pair, L, hkv, ps, d)
+    taus = [1 + (5 * i) % 40 for i in range(n)]
+    pair.gpu.crop_batch(seqs, taus)
+    for s, tau in zip(seqs, taus):
+        pair.orc.crop(s, tau)
+    pair.check_state(seqs)
+    _check_pools(pair, L, hkv, ps, d)
+
+
+@pytest.mark.parametrize("branches", [1, 63, 64, 65])
+def test_copy_on_write_of_many_branches_in_one_append(branches):
+    """Each branch of a base whose last page is half full gets its own copy of that page in one append."""
+    hkv, d, ps, L, T = 2, 64, 16, 2, 40
+    pair = Pair(L, hkv, d, ps, 3 + 2 * branches + 4, branches + 1, 5, seed=branches)
+    g = synth.rng(branches, 73)
+    base = pair.seq()
+    pair.append(base, synth.normal_bf16(g, (L, T, hkv, d)), synth.normal_bf16(g, (L, T, hkv, d)))
+    seqs = []
+    for _ in range(branches):
+        a, b = pair.gpu.seq_fork(base), pair.orc.seq_fork(base)
+        assert a == b
+        seqs.append(a)
+    cu = list(range(0, 3 * branches + 1, 3))
+    k, v = (synth.normal_bf16(g, (L, cu[-1], hkv, d)) for _ in range(2))
+    pair.gpu.append_kv_batch(seqs, dev(k), dev(v), cu)
+    for i, s in enumerate(seqs):
+        pair.orc.append(s, k[:, cu[i]:cu[i + 1]], v[:, cu[i]:cu[i + 1]])
+    pair.check_state([base] + seqs)
+    _check_pools(pair, L, hkv, ps, d)
