@@ -1351,18 +1351,19 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         const bool many = grp_units >= 2 * static_cast<int64_t>(c->num_sms);
         const double x = grp_tiles / n_sm;                                                  // key tiles per SM
         const double xw = all_lone ? x : x - (1.0 - sk_lone_cost(d)) * grp_lone_tiles / n_sm;  // as plan_sk weighs them
-        // One pass of a launch with pairs: its waves, the last one counted for most of what it lacks of a full
+        // One pass: its waves, the last one counted for most of what it lacks of a full
         // one (less where one sequence's heaviest-first items end it with the light ones).
         const double waves = units / n_sm;
-        const double wave_us = (d == 64 ? 1.05 : 1.38) * x / waves + (d == 64 ? 5.0 : 6.0);
+        const double wave_us = d == 128 ? 1.38 * x / waves + 6.0
+                                        : (all_lone ? 0.87 * x / waves + 6.5 : 1.05 * x / waves + 5.0);
         const double last = waves <= 1.0 ? 1.0 : (hi - lo == 1 && waves > 3.0 ? 0.4 : 0.8);
         const double pass_us = wave_us * (waves + last * (std::ceil(waves) - waves));
         const double plan_us = (tail ? tp.est : plan_est) * 1e6;
         double sk_us, one_us;
         if (all_lone) {
-            sk_us = d == 64 ? 0.74 * x + (one_pass ? 8.0 + 3.0 * waves : 17.0)
+            sk_us = d == 64 ? 0.74 * x + (one_pass && waves > 0.8 ? 8.0 + 3.0 * waves : 17.0)
                             : 1.37 * x + 21.0 + 8.0 * std::max(0.0, 1.0 / waves - 3.0);
-            one_us = plan_us * (one_pass ? (d == 64 ? 0.9 : 0.77) : 0.95);
+            one_us = !one_pass ? 0.95 * plan_us : d == 64 ? 0.97 * pass_us : 0.77 * plan_us;
         } else if (d == 64) {
             sk_us = 13.0 + 1.05 * xw + 2.7 * waves;
             one_us = one_pass ? 0.97 * pass_us : 1.04 * plan_us;
