@@ -308,21 +308,21 @@ def oracle_tokens_per_s(units, budget_s, seed=7):
 # DRAM traffic per attention launch from one ncu capture (profiles/), valid only
 # while the kernel source is the one that was captured.
 NCU_TRAFFIC = {
-    "tiny": {"bytes": 1.5081e6, "profile": "profiles/traffic_attention_configs.md", "kernels": ["prefill"],
-             "src_sha256": {"prefill": "91bcdf4963eaa5385a46b5fc32b465f5b50af0d236a020b33013751418d6a9b6"}},
-    "agent_batch": {"bytes": 684.646e6 + 315.236e6, "profile": "profiles/traffic_attention_configs.md",
-                    "kernels": ["prefill"], "src_sha256": {"prefill": "91bcdf4963eaa5385a46b5fc32b465f5b50af0d236a020b33013751418d6a9b6"}},
-    "short_suffix": {"bytes": 1.0883e9 + 5.88058e6, "profile": "profiles/traffic_attention_configs.md",
-                     "kernels": ["prefill_sk"], "src_sha256": {"prefill_sk": "b25d958540e6002039fda210f04a46af7fb34514ee9402af13b2c16be2709172"}},
-    "long_suffix": {"bytes": 1.41056e9 + 1.0372e9, "profile": "profiles/traffic_attention_configs.md",
-                    "kernels": ["prefill"], "src_sha256": {"prefill": "91bcdf4963eaa5385a46b5fc32b465f5b50af0d236a020b33013751418d6a9b6"}},
+    "tiny": {"bytes": 1.510912e6, "profile": "profiles/traffic_attention_configs.md", "kernels": ["prefill"],
+             "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f"}},
+    "agent_batch": {"bytes": 685.47584e6 + 315.327744e6, "profile": "profiles/traffic_attention_configs.md",
+                    "kernels": ["prefill"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f"}},
+    "short_suffix": {"bytes": 1.087881216e9 + 5.398016e6, "profile": "profiles/traffic_attention_configs.md",
+                     "kernels": ["prefill_sk"], "src_sha256": {"prefill_sk": "3818ae2364ef494941b6919759e1d90d82f93b7381afc5fd873033a9b55a4392"}},
+    "long_suffix": {"bytes": 1.41151616e9 + 1.03740288e9, "profile": "profiles/traffic_attention_configs.md",
+                    "kernels": ["prefill"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f"}},
     # one sweep step's 224 attention launches (5 forget requests x 32 layers, two launches per layer where a
     # tail launch runs), per layer: bytes / 160
-    "tau_sweep": {"bytes": (48092.5e6 + 8159.95e6) / 160, "profile": "profiles/traffic_attention_configs.md",
-                  "kernels": ["prefill", "prefill_sk"], "src_sha256": {"prefill": "91bcdf4963eaa5385a46b5fc32b465f5b50af0d236a020b33013751418d6a9b6", "prefill_sk": "b25d958540e6002039fda210f04a46af7fb34514ee9402af13b2c16be2709172"}},
-    "decode_batch": {"bytes": 341.569792e6 + 3.933952e6, "profile": "profiles/decode_tc_decode_batch.md",
+    "tau_sweep": {"bytes": (47813.435e6 + 7977.683e6) / 160, "profile": "profiles/traffic_attention_configs.md",
+                  "kernels": ["prefill", "prefill_sk"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f", "prefill_sk": "3818ae2364ef494941b6919759e1d90d82f93b7381afc5fd873033a9b55a4392"}},
+    "decode_batch": {"bytes": 341.534464e6 + 3.879168e6, "profile": "profiles/decode_tc_decode_batch.md",
                      "kernels": ["decode"],
-                     "src_sha256": {"decode": "a29203afa92b6d3d8108227a2ee31a613331b3c42dd2904b8ef84b5de69006ab"}},
+                     "src_sha256": {"decode": "92c511c1911bfb21c61432aa9bdf4df8b5b389e7497f2625650667460bf98173"}},
 }
 CSRC = os.path.join(ROOT, "paper_2609_04875_gb300", "csrc")
 # (file, first line of the kernel's source, the text that follows it): the span that is hashed

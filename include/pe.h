@@ -261,10 +261,10 @@ pe_status pe_cache_pools(const pe_cache *cache, void **k_pool, void **v_pool);
  * tcgen05 with keys on the MMA's M side (d = 64 and 128), split items merged
  * by a combine launch; 2: CUDA cores, split-KV merged in-kernel; 0: no
  * decode kernel (the prefill kernel serves every call); "attn_kernel" = 1
- * (default) / 2 / 0: the prefill kernel -- 1: the persistent stream-K kernel
- * for launch groups whose one-work-item-per-CTA plan would need key splits or
- * a tail launch and whose q-tile pairs x Hkv number between a quarter of the
- * SMs and two waves, the one-item kernel otherwise; 2: always persistent; 0:
+ * (default) / 2 / 0: the prefill kernel -- 1: the one-item kernel or the
+ * persistent stream-K kernel, whichever plan's estimated time is smaller (the
+ * persistent one from q-tile pairs x Hkv of a quarter of the SMs on, and with
+ * "splitkv" = 0 not in place of a single pass); 2: always persistent; 0:
  * always one-item; "attn_ctas" = 0 (auto) or the persistent kernel's CTA
  * count; "attn_order" = -1 (auto) / 0 / 1: how the one-item kernel numbers a
  * sequence's CTAs -- 0: kv-heads fastest, every head's heaviest q-tile pairs
