@@ -132,6 +132,7 @@ struct pe_cache {
     int attn_ctas = 0;            // persistent kernel's CTA count (0 = chosen by the planner)
     int attn_order = -1;          // one-item kernel's item order: -1 auto, 0 kv-heads fastest, 1 pairs fastest
     int64_t launches = 0;
+    bool ends_in_merge = false;   // the last attention call's last launch was the decode merge
     int32_t last_split = 0, last_splits = 0, last_ctas = 0;  // plan of the last attention launch
     Journal jr;                   // changes of the call in progress
     std::vector<int64_t> *plan_rec = nullptr;  // set only inside pe_attn_plan_launches: record, do not launch
@@ -543,8 +544,10 @@ pe_status apply_cow(pe_cache *c, int32_t seq, CowList &cow, cudaStream_t st)
 // Pops pages for every plan (the caller checked there are enough), then
 // launches the copies.  Launches are cut so that each carries at most
 // kMaxSegs segments and kAppendMaxPages new page ids.
+// `beside`: the stream's last launch is a decode merge of the same call, and the
+// first append launch may run beside it (not one that follows copies-on-write).
 pe_status apply_appends(pe_cache *c, const std::vector<AppendPlan> &plans, const void *K, const void *V,
-                        int64_t n_total, cudaStream_t st)
+                        int64_t n_total, cudaStream_t st, bool beside = false)
 {
     const int ps = c->cfg.page_size;
     AppendParams pbuf;  // (only the header, the segments and the page ids in use are written: 15 KB otherwise)
@@ -568,6 +571,8 @@ pe_status apply_appends(pe_cache *c, const std::vector<AppendPlan> &plans, const
     CowList cow;
     auto flush = [&]() -> pe_status {
         if (p->n_segs == 0) return PE_OK;
+        p->beside = beside && cow.p.n == 0 ? 1 : 0;
+        beside = false;
         pe_status cs = cow.flush(c, st);
         if (cs != PE_OK) return cs;
         p->n_new = pages_in_launch;
@@ -797,6 +802,7 @@ pe_status run_decode(pe_cache *c, const std::vector<AttnItem> &items, int32_t la
             cudaError_t e = launch_decode_attn(d, rb, true, c->tm_kd, c->tm_vd, p, st);
             if (e != cudaSuccess) return cuda_fail(e, "decode attention launch");
             c->launches++;
+            c->ends_in_merge = any_split;
             continue;
         }
         int64_t max_rows = 1, work = 0, max_tiles = 1;
@@ -1140,6 +1146,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
             record_launch(c, 3, false, dp, 0);
         }
     } else if (!dec.empty()) {
+        c->ends_in_merge = false;
         pe_status s = run_decode(c, dec, layer, Q, out, hq, scale, st);
         if (s != PE_OK) return s;
     }
@@ -1147,6 +1154,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         return c->len[a.seq] > c->len[b.seq];
     });
     if (order.empty()) return PE_OK;
+    c->ends_in_merge = false;
 
     CUtensorMap tm_q, tm_o;  // Q, and the output as a map of the same shape (TMA stores of full q-tiles)
     const bool rec = c->plan_rec != nullptr;  // a plan query: no tensors, no launches
@@ -1895,6 +1903,15 @@ pe_status pe_replay_rounds(pe_cache *c, int32_t n, const int32_t *seqs, int32_t 
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     CallTxn tx(c, st);
     const int64_t row_bytes = static_cast<int64_t>(num_q_heads) * c->cfg.head_dim * 2;  // one bf16 [Hq][d] row
+    // A round's append may run beside the merge of the round before, which writes `out`.
+    auto apart = [](const void *a, int64_t na, const void *b, int64_t nb) {
+        const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+        return x + static_cast<uint64_t>(na) <= y || y + static_cast<uint64_t>(nb) <= x;
+    };
+    const int64_t out_bytes = c->cfg.num_layers * N * row_bytes;
+    const int64_t kv_bytes = static_cast<int64_t>(c->cfg.num_layers) * N * c->cfg.num_kv_heads * c->cfg.head_dim * 2;
+    const bool out_apart = apart(out, out_bytes, K, kv_bytes) && apart(out, out_bytes, V, kv_bytes);
+    bool after_merge = false;  // the call's last launch is a decode merge
     std::vector<int32_t> done(n, 0);
     std::vector<AppendPlan> plans;
     std::vector<AttnItem> items;
@@ -1912,7 +1929,7 @@ pe_status pe_replay_rounds(pe_cache *c, int32_t n, const int32_t *seqs, int32_t 
             done[i] += t;
         }
         if (plans.empty()) continue;
-        if ((s = apply_appends(c, plans, K, V, N, st)) != PE_OK) return tx.end(s);
+        if ((s = apply_appends(c, plans, K, V, N, st, after_merge && out_apart)) != PE_OK) return tx.end(s);
         if (c->host_only) continue;
         for (int32_t layer = 0; layer < c->cfg.num_layers; ++layer) {
             const int64_t off = static_cast<int64_t>(layer) * N * row_bytes;
@@ -1920,6 +1937,7 @@ pe_status pe_replay_rounds(pe_cache *c, int32_t n, const int32_t *seqs, int32_t 
                               num_q_heads, softmax_scale, st);
             if (s != PE_OK) return tx.end(s);
         }
+        after_merge = c->ends_in_merge;
     }
     return tx.end(PE_OK);
 }

@@ -43,6 +43,7 @@ struct AppendParamsT {
     int64_t *seq_len;      // device mirror [max_seqs]
     int32_t L, hkv, dvec, ps, num_pages, n_total, n_segs, seg_tokens;
     int32_t n_new;         // page ids carried
+    int32_t beside;        // 1: runs beside the decode merge launched just before (append_kv_kernel)
     AppendSeg segs[SEGS];
     int32_t new_pages[PAGES];
 };

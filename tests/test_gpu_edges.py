@@ -145,3 +145,40 @@ def test_copy_on_write_of_many_branches_in_one_append(branches):
         pair.orc.append(s, k[:, cu[i]:cu[i + 1]], v[:, cu[i]:cu[i + 1]])
     pair.check_state([base] + seqs)
     _check_pools(pair, L, hkv, ps, d)
+
+
+@pytest.mark.parametrize("keys", [(60, 90), (700, 1300), (100, 3000)])
+def test_rounds_equal_their_calls_one_by_one(keys):
+    """Decode rounds in one call, where a round's append runs beside the merge before it, against the same
+    appends and attention calls made one by one: the same output bits, pages and lengths.  Items of one
+    chunk (no merge), of several, and both; a fork's copy-on-write before the first append."""
+    hq, hkv, d, ps, rounds = 32, 8, 128, 16, 12
+    g = synth.rng(sum(keys), 74)
+    base = [(synth.normal_bf16(g, (1, n, hkv, d)), synth.normal_bf16(g, (1, n, hkv, d))) for n in keys]
+    n = len(keys) + 1
+    cu = [rounds * i for i in range(n + 1)]
+    K, V, Q = (dev(synth.normal_bf16(g, (1, cu[-1], h, d))) for h in (hkv, hkv, hq))
+    outs, pools = [], []
+    for whole in (True, False):
+        pair = Pair(1, hkv, d, ps, sum(-(-k // ps) for k in keys) + 2 * n + 8, n, 220, seed=6)
+        seqs = []
+        for k, v in base:
+            s = pair.seq()
+            pair.append(s, k, v)
+            seqs.append(s)
+        seqs.append(pair.gpu.seq_fork(seqs[0]))
+        out = torch.zeros((1, cu[-1], hq, d), dtype=torch.bfloat16, device="cuda")
+        if whole:
+            pair.gpu.replay_rounds(seqs, [[1] * n] * rounds, cu, K, V, Q, out=out)
+        else:
+            for r in range(rounds):
+                idx = torch.tensor([c + r for c in cu[:-1]], device="cuda")
+                pair.gpu.append_kv_batch(seqs, K[:, idx].contiguous(), V[:, idx].contiguous(), list(range(n + 1)))
+                out[0, idx] = pair.gpu.replay_attn_batch(seqs, 0, Q[0, idx].contiguous(), list(range(n + 1)))
+        torch.cuda.synchronize()
+        assert pair.gpu.device_status() == 0
+        outs.append(out)
+        pools.append([(x, pair.gpu.page_table(s)) for s in seqs for x in [pair.gpu.seq_info(s)]])
+    assert torch.equal(outs[0], outs[1])
+    assert pools[0] == pools[1]
+    assert outs[0].float().abs().sum() > 0
