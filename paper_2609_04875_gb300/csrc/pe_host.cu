@@ -1377,11 +1377,11 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
             one_us = one_pass ? 0.97 * pass_us : 1.04 * plan_us;
         } else if (many) {
             sk_us = 13.0 + 1.5 * xw + 4.5 * waves;
-            one_us = one_pass ? 0.95 * pass_us : tail ? 0.0 : 0.9 * plan_us;
+            one_us = one_pass ? 0.95 * pass_us : (tail ? 0.985 : 0.9) * plan_us;
         } else {
             sk_us = 21.0 + 1.36 * xw + 8.0 * std::max(0.0, 1.0 / waves - 3.0);
             // (a unit of one q-tile among pairs is less work than the cost model counts)
-            one_us = plan_us * (0.90 - 0.15 * grp_lone / units) * (one_pass ? 0.9 : 1.0);
+            one_us = tail ? plan_us : plan_us * (0.90 - 0.15 * grp_lone / units) * (one_pass ? 0.9 : 1.0);
         }
         const bool sk_fits = 4 * grp_units >= c->num_sms && grp_units <= 16384 && !(all_lone && d != 64 && many);
         const bool sk_wins = sk_fits && !(one_pass && c->splitkv == 0) && sk_us <= one_us;
