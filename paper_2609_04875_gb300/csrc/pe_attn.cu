@@ -758,7 +758,7 @@ template <int HD, int kCombCols, int kCombBatch>
 __global__ void __launch_bounds__(256) splitkv_combine_kernel(const __grid_constant__ AttnParams p)
 {
     // launched with programmatic serialization after the attention grid: the item is found before the
-    // wait for its partials, and the next kernel may start its own set-up during the merge
+    // wait for its partials
     constexpr int kGroups = HD / kCombCols;  // column groups
     constexpr int kChunks = kCombCols / 4;   // 16-byte chunks of one
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -778,8 +778,9 @@ __global__ void __launch_bounds__(256) splitkv_combine_kernel(const __grid_const
     const int qi = qt * (kBM / g) + row / g;
     const int64_t base = sq.part_row0 + static_cast<int64_t>(unit) * sq.n_splits * kBM + row;
     const int ns = sq.n_splits;
-    ptx::griddep_wait();
+    // the next kernel's set-up from here on (32 layers of 133 tokens 407 -> 401 us against after the wait)
     ptx::griddep_launch_dependents();
+    ptx::griddep_wait();
     if (qi >= sq.n_q) return;
     float mx = -INFINITY, den = 0.f;
     float4 acc[kChunks];
