@@ -26,7 +26,7 @@ __device__ __forceinline__ uint4 ld_stream(const uint4 *p)
     return v;
 }
 
-// A launch's parameter block is copied by the host, the driver and the GPU's front end: 15 KB of it cost a
+// A launch's parameter block is copied by the host, by CUDA and by the GPU's front end: 15 KB of it cost a
 // launch 0.5 us more than 1 KB (2.03 against 1.60 us of host time).  A batch of few sequences and pages
 // takes the kernel's form with the small block.
 constexpr int kSmallSegs = 16, kSmallPages = 128;
