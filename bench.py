@@ -312,14 +312,14 @@ NCU_TRAFFIC = {
              "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f"}},
     "agent_batch": {"bytes": 685.47584e6 + 315.327744e6, "profile": "profiles/traffic_attention_configs.md",
                     "kernels": ["prefill"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f"}},
-    "short_suffix": {"bytes": 1.087881216e9 + 5.398016e6, "profile": "profiles/traffic_attention_configs.md",
-                     "kernels": ["prefill_sk"], "src_sha256": {"prefill_sk": "3818ae2364ef494941b6919759e1d90d82f93b7381afc5fd873033a9b55a4392"}},
+    "short_suffix": {"bytes": 1.08885632e9 + 5.18144e6, "profile": "profiles/traffic_attention_configs.md",
+                     "kernels": ["prefill_sk"], "src_sha256": {"prefill_sk": "d87018c7e548d16cb249d9d52d359f90916e3d8dd6982d6660c72bead3f55b6a"}},
     "long_suffix": {"bytes": 1.41151616e9 + 1.03740288e9, "profile": "profiles/traffic_attention_configs.md",
                     "kernels": ["prefill"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f"}},
     # one sweep step's 224 attention launches (5 forget requests x 32 layers, two launches per layer where a
     # tail launch runs), per layer: bytes / 160
-    "tau_sweep": {"bytes": (47813.435e6 + 7977.683e6) / 160, "profile": "profiles/traffic_attention_configs.md",
-                  "kernels": ["prefill", "prefill_sk"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f", "prefill_sk": "3818ae2364ef494941b6919759e1d90d82f93b7381afc5fd873033a9b55a4392"}},
+    "tau_sweep": {"bytes": (47659.393e6 + 8008.357e6) / 160, "profile": "profiles/traffic_attention_configs.md",
+                  "kernels": ["prefill", "prefill_sk"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f", "prefill_sk": "d87018c7e548d16cb249d9d52d359f90916e3d8dd6982d6660c72bead3f55b6a"}},
     "decode_batch": {"bytes": 341.534464e6 + 3.879168e6, "profile": "profiles/decode_tc_decode_batch.md",
                      "kernels": ["decode"],
                      "src_sha256": {"decode": "92c511c1911bfb21c61432aa9bdf4df8b5b389e7497f2625650667460bf98173"}},
