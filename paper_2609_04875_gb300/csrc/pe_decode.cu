@@ -443,7 +443,8 @@ __global__ void __launch_bounds__(kDecThreads, DecCfg<HD, RB>::kMinBlocks)
 // Tensor-core form (d = 128 and d = 64).  With keys on the M side of the MMA
 // the few query rows become N = 16 (rows padded):
 //     S^T [128 keys x 16] = K [128 x d] . Q^T          (A = K tile, B = Q; K-major)
-//     O^T [d x 16]       += V^T [d x 128 keys] . P^T   (A = V tile, MN-major; B = P^T, K-major)
+//     O^T [d x kPRows]   += V^T [d x 128 keys] . P^T   (A = V tile, MN-major; B = P^T, K-major, its weights
+//                                                       in two bf16 parts, a row each: TcCfg::kPRows)
 // both accumulated in TMEM (lane = key for S^T, lane = d-column for O^T), so a
 // softmax thread owns one key and touches only its RB valid row values per
 // 128-key tile.  For d = 64 the O^T GEMM keeps M = 128: the A operand's second
@@ -464,11 +465,11 @@ __global__ void __launch_bounds__(kDecThreads, DecCfg<HD, RB>::kMinBlocks)
 //
 // Roles (384 threads):
 //   warps 0-3  softmax: thread t = key t of the tile (TMEM lane t); masks,
-//              exp2 against a per-row reference, P^T (bf16) to shared memory,
+//              exp2 against a per-row reference, P^T (two bf16 parts) to shared memory,
 //              per-thread partial row sums; per chunk, the row statistics
 //              (m, l) for the epilogue.
-//   warps 7-10 epilogue: thread = d-column (TMEM lane); per chunk, reads O^T
-//              (double-buffered in TMEM, so the next chunk accumulates into
+//   warps 7-10 epilogue: thread = d-column (TMEM lane); per chunk, reads O^T, adds
+//              its two parts (double-buffered in TMEM, so the next chunk accumulates into
 //              the other buffer meanwhile), writes the output or the chunk's
 //              partial.
 //   warp 11    scheduler + page-id loader: takes chunk ids (one chunk ahead of
@@ -505,8 +506,19 @@ struct TcCfg {
     static constexpr int kLoadBytes = kTcKeys * HD * 2;     // bytes the TMA boxes of one tile deliver
     static constexpr int kOffV = kTcKStages * kTileBytes;   // K ring, then V ring
     static constexpr int kOffQ = (kTcKStages + kTcVStages) * kTileBytes;  // Q x2: [16 rows][128] bf16, 2 x 2 KB each
-    static constexpr int kOffP = kOffQ + 2 * 4096;          // P^T x2: [16 rows][128 keys] bf16, 2 regions x 2 KB each
-    static constexpr int kOffRed = kOffP + 2 * 4096;        // float [4 warps][16]
+    // P^T x2: [kPRows][128 keys] bf16, 2 regions of 64 keys each.  A weight is held as two bf16 parts, its
+    // upper 16 bits in row r and what they leave over in row kLo + r, both multiplied by the one MMA (for
+    // up to 8 rows in columns its N = 16 has anyway), so the weights carry 16 bits and only the output's
+    // rounding is left: the error against 64 bits is 1.7e-3 of the output whatever the chunk length.  (Rounded
+    // once, a chunk's largest weight of its first tile is exactly 1, so the error grew from 2.25e-3 with chunks
+    // of 2 tiles to 2.33e-3 with 8.)  It costs 1.2 % where a layer is a few tiles per SM (64 heads on 12k, 17.3 ->
+    // 17.5 us a layer), nothing at 16 agents (66.0 us), 3 % with 16 rows.
+    static constexpr int kPRows = RB <= 8 ? 16 : 32;
+    static constexpr int kLo = kPRows / 2;
+    static constexpr int kPRegion = kPRows * 128;
+    static constexpr int kPBytes = 2 * kPRegion;
+    static constexpr int kOffP = kOffQ + 2 * 4096;
+    static constexpr int kOffRed = kOffP + 2 * kPBytes;     // float [4 warps][16]
     static constexpr int kOffBar = kOffRed + 4 * 16 * 4;
     // k_full[KS], k_empty[KS], v_full[VS], v_empty[VS], s_full[2], p_full[2], o_done[2], q_ready[2], drain,
     // ch_full[R], ch_empty[R], o_item[2], o_free[2], stats[2], desc_full[D], desc_empty[D], q_free[2]
@@ -518,7 +530,8 @@ struct TcCfg {
     static constexpr int kOffDesc = kOffSeqs + kMaxSegs * static_cast<int>(sizeof(DecodeSeq) + 4);  // + rem_seq
     static constexpr int kSmem = kOffDesc + kDescRing * kDescInts * 4;
     static constexpr int kDynSmem = kSmem + 1024;
-    static constexpr uint32_t kTmemCols = 64;               // S^T buffers at 0 and 16, O^T buffers at 32 and 48
+    static constexpr uint32_t kTmemCols = RB <= 8 ? 64 : 128;  // S^T buffers at 0 and 16, O^T at 32 and 32 + kPRows
+    static_assert(32 + 2 * kPRows <= static_cast<int>(kTmemCols), "O^T buffers");
     static_assert(kDynSmem <= 232448, "shared memory budget");
     static_assert(RB == 4 || RB == 8 || RB == 16, "row capacity");
     static_assert(HD == 64 || HD == 128, "head dim");
@@ -665,8 +678,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         ptx::tmem_relinquish();
     }
     if (warp < 4) {
-        // both P^T buffers start at zero (rows past RB stay zero)
-        for (int e = threadIdx.x; e < 2 * 4096 / 16; e += 128)
+        // both P^T buffers start at zero (rows that hold neither part of a weight stay zero)
+        for (int e = threadIdx.x; e < 2 * C::kPBytes / 16; e += 128)
             reinterpret_cast<uint4 *>(smem + C::kOffP)[e] = make_uint4(0u, 0u, 0u, 0u);
         if (HD == 64) {  // the zero second half of every V stage (d-columns 64..127 of the O^T GEMM's A)
             for (int s = 0; s < kTcVStages; ++s)
@@ -693,7 +706,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     ptx::griddep_wait();
     const uint32_t tmem = *tmem_slot;
     const uint32_t t_s = tmem;         // S^T buffers: columns 0 and 16
-    const uint32_t t_o = tmem + 32;    // O^T buffers: columns 32..47 (even chunks) and 48..63 (odd)
+    const uint32_t t_o = tmem + 32;    // O^T buffers: kPRows columns each (even chunks, then odd)
 
     if (warp == 4 || warp == 6) {
         // ============================================================ producers (warp 4: K, warp 6: V)
@@ -844,7 +857,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         // ============================================================ MMA issuer (the whole warp, converged;
         // one elected lane issues.  Every decision is warp-uniform: probes and clocks go through a vote.)
         constexpr uint32_t kIdS = ptx::idesc_bf16_f32(128, 16, false, false);
-        constexpr uint32_t kIdPV = ptx::idesc_bf16_f32(128, 16, false, true);
+        constexpr uint32_t kIdPV = ptx::idesc_bf16_f32(128, C::kPRows, false, true);
         constexpr uint32_t kAll = 0xffffffffu;
         const uint32_t tm = __shfl_sync(kAll, tmem, 0);
         const uint64_t k_desc = ptx::smem_desc_sw128(sbase, 16, 1024);
@@ -918,11 +931,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 (p_done > 0 || np_chunk < 2 || ready(b_o_free + 8 * (np_chunk & 1), ((np_chunk - 2) >> 1) & 1))) {
                 ptx::tc_fence_after();
                 const uint64_t vd = v_desc + (np % kTcVStages) * (C::kTileBytes >> 4);
-                const uint64_t pd = p_desc + (np & 1) * (4096 >> 4);
+                const uint64_t pd = p_desc + (np & 1) * (C::kPBytes >> 4);
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
-                    mma_bf16_warp(tm + 32 + 16 * (np_chunk & 1), vd + (kk * 16 * 128 >> 4),
-                                  pd + (((kk >> 2) * 2048 + (kk & 3) * 32) >> 4), kIdPV,
+                    mma_bf16_warp(tm + 32 + C::kPRows * (np_chunk & 1), vd + (kk * 16 * 128 >> 4),
+                                  pd + (((kk >> 2) * C::kPRegion + (kk & 3) * 32) >> 4), kIdPV,
                                   (p_done > 0 || kk > 0) ? 1u : 0u);
                 mma_commit_warp(v_empty(np % kTcVStages));
                 mma_commit_warp(b_o_done + 8 * (np & 1));
@@ -1037,12 +1050,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         const bool done = wait_bar_warp(b_o_done + 8 * ((i - 1) & 1), ((i - 1) >> 1) & 1, wctx);
                         if (done) {
                             ptx::tc_fence_after();
-                            float o[RB];
-                            ptx::tmem_ld_n<RB>(t_o + 16 * (n & 1) + lane_off, o);
-                            ptx::tmem_wait_ld();
 #pragma unroll
-                            for (int r = 0; r < RB; ++r) o[r] *= f[r];
-                            ptx::tmem_st_n<RB>(t_o + 16 * (n & 1) + lane_off, o);
+                            for (int part = 0; part < 2; ++part) {
+                                const uint32_t to = t_o + C::kPRows * (n & 1) + part * C::kLo + lane_off;
+                                float o[RB];
+                                ptx::tmem_ld_n<RB>(to, o);
+                                ptx::tmem_wait_ld();
+#pragma unroll
+                                for (int r = 0; r < RB; ++r) o[r] *= f[r];
+                                ptx::tmem_st_n<RB>(to, o);
+                            }
                             ptx::tmem_wait_st();
                         }
                     }
@@ -1051,12 +1068,23 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 for (int r = 0; r < RB; ++r) lpart[r] += pr[r];
                 // P^T(i) into buffer i & 1 once O^T += V^T P^T(i - 2) has read it
                 if (i >= 2) (void)wait_bar_warp(b_o_done + 8 * (i & 1), ((i - 2) >> 1) & 1, wctx);
-                uint8_t *pt = smem + C::kOffP + (i & 1) * 4096 + (t >> 6) * 2048;
+                uint8_t *pt = smem + C::kOffP + (i & 1) * C::kPBytes + (t >> 6) * C::kPRegion;
                 const int chunk = (t & 63) >> 3;
+                // a weight's upper part is its upper 16 bits (cut, not rounded: no conversion), the rest rounds to the
+                // lower part, two rows a conversion
 #pragma unroll
-                for (int r = 0; r < RB; ++r)
-                    *reinterpret_cast<__nv_bfloat16 *>(pt + r * 128 + ((chunk ^ (r & 7)) << 4) + (t & 7) * 2) =
-                        __float2bfloat16_rn(pr[r]);
+                for (int r = 0; r < RB; r += 2) {
+                    const uint32_t w0 = __float_as_uint(pr[r]), w1 = __float_as_uint(pr[r + 1]);
+                    const uint32_t lo = pack_bf16(pr[r] - __uint_as_float(w0 & 0xffff0000u),
+                                                  pr[r + 1] - __uint_as_float(w1 & 0xffff0000u));
+                    // (row kLo + r has row r's place in its swizzle atom)
+                    uint8_t *d0 = pt + r * 128 + ((chunk ^ (r & 7)) << 4) + (t & 7) * 2;
+                    uint8_t *d1 = pt + (r + 1) * 128 + ((chunk ^ ((r + 1) & 7)) << 4) + (t & 7) * 2;
+                    *reinterpret_cast<uint16_t *>(d0) = static_cast<uint16_t>(w0 >> 16);
+                    *reinterpret_cast<uint16_t *>(d1) = static_cast<uint16_t>(w1 >> 16);
+                    *reinterpret_cast<uint16_t *>(d0 + C::kLo * 128) = static_cast<uint16_t>(lo);
+                    *reinterpret_cast<uint16_t *>(d1 + C::kLo * 128) = static_cast<uint16_t>(lo >> 16);
+                }
                 ptx::fence_proxy_async_smem();
                 ptx::tc_fence_before();
                 ptx::mbar_arrive(b_p_full + 8 * (i & 1));
@@ -1117,8 +1145,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             if (wait_bar_warp(b_o_item + 8 * (n & 1), (n >> 1) & 1, wctx)) {
                 ptx::tc_fence_after();
-                ptx::tmem_ld_n<RB>(t_o + 16 * (n & 1) + lane_off, o);
+                float o_lo[RB];
+                ptx::tmem_ld_n<RB>(t_o + C::kPRows * (n & 1) + lane_off, o);
+                ptx::tmem_ld_n<RB>(t_o + C::kPRows * (n & 1) + C::kLo + lane_off, o_lo);
                 ptx::tmem_wait_ld();
+#pragma unroll
+                for (int r = 0; r < RB; ++r) o[r] += o_lo[r];
             }
             ptx::tc_fence_before();
             ptx::mbar_arrive(b_o_free + 8 * (n & 1));  // O^T buffer and stats slot may be reused

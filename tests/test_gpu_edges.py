@@ -182,3 +182,34 @@ def test_rounds_equal_their_calls_one_by_one(keys):
     assert torch.equal(outs[0], outs[1])
     assert pools[0] == pools[1]
     assert outs[0].float().abs().sum() > 0
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("hq,hkv,nq", [(8, 8, 1), (32, 8, 1), (24, 3, 1), (32, 8, 3), (32, 4, 2)])
+@pytest.mark.parametrize("chunks_per_sm", [None, 1, 64])
+def test_decode_weights_carry_more_than_one_bf16(d, hq, hkv, nq, chunks_per_sm):
+    """1 to 16 rows per kv-head, chunks of 1 to 8 tiles: what is off is the output's rounding to bf16, at most 2^-9
+    of each value, whatever the chunk length.  The weights' 16 bits and the fp32 sums add less than 2^-18 of the
+    mean weighted |V|, some 50 |O| here and independent across keys: below 4e-5 of the output.  (Weights of
+    one bf16 alone put it at 2.2e-3 to 2.4e-3.)"""
+    lens = [9000, 4097, 1100, 300]
+    npg = sum(-(-n // 16) for n in lens) + 4
+    pair = Pair(1, hkv, d, 16, npg, len(lens), max(lens) // 16 + 2, seed=d + hq)
+    if chunks_per_sm is not None:
+        pair.gpu.set_option("decode_chunks_per_sm", chunks_per_sm)
+    g = synth.rng(d + hq + nq, 75)
+    seqs = []
+    for n in lens:
+        s = pair.seq()
+        pair.append(s, synth.normal_bf16(g, (1, n, hkv, d)), synth.normal_bf16(g, (1, n, hkv, d)))
+        seqs.append(s)
+    cu = [nq * i for i in range(len(lens) + 1)]
+    q = synth.normal_bf16(g, (cu[-1], hq, d))
+    out = pair.gpu.replay_attn_batch(seqs, 0, dev(q), cu)
+    torch.cuda.synchronize()
+    assert pair.gpu.device_status() == 0
+    for i, s in enumerate(seqs):
+        ref = oracle.replay_attention(pair.orc, s, 0, q[cu[i]:cu[i + 1]], 1 / math.sqrt(d))
+        got = out[cu[i]:cu[i + 1]].double().cpu().numpy()
+        err = np.linalg.norm(got - ref) / np.linalg.norm(ref)
+        assert err <= 2.0 ** -9 + 4e-5, (lens[i], err)
