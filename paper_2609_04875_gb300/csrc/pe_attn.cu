@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
                                                 o[4 * k + 3] * inv);
                         }
                     }
-                    if (valid) p.part_lse[prow] = l > 0.f ? m_ref + __log2f(l) : -INFINITY;
+                    if (valid) p.part_lse[prow] = l == 0.f ? -INFINITY : m_ref + __log2f(l);  // (l NaN: kept)
                 }
             }
         }
@@ -799,9 +799,13 @@ __global__ void __launch_bounds__(256) splitkv_combine_kernel(const __grid_const
                 v[u][k] = in ? __ldcg(part_chunk<HD>(p.part_o, r, cg * kChunks + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         float bmx = mx;
+        bool any = mx != -INFINITY;
 #pragma unroll
-        for (int u = 0; u < kCombBatch; ++u) bmx = fmaxf(bmx, lse[u]);
-        if (bmx == -INFINITY) continue;  // no visible key so far
+        for (int u = 0; u < kCombBatch; ++u) {
+            bmx = fmaxf(bmx, lse[u]);
+            any = any || lse[u] != -INFINITY;  // (a NaN, which fmaxf passes over, counts)
+        }
+        if (!any) continue;  // no visible key so far
         const float f = mx == -INFINITY ? 0.f : ex2(mx - bmx);
         den *= f;
 #pragma unroll

@@ -232,7 +232,7 @@ __device__ __noinline__ void merge_own_row(const SkParams &P, int slot, int t, i
     const AttnParams &p = P.a;
     constexpr int64_t kStride = 2 * kBM;
     const int64_t r0 = static_cast<int64_t>(slot) * P.max_parts * kStride + t * kBM + row;
-    const float lse_own = (has_tmem && l > 0.f) ? m_ref + __log2f(l) : -INFINITY;
+    const float lse_own = (!has_tmem || l == 0.f) ? -INFINITY : m_ref + __log2f(l);  // (as a written part)
     const float inv_own = l > 0.f ? 1.0f / l : 0.f;
     float lse[kMaxOwnMergeParts];
 #pragma unroll
@@ -842,7 +842,7 @@ __global__ void __launch_bounds__(kPrefillThreads, 1)
                                                 o[4 * q + 3] * inv);
                         }
                     }
-                    if (valid) p.part_lse[prow] = l > 0.f ? m_ref + __log2f(l) : -INFINITY;
+                    if (valid) p.part_lse[prow] = l == 0.f ? -INFINITY : m_ref + __log2f(l);  // (l NaN: kept)
                 }
                 // O_t has been read: the next piece's first P V GEMM may overwrite it
                 ptx::tc_fence_before();

@@ -213,3 +213,33 @@ def test_decode_weights_carry_more_than_one_bf16(d, hq, hkv, nq, chunks_per_sm):
         got = out[cu[i]:cu[i + 1]].double().cpu().numpy()
         err = np.linalg.norm(got - ref) / np.linalg.norm(ref)
         assert err <= 2.0 ** -9 + 4e-5, (lens[i], err)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("nq", [1, 40, 130])
+@pytest.mark.parametrize("options", [{}, {"attn_kernel": 0, "splitkv": 0}, {"attn_kernel": 0, "num_splits": 3, "splitkv": 1},
+                                     {"attn_kernel": 0, "num_splits": 20, "splitkv": 1}, {"attn_kernel": 2, "attn_ctas": 9},
+                                     {"attn_kernel": 2, "attn_ctas": 60}])
+@pytest.mark.parametrize("where", ["one", "most"])
+def test_a_nan_key_reaches_every_output_that_attends_it(d, nq, options, where):
+    """A NaN among one kv-head's keys makes that head's outputs NaN, whatever parts the keys are cut into: one
+    part with the NaN, or a NaN in each but the last (more such parts than a merge takes at once).  The other
+    heads are not touched."""
+    hq, hkv, n = 8, 2, 2600
+    pair = Pair(1, hkv, d, 16, n // 16 + 4, 1, n // 16 + 2, seed=d + nq)
+    for key, value in options.items():
+        pair.gpu.set_option(key, value)
+    g = synth.rng(d + nq, 76)
+    s = pair.seq()
+    k, v = (synth.normal_bf16(g, (1, n, hkv, d)) for _ in range(2))
+    q = synth.normal_bf16(g, (nq, hq, d))
+    pair.orc.append(s, k, v)
+    ref = oracle.replay_attention(pair.orc, s, 0, q, 1 / math.sqrt(d))
+    bad = k.copy()
+    bad[0, [5] if where == "one" else list(range(3, 2400, 128)), 1, 7] = 0x7FC0
+    pair.gpu.append_kv(s, dev(bad), dev(v))
+    out = pair.gpu.replay_attn(s, 0, dev(q))
+    torch.cuda.synchronize()
+    assert pair.gpu.device_status() == 0
+    assert_close(out[:, :4], ref[:, :4], f"{options}")
+    assert torch.isnan(out[:, 4:]).all(), (options, pair.gpu.last_attn_plan())
