@@ -244,7 +244,6 @@ class PagedKVCache:
             self._bf16 = torch.bfloat16
             self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
             self._cur_dev = getattr(torch._C, "_cuda_getDevice", None)
-        self._default_scale = 1.0 / math.sqrt(head_dim)
         self._pools = (k_pool, v_pool)  # keep caller tensors alive
         if k_pool is not None:
             cfg.k_pool = _dev_ptr(k_pool, "k_pool", self._device).value
@@ -257,6 +256,7 @@ class PagedKVCache:
         h = ctypes.c_void_p()
         _check(_lib.pe_cache_create(ctypes.byref(cfg), ctypes.byref(h)))
         self._h = h
+        self._default_scale = 1.0 / math.sqrt(head_dim)  # (after the library has refused any but 64 and 128)
 
     # -- lifetime ------------------------------------------------------------
     def close(self):

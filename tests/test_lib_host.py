@@ -186,6 +186,10 @@ def test_error_codes():
     with pytest.raises(binding.PEError) as e:
         pe.PagedKVCache(1, 1, 64, 16, 4, 2, 4, init_free_order=[0, 1, 1, 2], host_only=True)
     assert e.value.kind == "invalid"
+    for head_dim in (0, -64, 96):            # the library's refusal, whatever the value
+        with pytest.raises(binding.PEError) as e:
+            pe.PagedKVCache(1, 1, head_dim, 16, 4, 2, 4, host_only=True)
+        assert e.value.kind == "unsupported", head_dim
 
 
 def test_golden_fork_trace():
