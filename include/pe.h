@@ -260,7 +260,11 @@ pe_status pe_cache_pools(const pe_cache *cache, void **k_pool, void **v_pool);
  * whose n_q x (Hq/Hkv) query rows fit in 16 take a decode kernel -- 1:
  * tcgen05 with keys on the MMA's M side (d = 64 and 128), split items merged
  * by a combine launch; 2: CUDA cores, split-KV merged in-kernel; 0: no
- * decode kernel (the prefill kernel serves every call); "attn_kernel" = 1
+ * decode kernel (the prefill kernel serves every call);
+ * "decode_chunks_per_sm" = 0 (auto, default) or 1..64: how many chunks of
+ * 1..8 key tiles per SM the tcgen05 decode kernel cuts a launch's keys into --
+ * auto takes the chunk length with the earliest estimated finish;
+ * "attn_kernel" = 1
  * (default) / 2 / 0: the prefill kernel -- 1: the one-item kernel or the
  * persistent stream-K kernel, whichever plan's estimated time is smaller (the
  * persistent one from q-tile pairs x Hkv of a quarter of the SMs on, and with

@@ -127,7 +127,8 @@ struct pe_cache {
     CUtensorMap tm_k{}, tm_v{};    // tensor-core kernel: 64 x ps boxes
     CUtensorMap tm_kd{}, tm_vd{};  // decode kernel: 64 x min(ps, 64) boxes
     // options
-    int splitkv = -1, num_splits = 0, debug_poison = 0, decode_kernel = 1, dec_chunks_per_sm = 0;
+    int splitkv = -1, num_splits = 0, debug_poison = 0, decode_kernel = 1;
+    int dec_chunks_per_sm = 0;    // decode chunks per SM (0 = the length with the earliest estimated finish)
     int attn_kernel = 1;          // prefill kernel: 1 auto, 2 persistent stream-K, 0 one work item per CTA
     int attn_ctas = 0;            // persistent kernel's CTA count (0 = chosen by the planner)
     int attn_order = -1;          // one-item kernel's item order: -1 auto, 0 kv-heads fastest, 1 pairs fastest
@@ -2091,7 +2092,7 @@ pe_status pe_set_option(pe_cache *c, const char *key, int64_t value)
     } else if (!std::strcmp(key, "debug_poison")) {
         c->debug_poison = value ? 1 : 0;
     } else if (!std::strcmp(key, "decode_chunks_per_sm")) {
-        if (value < 1 || value > 64) return fail(PE_ERR_INVALID, "decode_chunks_per_sm must be 1..64");
+        if (value < 0 || value > 64) return fail(PE_ERR_INVALID, "decode_chunks_per_sm must be 0 (auto) or 1..64");
         c->dec_chunks_per_sm = static_cast<int>(value);
     } else if (!std::strcmp(key, "decode_kernel")) {
         if (value < 0 || value > 2) return fail(PE_ERR_INVALID, "decode_kernel must be 0, 1 or 2");

@@ -101,6 +101,24 @@ def test_decode_merges_of_one_and_many_chunks(d, hq, hkv, chunks_per_sm):
     _batch(d, hq, hkv, 16, [100, 128, 1025, 9000, 4097], [1] * 5, options, seed=d + hq)
 
 
+def test_decode_chunk_option_returns_to_its_default():
+    """"decode_chunks_per_sm" set and set back to 0: the plan and the bits of a cache that never had it set."""
+    hq, hkv, d, n = 32, 8, 128, 6000
+    g = synth.rng(3, 77)
+    k, v, q = (dev(synth.normal_bf16(g, (1, n, h, d))) for h in (hkv, hkv, hq))
+    got = []
+    for values in ([], [64], [64, 0]):
+        pair = Pair(1, hkv, d, 16, n // 16 + 4, 1, n // 16 + 2, seed=3)
+        s = pair.gpu.seq_create()
+        pair.gpu.append_kv(s, k, v)
+        for value in values:
+            pair.gpu.set_option("decode_chunks_per_sm", value)
+        out = pair.gpu.replay_attn(s, 0, q[0, :1].contiguous())
+        got.append((pair.gpu.last_attn_plan(), out))
+    assert got[2][0] == got[0][0] != got[1][0]
+    assert torch.equal(got[2][1], got[0][1])
+
+
 @pytest.mark.parametrize("n", [1, 16, 17, 40])
 def test_append_and_crop_around_the_small_parameter_blocks(n):
     """n sequences appended and cropped in one call each, the first append of 8 pages a sequence: 16 sequences

@@ -178,7 +178,8 @@ def test_error_codes():
     with pytest.raises(binding.PEError) as e:
         c.set_option("nonsense", 1)
     assert e.value.kind == "invalid"
-    for key, good, bad in (("attn_order", 1, 2), ("attn_kernel", 2, 3), ("splitkv", -1, 2)):
+    for key, good, bad in (("attn_order", 1, 2), ("attn_kernel", 2, 3), ("splitkv", -1, 2),
+                           ("decode_chunks_per_sm", 64, 65), ("decode_chunks_per_sm", 0, -1)):
         c.set_option(key, good)
         with pytest.raises(binding.PEError) as e:
             c.set_option(key, bad)
