@@ -899,8 +899,23 @@ struct SkBound {
     bool operator==(const SkBound &o) const { return u == o.u && t == o.t; }
 };
 
+// Bytes of one part of a cut unit in the workspace: 256 rows (two q-tiles) of fp32 O and a log-sum-exp.
+int64_t sk_part_bytes(int head_dim) { return 2 * kBM * (static_cast<int64_t>(head_dim) * 4 + 4); }
+
+// CTAs among which `units` units can be cut before the parts outgrow the workspace: k CTAs start in k - 1 places,
+// nearly all inside a unit, so min(units, k - 1) units have k - 1 parts beyond their first ones.
+int64_t sk_ctas_that_fit(const pe_cache *c, int64_t units)
+{
+    const int64_t parts = c->ws_bytes / sk_part_bytes(c->cfg.head_dim);
+    if (parts < 2) return 1;
+    return parts / 2 <= units ? parts / 2 + 1 : parts - units + 1;
+}
+
+// max_tries: CTA counts tried for a plan with cuts before it is given up (the parts do not fit the workspace);
+// *cuts_fit: cuts are in the plan, or off, or a plan of every CTA with them fitted and gained too little.
 pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, size_t hi, int32_t layer, void *out,
-                  int32_t hq, float scale, SkParams &P, std::vector<int32_t> *unit_tiles = nullptr)
+                  int32_t hq, float scale, SkParams &P, std::vector<int32_t> *unit_tiles = nullptr,
+                  int max_tries = INT32_MAX, bool *cuts_fit = nullptr)
 {
     const pe_cache_config &cf = c->cfg;
     const int hkv = cf.num_kv_heads, d = cf.head_dim, g = hq / hkv, bmq = kBM / g;
@@ -921,7 +936,14 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
     std::vector<double> wt;        // cost of one of its key tiles
     std::vector<double> cum{0.0};  // cost before each unit
     bool pairs = false;            // some unit has two q-tiles
-    for (size_t i = lo; i < hi; ++i) pairs = pairs || static_cast<int64_t>(order[i].n_q) * g > kBM;
+    int64_t n_units = 0;
+    for (size_t i = lo; i < hi; ++i) {
+        pairs = pairs || static_cast<int64_t>(order[i].n_q) * g > kBM;
+        n_units += ceil_div(static_cast<int64_t>(order[i].n_q) * g, 2 * kBM) * hkv;
+    }
+    n_all.reserve(n_units);
+    wt.reserve(n_units);
+    cum.reserve(n_units + 1);
     const double lone_cost = pairs ? sk_lone_cost(d) : 1.0;
     for (size_t i = lo; i < hi; ++i) {
         const AttnItem &it = order[i];
@@ -1010,6 +1032,7 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
     std::vector<int32_t> slot_of;
     std::vector<int32_t> cuts_in;  // interior boundaries per cut unit
     int32_t n_slots = 0, max_parts = 1;
+    const int64_t parts_that_fit = c->ws_bytes / sk_part_bytes(d);
     auto slots_for = [&](const std::vector<SkBound> &bb) {
         slot_of.assign(U, -1);
         cuts_in.clear();
@@ -1026,8 +1049,7 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
             cuts_in[slot_of[x.u]] += 1;
         }
         for (int32_t k = 0; k < n_slots; ++k) max_parts = std::max(max_parts, cuts_in[k] + 1);
-        const int64_t rows = static_cast<int64_t>(n_slots) * max_parts * 2 * kBM;
-        return n_slots <= kMaxSkCtas && max_parts <= 32 && rows * (static_cast<int64_t>(d) * 4 + 4) <= c->ws_bytes;
+        return n_slots <= kMaxSkCtas && max_parts <= 32 && static_cast<int64_t>(n_slots) * max_parts <= parts_that_fit;
     };
 
     // CTAs: one per SM, fewer when the work is small (about 3 cost units each at least)
@@ -1037,14 +1059,24 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
     Plan whole, cut;
     make(n_cta, false, whole);
     bool cuts = false;
+    if (cuts_fit) *cuts_fit = true;
     if (c->splitkv != 0) {
-        // fewer CTAs when a unit would be cut into more than 32 parts or the partials overflow the workspace
-        for (int32_t nc = n_cta; nc >= 2; nc = std::min(nc - 1, nc * 31 / std::max<int32_t>(max_parts, 32))) {
+        // fewer CTAs when a unit would be cut into more than 32 parts or the parts overflow the workspace (their
+        // number falls with the CTAs', so the next count is about the one that fits)
+        int32_t nc = n_cta;
+        int tries = 0;
+        while (nc >= 2) {
             make(nc, true, cut);
-            if (!slots_for(cut.b)) continue;
-            if (n_slots > 0 && (c->splitkv == 1 || busiest(cut) + 2.0 < 0.95 * busiest(whole))) cuts = true;
-            break;
+            if (slots_for(cut.b)) {
+                if (n_slots > 0 && (c->splitkv == 1 || busiest(cut) + 2.0 < 0.95 * busiest(whole))) cuts = true;
+                break;
+            }
+            if (++tries == max_tries) nc = 1;  // (cuts stays off)
+            const int64_t need = static_cast<int64_t>(n_slots) * max_parts;
+            nc = static_cast<int32_t>(std::min<int64_t>(
+                std::min(nc - 1, nc * 31 / std::max<int32_t>(max_parts, 32)), need > 0 ? nc * parts_that_fit / need : nc));
         }
+        if (cuts_fit) *cuts_fit = cuts || n_cta < 2 || nc == n_cta;
     }
     const Plan &pl = cuts ? cut : whole;
     if (!cuts) {
@@ -1359,7 +1391,11 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         const bool one_pass = !split && !tail, all_lone = grp_lone == grp_units;
         const bool many = grp_units >= 2 * static_cast<int64_t>(c->num_sms);
         const double x = grp_tiles / n_sm;                                                  // key tiles per SM
-        const double xw = all_lone ? x : x - (1.0 - sk_lone_cost(d)) * grp_lone_tiles / n_sm;  // as plan_sk weighs them
+        // the persistent plan's key tiles per CTA: of as many CTAs as the workspace holds the parts of cut units
+        // for, and as plan_sk weighs them
+        const double sk_share = n_sm / std::min<double>(n_sm, static_cast<double>(sk_ctas_that_fit(c, grp_units)));
+        const double xs = x * sk_share;
+        const double xw = all_lone ? xs : xs - (1.0 - sk_lone_cost(d)) * grp_lone_tiles / n_sm * sk_share;
         // One pass: its waves, the last one counted for most of what it lacks of a full
         // one (less where one sequence's heaviest-first items end it with the light ones).
         const double waves = units / n_sm;
@@ -1370,8 +1406,8 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         const double plan_us = (tail ? tp.est : plan_est) * 1e6;
         double sk_us, one_us;
         if (all_lone) {
-            sk_us = d == 64 ? 0.74 * x + (one_pass && waves > 0.8 ? 8.0 + 3.0 * waves : 17.0)
-                            : 1.37 * x + 21.0 + 8.0 * std::max(0.0, 1.0 / waves - 3.0);
+            sk_us = d == 64 ? 0.74 * xs + (one_pass && waves > 0.8 ? 8.0 + 3.0 * waves : 17.0)
+                            : 1.37 * xs + 21.0 + 8.0 * std::max(0.0, 1.0 / waves - 3.0);
             one_us = !one_pass ? 0.95 * plan_us : d == 64 ? 0.97 * pass_us : 0.77 * plan_us;
         } else if (d == 64) {
             sk_us = 13.0 + 1.05 * xw + 2.7 * waves;
@@ -1390,9 +1426,13 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         if (sk) {
             if (sbuf.empty()) sbuf.resize(sizeof(SkParams));
             SkParams &P = *reinterpret_cast<SkParams *>(sbuf.data());
-            if ((s = plan_sk(c, order, lo, hi, layer, out, hq, scale, P)) != PE_OK) return s;
-            // no unit cut (the workspace is too small for the parts): nothing gained over the one pass
-            if (c->attn_kernel == 1 && one_pass && d != 64 && !many && P.n_slots == 0) sk = false;
+            const bool forced = c->attn_kernel == 2;
+            bool cuts_fit = true;
+            s = plan_sk(c, order, lo, hi, layer, out, hq, scale, P, nullptr, forced ? INT32_MAX : 3, &cuts_fit);
+            if (s != PE_OK) return s;
+            // the estimate counts on the balance that cuts give: not without them where the workspace is too small
+            // for the parts, nor where nothing is gained over the one pass
+            if (!forced && (!cuts_fit || (one_pass && d != 64 && !many && P.n_slots == 0))) sk = false;
         }
         if (sk) {
             SkParams &P = *reinterpret_cast<SkParams *>(sbuf.data());

@@ -461,3 +461,40 @@ def test_persistent_launches_agree_with_the_persistent_plan():
         assert [q["seq"] for q in rec["seqs"]] == plan["order"]
         assert rec["ctas"] == plan["n_ctas"] and rec["split"] == (plan["n_slots"] > 0)
         c.close()
+
+
+def _auto_plan(hkv, d, lens, nqs, hq, ws, options=()):
+    c = pe.PagedKVCache(1, hkv, d, 16, 400000, len(lens), 4100, host_only=True, workspace_bytes=ws)
+    for key, value in options:
+        c.set_option(key, value)
+    seqs = []
+    for n in lens:
+        s = c.seq_create()
+        c.append_kv(s, n_tokens=n)
+        seqs.append(s)
+    return c, lambda: c.plan_launches(seqs, nqs, hq, num_sms=152)
+
+
+SMALL_WORKSPACE = [(8, 64, [8192] * 8, [20] * 8, 32, 1 << 20), (8, 128, [32784] * 8, [16] * 8, 64, 4 << 20),
+                   (8, 128, [16384], [1638], 32, 4 << 20), (8, 128, [12000] * 3, [400] * 3, 64, 1 << 20)]
+
+
+@pytest.mark.parametrize("hkv,d,lens,nqs,hq,ws", SMALL_WORKSPACE)
+def test_planning_with_a_small_workspace_costs_the_host_little(hkv, d, lens, nqs, hq, ws):
+    """A workspace that cannot hold the parts of cut units: planning costs the host little more than the one-item
+    plan (a persistent plan remade for one CTA count after another took 10 to 40 times as long; at most one is
+    made, 2 to 3 times, and 5 leaves room for a busy machine)."""
+    import time
+    c0, one = _auto_plan(hkv, d, lens, nqs, hq, ws, [("attn_kernel", 0)])
+    c1, auto = _auto_plan(hkv, d, lens, nqs, hq, ws)
+
+    def best(f):
+        times = []
+        for _ in range(30):
+            t0 = time.perf_counter()
+            f()
+            times.append(time.perf_counter() - t0)
+        return min(times)
+    assert best(auto) <= 5 * best(one)
+    c0.close()
+    c1.close()
