@@ -911,11 +911,10 @@ int64_t sk_ctas_that_fit(const pe_cache *c, int64_t units)
     return parts / 2 <= units ? parts / 2 + 1 : parts - units + 1;
 }
 
-// max_tries: CTA counts tried for a plan with cuts before it is given up (the parts do not fit the workspace);
-// *cuts_fit: cuts are in the plan, or off, or a plan of every CTA with them fitted and gained too little.
+// max_tries: CTA counts tried for a plan with cuts before it is given up (the parts do not fit the workspace).
 pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, size_t hi, int32_t layer, void *out,
                   int32_t hq, float scale, SkParams &P, std::vector<int32_t> *unit_tiles = nullptr,
-                  int max_tries = INT32_MAX, bool *cuts_fit = nullptr)
+                  int max_tries = INT32_MAX)
 {
     const pe_cache_config &cf = c->cfg;
     const int hkv = cf.num_kv_heads, d = cf.head_dim, g = hq / hkv, bmq = kBM / g;
@@ -1059,7 +1058,6 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
     Plan whole, cut;
     make(n_cta, false, whole);
     bool cuts = false;
-    if (cuts_fit) *cuts_fit = true;
     if (c->splitkv != 0) {
         // fewer CTAs when a unit would be cut into more than 32 parts or the parts overflow the workspace (their
         // number falls with the CTAs', so the next count is about the one that fits)
@@ -1076,7 +1074,6 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
             nc = static_cast<int32_t>(std::min<int64_t>(
                 std::min(nc - 1, nc * 31 / std::max<int32_t>(max_parts, 32)), need > 0 ? nc * parts_that_fit / need : nc));
         }
-        if (cuts_fit) *cuts_fit = cuts || n_cta < 2 || nc == n_cta;
     }
     const Plan &pl = cuts ? cut : whole;
     if (!cuts) {
@@ -1125,6 +1122,141 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
     }
     if (unit_tiles) *unit_tiles = n_all;
     return PE_OK;
+}
+
+// ---- estimated times of the prefill plans, in us; the plan with the smallest is launched
+// A CTA (the persistent kernel: a unit) costs a set-up and its key tiles.  It is a pair of q-tiles, a lone q-tile
+// in a launch that has pairs too, or one in a launch of lone q-tiles only (which has a kernel form of its own at
+// d = 128).  CTAs start in order, the heaviest first, so a launch lasts as long as its longest CTA, or as the SMs'
+// equal share with the last, partly filled wave's CTAs counted for the idle SMs beside them too; and never less
+// than reading K and V once takes.  Every term is continuous in the sizes but for the waves themselves.
+// The constants are least-squares fits (of the logarithm) to 37,700 launches: 1 to 64 sequences, equal and ragged, of 50
+// to 40k keys and 17 to 20k queries, 3 to 16 kv-heads, g = 1 to 8, d = 64 and 128, up to 900 key tiles per SM, each
+// timed in one pass, as the persistent kernel and with several splits.  The estimates are off by 4 to 10 % (standard
+// deviation; one pass least), and the plans they choose 0.9 % slower than the best of those timed (geometric mean,
+// with the margins that a second launch and the longer plan ask for; 0.6 % without).  Estimates in tile times with
+// a step wherever the kind of launch changed were 1.7 %, and 53 % at the worst (one sequence of 159 units: a tail launch
+// for 44.6 us where one pass takes 29.2).
+struct PrefillCosts {
+    double setup[3], tile[3];        // one-item kernel: pair, lone among pairs, all lone
+    double split_setup[2], split_tile[2];  // its CTAs with key splits: with pairs, all lone
+    double wave[2], uneven[2];       // of a piece: the last wave's idle SMs; a longest piece beyond the mean
+    double merge[2], merge_rate[2];  // the combine launch, and its partials' bytes per us (written and read)
+    double sk_setup[3], sk_tile[3];  // persistent kernel
+    double sk_whole, sk_cut, sk_part;  // its start and end without and with cut units, and per part of one
+};
+constexpr PrefillCosts kCosts64 = {{4.9, 4.3, 4.2}, {1.01, 0.85, 0.85}, {3.1, 3.8}, {1.065, 0.842}, {0.70, 0.75}, {0.35, 1.6},
+                                   {3.2, 1.9}, {8.3e6, 7.1e6}, {3.3, 3.3, 2.7}, {1.03, 0.82, 0.725}, 3.3, 8.4, 1.56};
+constexpr PrefillCosts kCosts128 = {{5.6, 5.2, 4.8}, {1.255, 1.21, 0.77}, {3.8, 5.25}, {1.34, 0.77}, {0.68, 0.66}, {0.26, 3.1},
+                                    {3.0, 0.9}, {8.15e6, 6.3e6}, {5.3, 3.0, 2.5}, {1.357, 1.5, 1.3}, 2.35, 11.5, 1.75};
+
+// K and V read once, after `start`: out of L2 (about 110 MB of it) at 9 TB/s, beyond at `rate` bytes per us.
+double kv_read_us(double bytes, double start, double rate)
+{
+    constexpr double kL2 = 110e6;
+    return start + std::min(bytes, kL2) / 9e6 + std::max(0.0, bytes - kL2) / rate;
+}
+
+// What the estimates need of a launch group; tables by kind (pair, lone among pairs, all lone).
+struct GroupShape {
+    double units = 0, tiles[3] = {0, 0, 0}, count[3] = {0, 0, 0};
+    double last_tiles[3] = {0, 0, 0}, last_count[3] = {0, 0, 0}, last = 0;  // of the last, partly filled wave
+    int64_t longest[3] = {0, 0, 0};                                          // key tiles of the longest unit
+    double kv_bytes = 0;
+    bool lone = false;  // all lone
+};
+
+// skip: the sequence's (one sequence only) lightest pairs that are not in the launch
+GroupShape group_shape(const pe_cache *c, const std::vector<AttnItem> &order, size_t lo, size_t hi, int g, int64_t skip)
+{
+    const int64_t hkv = c->cfg.num_kv_heads, bmq = kBM / g;
+    GroupShape s;
+    s.lone = true;
+    int64_t units = 0;
+    for (size_t i = lo; i < hi; ++i) {
+        const int64_t nqt = ceil_div(static_cast<int64_t>(order[i].n_q) * g, kBM);
+        s.lone = s.lone && nqt == 1;
+        units += (ceil_div(nqt, 2) - skip) * hkv;
+        s.kv_bytes += static_cast<double>(ceil_div(c->len[order[i].seq], kBN) * kBN * hkv * c->cfg.head_dim * 4);
+    }
+    s.units = static_cast<double>(units);
+    int64_t last = units % c->num_sms;
+    if (last == 0) last = std::min<int64_t>(units, c->num_sms);
+    s.last = static_cast<double>(last);
+    for (size_t i = hi; i-- > lo;) {  // from the last CTA in the launch's order
+        const AttnItem &it = order[i];
+        const int64_t nqt = ceil_div(static_cast<int64_t>(it.n_q) * g, kBM);
+        for (int64_t pp = skip; pp < ceil_div(nqt, 2); ++pp) {
+            const int64_t q_last = std::min<int64_t>((std::min(2 * pp + 1, nqt - 1) + 1) * bmq, it.n_q) - 1;
+            const int64_t n = ceil_div(c->len[it.seq] - it.n_q + q_last + 1, kBN);
+            const int k = 2 * pp + 1 < nqt ? 0 : (s.lone ? 2 : 1);
+            s.tiles[k] += static_cast<double>(n * hkv);
+            s.count[k] += static_cast<double>(hkv);
+            s.longest[k] = std::max(s.longest[k], n);
+            const int64_t l = std::min(last, hkv);
+            s.last_tiles[k] += static_cast<double>(n * l);
+            s.last_count[k] += static_cast<double>(l);
+            last -= l;
+        }
+    }
+    return s;
+}
+
+// Sum of the units' costs, and how long they take on the SMs.
+double shape_sum(const GroupShape &s, const double (&setup)[3], const double (&tile)[3])
+{
+    double S = 0;
+    for (int k = 0; k < 3; ++k) S += setup[k] * s.count[k] + tile[k] * s.tiles[k];
+    return S;
+}
+
+double shape_span(const GroupShape &s, const double (&setup)[3], const double (&tile)[3], double n_sm)
+{
+    double last = 0, longest = 0;
+    for (int k = 0; k < 3; ++k) {
+        last += setup[k] * s.last_count[k] + tile[k] * s.last_tiles[k];
+        if (s.count[k] > 0) longest = std::max(longest, setup[k] + tile[k] * static_cast<double>(s.longest[k]));
+    }
+    return std::max(longest, (shape_sum(s, setup, tile) - last) / n_sm + last / std::max(1.0, s.last));
+}
+
+double one_pass_us(const PrefillCosts &t, const GroupShape &s, double n_sm)
+{
+    return std::max(shape_span(s, t.setup, t.tile, n_sm), kv_read_us(s.kv_bytes, 5.0, 5.6e6));
+}
+
+// The combine launch of `rows` partial rows (of one split) in ns splits.
+double merge_us(const PrefillCosts &t, bool lone, int head_dim, int64_t rows, int64_t ns)
+{
+    const double bytes = 2.0 * static_cast<double>(rows * ns) * (head_dim * 4 + 4);
+    return t.merge[lone] + 0.43 * static_cast<double>(ceil_div(ns, 8)) + bytes / t.merge_rate[lone];
+}
+
+// `pieces` CTAs of at most split_tiles key tiles each, `tiles` in all, in ns splits, and their merge.
+double split_us(const PrefillCosts &t, const GroupShape &s, double n_sm, double pieces, int64_t split_tiles, int64_t ns,
+                int64_t rows, int head_dim)
+{
+    const double one = t.split_setup[s.lone] + t.split_tile[s.lone] * static_cast<double>(split_tiles);
+    double span = one;
+    if (pieces > n_sm) {
+        const double S = t.split_setup[s.lone] * pieces + t.split_tile[s.lone] * (s.tiles[0] + s.tiles[1] + s.tiles[2]);
+        const double r = pieces - n_sm * (std::ceil(pieces / n_sm) - 1.0);  // CTAs of the last wave
+        span = std::max(one, S / n_sm + t.wave[s.lone] * one * (1.0 - r / n_sm) +
+                                 t.uneven[s.lone] * std::max(0.0, one - S / pieces));
+    }
+    return std::max(span, kv_read_us(s.kv_bytes, 2.6, 5.0e6)) + merge_us(t, s.lone, head_dim, rows, ns);
+}
+
+// The persistent kernel with whole units, and with the work cut equally over n_cta CTAs.
+double sk_whole_us(const PrefillCosts &t, const GroupShape &s, double n_sm)
+{
+    return std::max(t.sk_whole + shape_span(s, t.sk_setup, t.sk_tile, n_sm), kv_read_us(s.kv_bytes, 6.5, 6.2e6));
+}
+
+double sk_cut_us(const PrefillCosts &t, const GroupShape &s, double n_cta)
+{
+    return std::max(t.sk_cut + shape_sum(s, t.sk_setup, t.sk_tile) / n_cta + t.sk_part * n_cta / s.units,
+                    kv_read_us(s.kv_bytes, 6.5, 6.2e6));
 }
 
 // Plan query (pe_attn_plan_launches): one launch as words -- kind, split,
@@ -1195,68 +1327,52 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
     if (!rec && (s = encode_q(&tm_q, Q, q_rows, hq, d, g)) != PE_OK) return s;
     if (!rec && (s = encode_q(&tm_o, out, q_rows, hq, d, g)) != PE_OK) return s;
 
-    // split-KV decision over the whole launch group; plan_est: the cost model's time of the plan
-    double plan_est = 0.0;
-    // the group's units (pairs of q-tiles x kv-heads) and their key tiles, and those of units of one q-tile
-    int64_t grp_units = 0, grp_tiles = 0, grp_lone = 0, grp_lone_tiles = 0;
-    // time of one key tile per CTA in the cost models: about 1.5 us, compute- or HBM-bound alike; 1 us at
-    // d = 64, whose next S GEMM overlaps the softmax
-    const double tile_s = d == 64 ? 1.0e-6 : 1.5e-6;
+    const PrefillCosts &costs = d == 64 ? kCosts64 : kCosts128;
+    const double n_sm = c->num_sms;
+    // split-KV decision over the whole launch group; shape: the group's, plan_us: the chosen plan's estimated time
+    GroupShape shape;
+    double plan_us = 0.0;
     // splitkv: the "splitkv" option's value for this plan (-1 auto, 0 never, 1 always)
     auto plan_group = [&](size_t lo, size_t hi, AttnParams &p, bool &split, int splitkv) -> pe_status {
-        // C CTAs (pairs of q-tiles x kv-heads), W key tiles per CTA on average.
-        int64_t C = 0, tiles = 0, lone_tiles = 0, rows = 0, valid_rows = 0, max_tiles = 0;
+        shape = group_shape(c, order, lo, hi, g, 0);
+        int64_t rows = 0, valid_rows = 0, max_tiles = 0;
         for (size_t i = lo; i < hi; ++i) {
-            const AttnItem &it = order[i];
-            const int64_t len = c->len[it.seq];
-            const int64_t nqt = ceil_div(static_cast<int64_t>(it.n_q) * g, kBM);
-            for (int64_t pp = 0; pp < ceil_div(nqt, 2); ++pp) {
-                const int64_t q_last = std::min<int64_t>((std::min(2 * pp + 1, nqt - 1) + 1) * bmq, it.n_q) - 1;
-                const int64_t n = ceil_div(len - it.n_q + q_last + 1, kBN) * hkv;
-                tiles += n;
-                if (2 * pp + 1 >= nqt) lone_tiles += n;
-            }
-            C += ceil_div(nqt, 2) * hkv;
-            rows += nqt * hkv * kBM;                               // workspace slots (whole tiles)
-            valid_rows += static_cast<int64_t>(it.n_q) * g * hkv;  // partial rows written and read
-            max_tiles = std::max(max_tiles, ceil_div(len, kBN));
+            rows += ceil_div(static_cast<int64_t>(order[i].n_q) * g, kBM) * hkv * kBM;  // workspace slots (whole tiles)
+            valid_rows += static_cast<int64_t>(order[i].n_q) * g * hkv;                 // partial rows written and read
+            max_tiles = std::max(max_tiles, ceil_div(c->len[order[i].seq], kBN));
         }
-        // Estimated time with s key splits: the CTAs run in ceil(C s / N) waves of
-        // (W/s + 2) tile times, and never faster than the longest CTA
-        // (max_tiles/s + 2); splits add a combine launch: 2.5 us, 1 us per batch of 8 splits, and the round
-        // trip of their fp32 partials, twice as fast while they are few (measured at d = 64, 64 CTAs of 12
-        // tiles: one pass 17.9 us, 2 splits 14.8; 32 CTAs of 11: 16.5, 4 splits 11.9).
-        const double W = C > 0 ? static_cast<double>(tiles) / C : 0.0;
+        const int64_t C = static_cast<int64_t>(shape.units);
         const int64_t row_bytes = static_cast<int64_t>(d) * 4 + 4;
         auto cost = [&](int64_t sp) {
-            const double waves = std::ceil(static_cast<double>(C * sp) / c->num_sms);
-            double t = std::max(waves * (W / sp + 2.0), static_cast<double>(max_tiles) / sp + 2.0) * tile_s;
-            if (sp > 1) {
-                const double bytes = static_cast<double>(valid_rows * sp * row_bytes);
-                t += bytes * 2.0 / (bytes < 20e6 ? 12.0e12 : 6.0e12) + 2.5e-6 + 1e-6 * static_cast<double>(ceil_div(sp, 8));
-            }
-            return t;
+            if (sp == 1) return one_pass_us(costs, shape, n_sm);
+            const int64_t st = ceil_div(max_tiles, sp);
+            double pieces = 0;
+            for (size_t i = lo; i < hi; ++i)
+                pieces += static_cast<double>(ceil_div(static_cast<int64_t>(order[i].n_q) * g, 2 * kBM) * hkv *
+                                              ceil_div(ceil_div(c->len[order[i].seq], kBN), st));
+            return split_us(costs, shape, n_sm, pieces, st, ceil_div(max_tiles, st), valid_rows, d);
         };
         int64_t best = 1;
+        plan_us = cost(1);
         if (splitkv != 0) {
-            // at least 4 key tiles per split, unless the CTAs are too few to fill the SMs
+            // at least 4 key tiles per split, unless the CTAs are too few to fill the SMs; at most four waves
             int64_t s_max = std::min<int64_t>(128, std::max<int64_t>(1, max_tiles / 4));
             if (C > 0 && C * 2 <= c->num_sms) s_max = std::max(s_max, std::min<int64_t>(max_tiles, c->num_sms / C));
-            double best_t = splitkv == 1 ? 1e30 : cost(1);
+            if (C > 0) s_max = std::min(s_max, std::max<int64_t>(2, 4 * c->num_sms / C));
+            double best_t = 1e30;
             for (int64_t sp = 2; sp <= s_max; ++sp) {
                 if (rows * sp * row_bytes > c->ws_bytes) break;
                 const double t = cost(sp);
                 if (t < best_t) { best_t = t; best = sp; }
             }
-            // keep the single pass unless clearly faster, by more than a launch costs the host
-            if (splitkv == -1 && best > 1 && best_t > std::min(0.95 * cost(1), cost(1) - 1.0e-6)) best = 1;
+            // keep the single pass unless clearly faster; by more where a pass is short, for a second launch costs
+            // the host about 2 us, which the GPU's time no longer hides (8 CTAs of 5 key tiles, d = 64: one pass 10 us
+            // by estimate, 5 splits 8, and the request is no faster; 2 sequences of 1.4k keys, 16.0 and 14.9: slower)
+            const double gain = std::max(0.02 * plan_us, 0.5 + 1.5 * std::min(1.0, std::max(0.0, (24.0 - plan_us) / 8.0)));
+            if (splitkv == -1 && best > 1 && best_t > plan_us - gain) best = 1;
+            if (best > 1) plan_us = best_t;
         }
         if (splitkv != 0 && c->num_splits > 0) best = c->num_splits;
-        plan_est = cost(best);
-        grp_units = C;
-        grp_tiles = tiles;
-        grp_lone_tiles = lone_tiles;
-        grp_lone = 2 * C - rows / kBM;
         int split_tiles = static_cast<int>(max_tiles);
         split = best > 1 || splitkv == 1;
         if (split) split_tiles = static_cast<int>(std::max<int64_t>(1, ceil_div(max_tiles, std::max<int64_t>(best, 1))));
@@ -1325,10 +1441,10 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
     // Tail launch for a launch group of one sequence (one long agent): when its CTAs leave the last
     // wave mostly empty, the lightest q-tile pairs (the last CTAs in the heaviest-first order) move
     // to a second launch that splits their keys over every SM; the first launch then fills whole
-    // waves.  Chosen by the same cost model, when it beats the group's plan by 5 %.
+    // waves.  Chosen when its estimate beats the group's plan by 3 %.
     struct TailPlan {
         int64_t pairs = 0, splits = 0, split_tiles = 0, qtiles = 0;
-        double est = 0.0;  // estimated time of both launches
+        double est = 0.0;  // estimated time of both launches (us)
     };
     auto plan_tail = [&](const AttnItem &it, TailPlan &tp) -> bool {
         const int64_t len = c->len[it.seq];
@@ -1339,29 +1455,33 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         const int64_t cut = ceil_div(C % N, hkv);  // lightest pairs moved to the tail launch
         if (cut >= n_pairs) return false;
         const int64_t ktiles = ceil_div(len, kBN);
-        double wa = 0.0, wb = 0.0;  // mean key tiles of a pair in the first / tail launch
-        for (int64_t pp = 0; pp < n_pairs; ++pp) {
-            const int64_t q_last = std::min<int64_t>((std::min(2 * pp + 1, nqt - 1) + 1) * bmq, it.n_q) - 1;
-            const double t = static_cast<double>(ceil_div(len - it.n_q + q_last + 1, kBN));
-            (pp < cut ? wb : wa) += t;
-        }
-        wa /= static_cast<double>(n_pairs - cut);
-        wb /= static_cast<double>(cut);
         const int64_t qt_b = std::min<int64_t>(nqt, 2 * cut);
         const int64_t row_bytes = static_cast<int64_t>(d) * 4 + 4;
-        const double t_a = std::ceil(static_cast<double>(C - cut * hkv) / N) * (wa + 2.0) * tile_s;
+        const size_t at = static_cast<size_t>(&it - order.data());
+        const GroupShape first = group_shape(c, order, at, at + 1, g, cut);
+        double wb = 0.0;  // mean key tiles of a unit of the tail launch
+        for (int k = 0; k < 3; ++k) wb += shape.tiles[k] - first.tiles[k];
+        wb /= static_cast<double>(cut * hkv);
+        // (3 us more than a split launch: the tail's start behind the first launch's last CTAs)
+        const double t_a = shape_span(first, costs.setup, costs.tile, n_sm) + 3.0;
         double best_t = 1e30;
         for (int64_t sp = 2; sp <= std::min<int64_t>(128, std::max<int64_t>(2, ktiles / 4)); ++sp) {
             if (qt_b * hkv * sp * kBM * row_bytes > c->ws_bytes) break;
-            const double waves = std::ceil(static_cast<double>(cut * hkv * sp) / N);
-            const double t = t_a + waves * (wb / sp + 2.0) * tile_s +
-                             static_cast<double>(qt_b * hkv * kBM * sp * row_bytes * 2) / 6.0e12 + 10e-6;
+            const double waves = std::ceil(static_cast<double>(cut * hkv * sp) / n_sm);
+            const double piece = std::min(wb, static_cast<double>(ceil_div(ktiles, sp)));
+            const double t = t_a + waves * (costs.split_setup[0] + costs.tile[0] * piece) +
+                             merge_us(costs, false, d, qt_b * hkv * kBM, sp);
             if (t < best_t) {
                 best_t = t;
                 tp.splits = sp;
             }
         }
-        if (tp.splits == 0 || best_t > 0.95 * plan_est) return false;
+        // with the one-item kernel pinned the group's plan counts in whole waves: where they leave SMs idle for long
+        // the persistent kernel would be taken, and is not to be had
+        const double whole_waves = c->attn_kernel == 0 ? std::ceil(shape.units / n_sm) * shape_sum(shape, costs.setup, costs.tile) /
+                                                             shape.units
+                                                       : 0.0;
+        if (tp.splits == 0 || best_t > 0.97 * std::max(plan_us, whole_waves)) return false;
         tp.est = best_t;
         tp.pairs = cut;
         tp.qtiles = qt_b;
@@ -1378,61 +1498,32 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         if (s != PE_OK) return s;
         TailPlan tp;
         const bool tail = hi - lo == 1 && c->splitkv == -1 && c->num_splits == 0 && plan_tail(order[lo], tp);
-        // The persistent stream-K kernel where it should beat the one-item plan.  One CTA per SM takes an equal
+        // The persistent stream-K kernel where its estimate is smaller.  One CTA per SM takes an equal
         // stretch of key tiles and goes from unit to unit without a gap; its longer start and end (the parts
-        // of cut units are merged by single warps, about 2 us a part) pay where the one-item plan leaves SMs
+        // of cut units are merged by single warps, about 1.6 us a part) pay where the one-item plan leaves SMs
         // idle for long, and at d = 64, where the gaps between CTAs weigh more.  Measured, one-item / persistent
-        // us a layer, d = 128: 64 units of one q-tile 20 / 27 at 7 key tiles per SM, 50 / 57 at 27, 172 / 169 at
-        // 108; 64 pairs 34 / 41 at 13, 178 / 166 at 107; 168 pairs 143 / 120 at 70; 312 pairs 254 / 203 at 129; 5016
-        // pairs (the 16-agent batch) 1670 / 1805.  d = 64: 64 units of one q-tile 22 / 26 at 13, 115 / 95 at 108;
-        // 64 pairs 26 / 29 at 13, 136 / 129 at 108; 168 pairs 109 / 90 at 70; 768 pairs 136 / 118 at 81; 1584 pairs
-        // 355 / 343 at 286; 1440 pairs 877 / 883 at 796.
-        const double n_sm = c->num_sms, units = static_cast<double>(std::max<int64_t>(grp_units, 1));
-        const bool one_pass = !split && !tail, all_lone = grp_lone == grp_units;
-        const bool many = grp_units >= 2 * static_cast<int64_t>(c->num_sms);
-        const double x = grp_tiles / n_sm;                                                  // key tiles per SM
-        // the persistent plan's key tiles per CTA: of as many CTAs as the workspace holds the parts of cut units
-        // for, and as plan_sk weighs them
-        const double sk_share = n_sm / std::min<double>(n_sm, static_cast<double>(sk_ctas_that_fit(c, grp_units)));
-        const double xs = x * sk_share;
-        const double xw = all_lone ? xs : xs - (1.0 - sk_lone_cost(d)) * grp_lone_tiles / n_sm * sk_share;
-        // One pass: its waves, the last one counted for most of what it lacks of a full
-        // one (less where one sequence's heaviest-first items end it with the light ones).
-        const double waves = units / n_sm;
-        const double wave_us = d == 128 ? 1.38 * x / waves + 6.0
-                                        : (all_lone ? 0.87 * x / waves + 6.5 : 1.05 * x / waves + 5.0);
-        const double last = waves <= 1.0 ? 1.0 : (hi - lo == 1 && waves > 3.0 ? 0.4 : 0.8);
-        const double pass_us = wave_us * (waves + last * (std::ceil(waves) - waves));
-        const double plan_us = (tail ? tp.est : plan_est) * 1e6;
-        double sk_us, one_us;
-        if (all_lone) {
-            sk_us = d == 64 ? 0.74 * xs + (one_pass && waves > 0.8 ? 8.0 + 3.0 * waves : 17.0)
-                            : 1.37 * xs + 21.0 + 8.0 * std::max(0.0, 1.0 / waves - 3.0);
-            one_us = !one_pass ? 0.95 * plan_us : d == 64 ? 0.97 * pass_us : 0.77 * plan_us;
-        } else if (d == 64) {
-            sk_us = 13.0 + 1.05 * xw + 2.7 * waves;
-            one_us = one_pass ? 0.97 * pass_us : 1.04 * plan_us;
-        } else if (many) {
-            sk_us = 13.0 + 1.5 * xw + 4.5 * waves;
-            one_us = one_pass ? 0.95 * pass_us : (tail ? 0.985 : 0.9) * plan_us;
-        } else {
-            sk_us = 21.0 + 1.36 * xw + 8.0 * std::max(0.0, 1.0 / waves - 3.0);
-            // (a unit of one q-tile among pairs is less work than the cost model counts)
-            one_us = tail ? plan_us : plan_us * (0.90 - 0.15 * grp_lone / units) * (one_pass ? 0.9 : 1.0);
-        }
-        const bool sk_fits = 4 * grp_units >= c->num_sms && grp_units <= 16384 && !(all_lone && d != 64 && many);
-        const bool sk_wins = sk_fits && !(one_pass && c->splitkv == 0) && sk_us <= one_us;
+        // us a layer, d = 128: 64 units of one q-tile 20 / 27 at 7 key tiles per SM, 172 / 169 at 108; 64 pairs 34 /
+        // 41 at 13, 178 / 166 at 107; 168 pairs 143 / 120 at 70; 312 pairs 254 / 203 at 129; 5016 pairs (the 16-agent
+        // batch) 1670 / 1805.  d = 64: 64 units of one q-tile 22 / 26 at 13, 115 / 95 at 108; 168 pairs 109 / 90 at 70;
+        // 768 pairs 136 / 118 at 81; 1584 pairs 355 / 343 at 286; 1440 pairs 877 / 883 at 796.
+        const bool one_pass = !split && !tail;
+        const double one_us = tail ? tp.est : plan_us;
+        const int64_t units = static_cast<int64_t>(shape.units);
+        const int64_t cut_ctas = std::min<int64_t>(c->num_sms, sk_ctas_that_fit(c, units));
+        const double whole_us = sk_whole_us(costs, shape, n_sm), cut_us = sk_cut_us(costs, shape, static_cast<double>(cut_ctas));
+        const bool sk_fits = 4 * units >= c->num_sms && units <= 16384 && !(one_pass && c->splitkv == 0);
+        // (2 % and half a microsecond for the host, whose plan takes some 5 us longer)
+        const double sk_limit = std::min(0.98 * one_us, one_us - 0.5);
+        const bool sk_wins = sk_fits && std::min(whole_us, cut_us) <= sk_limit;
         bool sk = c->num_splits == 0 && (c->attn_kernel == 2 || (c->attn_kernel == 1 && sk_wins));
         if (sk) {
             if (sbuf.empty()) sbuf.resize(sizeof(SkParams));
             SkParams &P = *reinterpret_cast<SkParams *>(sbuf.data());
             const bool forced = c->attn_kernel == 2;
-            bool cuts_fit = true;
-            s = plan_sk(c, order, lo, hi, layer, out, hq, scale, P, nullptr, forced ? INT32_MAX : 3, &cuts_fit);
+            s = plan_sk(c, order, lo, hi, layer, out, hq, scale, P, nullptr, forced ? INT32_MAX : 3);
             if (s != PE_OK) return s;
-            // the estimate counts on the balance that cuts give: not without them where the workspace is too small
-            // for the parts, nor where nothing is gained over the one pass
-            if (!forced && (!cuts_fit || (one_pass && d != 64 && !many && P.n_slots == 0))) sk = false;
+            // no unit cut (nothing to gain, or the workspace is too small for the parts): whole units have to win
+            if (!forced && P.n_slots == 0 && whole_us > sk_limit) sk = false;
         }
         if (sk) {
             SkParams &P = *reinterpret_cast<SkParams *>(sbuf.data());

@@ -498,3 +498,67 @@ def test_planning_with_a_small_workspace_costs_the_host_little(hkv, d, lens, nqs
     assert best(auto) <= 5 * best(one)
     c0.close()
     c1.close()
+
+
+def test_uncut_persistent_plans_only_where_whole_units_win():
+    """Over random groups and workspaces: a default plan that is persistent without cuts is so because whole units
+    beat the one-item plan (then they do with a workspace that holds every cut too, or cuts do), never because of
+    cuts that the workspace does not hold: the choice with no workspace to speak of is then the same."""
+    rng = random.Random(77)
+    uncut = cut = 0
+    for _ in range(1200):
+        d, hkv, g = rng.choice([64, 128]), rng.choice([4, 8]), rng.choice([1, 4, 8])
+        n = rng.choice([1, 3, 8, 20, 40])
+        t = int(10 ** rng.uniform(2.6, 4.4))
+        lens = [rng.randint(t, 2 * t) for _ in range(n)]
+        nqs = [min(x, rng.randint(17, rng.choice([64, 2000]))) for x in lens]
+        kinds = []
+        for ws in (1 << 12, int(10 ** rng.uniform(5.0, 7.7)), 1 << 30):
+            c, auto = _auto_plan(hkv, d, lens, nqs, hkv * g, ws)
+            kinds.append([(x["kind"], x["split"]) for x in auto()])
+            c.close()
+        none, some, full = kinds
+        cut += some == [("persistent", True)]
+        if some == [("persistent", False)]:
+            uncut += 1
+            # whole units win over the pass by themselves, and with every cut to be had the kernel is the same
+            assert none == some and full[0][0] == "persistent", (d, hkv, g, lens, nqs, kinds)
+    assert uncut > 20 and cut > 20, (uncut, cut)
+
+
+@pytest.mark.parametrize("hq,hkv,d,n,keys,nq,kind", [
+    (24, 3, 128, 1, 2170, 1666, "one_item"),      # one pass 29.2 us, tail launch 44.6, persistent 35.0
+    (16, 4, 128, 1, 2778, 2656, "one_item"),      # 40.2, 55.3, 44.1
+    (16, 4, 128, 1, 8474, 8236, "one_item"),      # 175, 201, 184
+    (32, 8, 64, 1, 4231, 3651, "persistent"),     # 82.4, 91.9, 79.7
+    (8, 8, 64, 1, 13278, 11204, "persistent"),    # 178, 186, 161
+    (16, 16, 64, 19, 719, 34, "persistent"),      # one pass 19.1 us, persistent 15.4
+    (16, 16, 64, 14, 2262, 76, "persistent"),     # 39.9 (2 splits 41.4), 33.3
+    (16, 16, 64, 5, 4350, 20, "persistent"),      # 33.4 (5 splits 30.3), 24.2
+    (16, 16, 128, 1, 8181, 16, "decode"),
+])
+def test_plans_that_were_measured(hq, hkv, d, n, keys, nq, kind):
+    """Launches whose plans differ by 10 to 50 % in time (measured; in us) take the fastest, in one launch."""
+    c, auto = _auto_plan(hkv, d, [keys] * n, [nq] * n, hq, 0)
+    plan = auto()
+    assert [x["kind"] for x in plan] == [kind]
+    assert kind != "one_item" or not plan[0]["split"]
+    c.close()
+
+
+def test_plan_choice_does_not_flicker():
+    """Keys swept in steps of 4 % across the edges of every regime (waves of CTAs, lone q-tiles and pairs, short and
+    long): a kind of plan that gives way to another does not come back in the next step, nearly everywhere."""
+    for d, hkv, g, n in [(64, 8, 4, 1), (64, 16, 1, 7), (128, 8, 4, 1), (128, 8, 4, 5), (128, 16, 1, 9), (64, 8, 8, 20)]:
+        for nq in (20, 128, 700, 3000):
+            back = steps = 0
+            before, prev, keys = None, None, float(nq + 150)
+            while keys < 24000:
+                c, auto = _auto_plan(hkv, d, [int(keys)] * n, [nq] * n, hkv * g, 0)
+                kind = [x["kind"] for x in auto()][-1]
+                c.close()
+                back += before == kind != prev
+                before, prev = prev, kind
+                keys *= 1.04
+                steps += 1
+            assert back <= steps // 20, (d, hkv, g, n, nq, back, steps)
