@@ -329,8 +329,8 @@ CSRC = os.path.join(ROOT, "paper_2609_04875_gb300", "csrc")
 KERNEL_SRC = {
     "prefill": ("pe_attn.cu", "template <int HD, bool SPLIT, bool VAPART, bool ONE>\n__global__", "// Exercises the bounded wait on its own"),
     "prefill_sk": ("pe_attn_sk.cu", "// Merge of one row of a cut unit's q-tile", "template <int HD, bool ONE>\ncudaError_t launch_sk_t("),
-    "decode": ("pe_decode.cu", "template <int HD, int RB>\n__global__ void __launch_bounds__(kTcThreads, 1)",
-               "template <int HD, int RB>\ncudaError_t launch_tc("),
+    "decode": ("pe_decode.cu", "template <int HD, int RB, bool TWO>\n__global__ void __launch_bounds__(kTcThreads, 1)",
+               "template <int HD, int RB, bool TWO>\ncudaError_t launch_tc_t("),
 }
 
 

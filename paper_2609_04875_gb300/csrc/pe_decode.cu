@@ -443,8 +443,8 @@ __global__ void __launch_bounds__(kDecThreads, DecCfg<HD, RB>::kMinBlocks)
 // Tensor-core form (d = 128 and d = 64).  With keys on the M side of the MMA
 // the few query rows become N = 16 (rows padded):
 //     S^T [128 keys x 16] = K [128 x d] . Q^T          (A = K tile, B = Q; K-major)
-//     O^T [d x kPRows]   += V^T [d x 128 keys] . P^T   (A = V tile, MN-major; B = P^T, K-major, its weights
-//                                                       in two bf16 parts, a row each: TcCfg::kPRows)
+//     O^T [d x kPRows]   += V^T [d x 128 keys] . P^T   (A = V tile, MN-major; B = P^T, K-major, some launches'
+//                                                       weights in two bf16 parts, a row each: TcCfg::kPRows)
 // both accumulated in TMEM (lane = key for S^T, lane = d-column for O^T), so a
 // softmax thread owns one key and touches only its RB valid row values per
 // 128-key tile.  For d = 64 the O^T GEMM keeps M = 128: the A operand's second
@@ -465,11 +465,11 @@ __global__ void __launch_bounds__(kDecThreads, DecCfg<HD, RB>::kMinBlocks)
 //
 // Roles (384 threads):
 //   warps 0-3  softmax: thread t = key t of the tile (TMEM lane t); masks,
-//              exp2 against a per-row reference, P^T (two bf16 parts) to shared memory,
+//              exp2 against a per-row reference, P^T (bf16, or two bf16 parts) to shared memory,
 //              per-thread partial row sums; per chunk, the row statistics
 //              (m, l) for the epilogue.
-//   warps 7-10 epilogue: thread = d-column (TMEM lane); per chunk, reads O^T, adds
-//              its two parts (double-buffered in TMEM, so the next chunk accumulates into
+//   warps 7-10 epilogue: thread = d-column (TMEM lane); per chunk, reads O^T
+//              (its two parts added; double-buffered in TMEM, so the next chunk accumulates into
 //              the other buffer meanwhile), writes the output or the chunk's
 //              partial.
 //   warp 11    scheduler + page-id loader: takes chunk ids (one chunk ahead of
@@ -498,7 +498,7 @@ constexpr int kDescInts = 8 + 8 * 16;              // header, then the row of bo
 constexpr int kBarSoftmax = 2;                     // named barrier of the softmax warps
 constexpr float kTcWeightLimit = 1.8446744e19f;    // 2^64
 
-template <int HD, int RB>
+template <int HD, int RB, bool TWO>
 struct TcCfg {
     static constexpr int kRegs = HD / 64;                   // 64-column halves of a K, V or Q row
     static constexpr int kRegionBytes = kTcKeys * 128;      // 128 keys x 64 columns (bf16), 128-byte swizzle
@@ -506,14 +506,15 @@ struct TcCfg {
     static constexpr int kLoadBytes = kTcKeys * HD * 2;     // bytes the TMA boxes of one tile deliver
     static constexpr int kOffV = kTcKStages * kTileBytes;   // K ring, then V ring
     static constexpr int kOffQ = (kTcKStages + kTcVStages) * kTileBytes;  // Q x2: [16 rows][128] bf16, 2 x 2 KB each
-    // P^T x2: [kPRows][128 keys] bf16, 2 regions of 64 keys each.  A weight is held as two bf16 parts, its
-    // upper 16 bits in row r and what they leave over in row kLo + r, both multiplied by the one MMA (for
-    // up to 8 rows in columns its N = 16 has anyway), so the weights carry 16 bits and only the output's
-    // rounding is left: the error against 64 bits is 1.7e-3 of the output whatever the chunk length.  (Rounded
-    // once, a chunk's largest weight of its first tile is exactly 1, so the error grew from 2.25e-3 with chunks
-    // of 2 tiles to 2.33e-3 with 8.)  It costs 1.2 % where a layer is a few tiles per SM (64 heads on 12k, 17.3 ->
-    // 17.5 us a layer), nothing at 16 agents (66.0 us), 3 % with 16 rows.
-    static constexpr int kPRows = RB <= 8 ? 16 : 32;
+    // P^T x2: [kPRows][128 keys] bf16, 2 regions of 64 keys each.  Rounded once to bf16, a chunk's largest weight of
+    // its first tile is exactly 1, so the error against 64 bits grows with the chunk length (2.25e-3 of the output with
+    // chunks of 2 tiles, 2.33e-3 with 8).  TWO, for launches whose chunks are longer than three a SM: a weight is held
+    // as two bf16 parts, nearly its upper 16 bits in row r and what they leave over in row kLo + r, both multiplied by
+    // the one MMA (for up to 8 rows in columns its N = 16 has anyway): 16 bits of it count and the output's rounding
+    // is what is left, 1.7e-3 for every chunk length.  64 heads on 12k: 17.1 -> 17.35 us a layer (20.8 with chunks of 2
+    // tiles); 16 rows a kv-head 1 to 4 %.  In the form for every launch, at run time, 10 agents of 16 rows took
+    // 2.5 % more with one part.
+    static constexpr int kPRows = TWO && RB > 8 ? 32 : 16;
     static constexpr int kLo = kPRows / 2;
     static constexpr int kPRegion = kPRows * 128;
     static constexpr int kPBytes = 2 * kPRegion;
@@ -530,7 +531,7 @@ struct TcCfg {
     static constexpr int kOffDesc = kOffSeqs + kMaxSegs * static_cast<int>(sizeof(DecodeSeq) + 4);  // + rem_seq
     static constexpr int kSmem = kOffDesc + kDescRing * kDescInts * 4;
     static constexpr int kDynSmem = kSmem + 1024;
-    static constexpr uint32_t kTmemCols = RB <= 8 ? 64 : 128;  // S^T buffers at 0 and 16, O^T at 32 and 32 + kPRows
+    static constexpr uint32_t kTmemCols = kPRows == 16 ? 64 : 128;  // S^T buffers at 0 and 16, O^T at 32 and 32 + kPRows
     static_assert(32 + 2 * kPRows <= static_cast<int>(kTmemCols), "O^T buffers");
     static_assert(kDynSmem <= 232448, "shared memory budget");
     static_assert(RB == 4 || RB == 8 || RB == 16, "row capacity");
@@ -586,12 +587,12 @@ __device__ __forceinline__ ChunkInfo tc_chunk(const DecodeParams &p, const Decod
     return ci;
 }
 
-template <int HD, int RB>
+template <int HD, int RB, bool TWO>
 __global__ void __launch_bounds__(kTcThreads, 1)
     decode_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                      const __grid_constant__ DecodeParams p)
 {
-    using C = TcCfg<HD, RB>;
+    using C = TcCfg<HD, RB, TWO>;
     constexpr int R = kChunkRing;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -1051,7 +1052,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         if (done) {
                             ptx::tc_fence_after();
 #pragma unroll
-                            for (int part = 0; part < 2; ++part) {
+                            for (int part = 0; part < (TWO ? 2 : 1); ++part) {
                                 const uint32_t to = t_o + C::kPRows * (n & 1) + part * C::kLo + lane_off;
                                 float o[RB];
                                 ptx::tmem_ld_n<RB>(to, o);
@@ -1070,20 +1071,27 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 if (i >= 2) (void)wait_bar_warp(b_o_done + 8 * (i & 1), ((i - 2) >> 1) & 1, wctx);
                 uint8_t *pt = smem + C::kOffP + (i & 1) * C::kPBytes + (t >> 6) * C::kPRegion;
                 const int chunk = (t & 63) >> 3;
-                // a weight's upper part is its upper 16 bits (cut, not rounded: no conversion), the rest rounds to the
-                // lower part, two rows a conversion
+                if constexpr (TWO) {
+                    // the upper part is cut from the float next below the weight, so that what is left over is not zero
+                    // (zero times an infinite V would be NaN); the lower parts round, two rows a conversion
+                    auto upper = [](float w) { return __float_as_uint(w * 0x0.ffffffp0f) & 0xffff0000u; };
 #pragma unroll
-                for (int r = 0; r < RB; r += 2) {
-                    const uint32_t w0 = __float_as_uint(pr[r]), w1 = __float_as_uint(pr[r + 1]);
-                    const uint32_t lo = pack_bf16(pr[r] - __uint_as_float(w0 & 0xffff0000u),
-                                                  pr[r + 1] - __uint_as_float(w1 & 0xffff0000u));
-                    // (row kLo + r has row r's place in its swizzle atom)
-                    uint8_t *d0 = pt + r * 128 + ((chunk ^ (r & 7)) << 4) + (t & 7) * 2;
-                    uint8_t *d1 = pt + (r + 1) * 128 + ((chunk ^ ((r + 1) & 7)) << 4) + (t & 7) * 2;
-                    *reinterpret_cast<uint16_t *>(d0) = static_cast<uint16_t>(w0 >> 16);
-                    *reinterpret_cast<uint16_t *>(d1) = static_cast<uint16_t>(w1 >> 16);
-                    *reinterpret_cast<uint16_t *>(d0 + C::kLo * 128) = static_cast<uint16_t>(lo);
-                    *reinterpret_cast<uint16_t *>(d1 + C::kLo * 128) = static_cast<uint16_t>(lo >> 16);
+                    for (int r = 0; r < RB; r += 2) {
+                        const uint32_t w0 = upper(pr[r]), w1 = upper(pr[r + 1]);
+                        const uint32_t lo = pack_bf16(pr[r] - __uint_as_float(w0), pr[r + 1] - __uint_as_float(w1));
+                        // (row kLo + r has row r's place in its swizzle atom)
+                        uint8_t *d0 = pt + r * 128 + ((chunk ^ (r & 7)) << 4) + (t & 7) * 2;
+                        uint8_t *d1 = pt + (r + 1) * 128 + ((chunk ^ ((r + 1) & 7)) << 4) + (t & 7) * 2;
+                        *reinterpret_cast<uint16_t *>(d0) = static_cast<uint16_t>(w0 >> 16);
+                        *reinterpret_cast<uint16_t *>(d1) = static_cast<uint16_t>(w1 >> 16);
+                        *reinterpret_cast<uint16_t *>(d0 + C::kLo * 128) = static_cast<uint16_t>(lo);
+                        *reinterpret_cast<uint16_t *>(d1 + C::kLo * 128) = static_cast<uint16_t>(lo >> 16);
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < RB; ++r)
+                        *reinterpret_cast<__nv_bfloat16 *>(pt + r * 128 + ((chunk ^ (r & 7)) << 4) + (t & 7) * 2) =
+                            __float2bfloat16_rn(pr[r]);
                 }
                 ptx::fence_proxy_async_smem();
                 ptx::tc_fence_before();
@@ -1145,12 +1153,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             if (wait_bar_warp(b_o_item + 8 * (n & 1), (n >> 1) & 1, wctx)) {
                 ptx::tc_fence_after();
-                float o_lo[RB];
                 ptx::tmem_ld_n<RB>(t_o + C::kPRows * (n & 1) + lane_off, o);
-                ptx::tmem_ld_n<RB>(t_o + C::kPRows * (n & 1) + C::kLo + lane_off, o_lo);
-                ptx::tmem_wait_ld();
+                if constexpr (TWO) {
+                    float o_lo[RB];
+                    ptx::tmem_ld_n<RB>(t_o + C::kPRows * (n & 1) + C::kLo + lane_off, o_lo);
+                    ptx::tmem_wait_ld();
 #pragma unroll
-                for (int r = 0; r < RB; ++r) o[r] += o_lo[r];
+                    for (int r = 0; r < RB; ++r) o[r] += o_lo[r];
+                } else {
+                    ptx::tmem_wait_ld();
+                }
             }
             ptx::tc_fence_before();
             ptx::mbar_arrive(b_o_free + 8 * (n & 1));  // O^T buffer and stats slot may be reused
@@ -1319,12 +1331,12 @@ __global__ void __launch_bounds__(kCombThreads) decode_tc_combine_kernel(const _
     *dst = make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
 }
 
-template <int HD, int RB>
-cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const DecodeParams &p, cudaStream_t st)
+template <int HD, int RB, bool TWO>
+cudaError_t launch_tc_t(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const DecodeParams &p, cudaStream_t st)
 {
-    using C = TcCfg<HD, RB>;
+    using C = TcCfg<HD, RB, TWO>;
     static std::atomic<uint64_t> configured{0};
-    cudaError_t e = set_dyn_smem_once(decode_tc_kernel<HD, RB>, C::kDynSmem, configured);
+    cudaError_t e = set_dyn_smem_once(decode_tc_kernel<HD, RB, TWO>, C::kDynSmem, configured);
     if (e != cudaSuccess) return e;
     // programmatic serialization: the CTAs' set-up may overlap the tail of the previous kernel
     cudaLaunchConfig_t cfg = {};
@@ -1337,7 +1349,7 @@ cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const De
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, decode_tc_kernel<HD, RB>, tm_k, tm_v, p);
+    e = cudaLaunchKernelEx(&cfg, decode_tc_kernel<HD, RB, TWO>, tm_k, tm_v, p);
     if (e != cudaSuccess) return e;
     if (!p.any_split) return cudaSuccess;  // every item was one chunk
     // the merges, also with programmatic serialization (its launch overlaps the decode grid's end)
@@ -1349,6 +1361,12 @@ cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const De
     ccfg.attrs = attr;
     ccfg.numAttrs = 1;
     return cudaLaunchKernelEx(&ccfg, decode_tc_combine_kernel<HD, RB>, p);
+}
+
+template <int HD, int RB>
+cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const DecodeParams &p, cudaStream_t st)
+{
+    return p.two_parts ? launch_tc_t<HD, RB, true>(tm_k, tm_v, p, st) : launch_tc_t<HD, RB, false>(tm_k, tm_v, p, st);
 }
 
 template <int HD, int RB>

@@ -796,6 +796,8 @@ pe_status run_decode(pe_cache *c, const std::vector<AttnItem> &items, int32_t la
             p.oob_row = static_cast<int32_t>(c->pool_rows);
             p.scale_log2 = scale * 1.4426950408889634f;
             p.any_split = any_split ? 1 : 0;
+            // longer chunks than three a SM round the weights more: two parts then (TcCfg::kPRows)
+            p.two_parts = k_per_sm == 0 && p.seqs[0].cta0 > std::max<int64_t>(1, std::min<int64_t>(8, ceil_div(tiles, 3 * c->num_sms)));
             c->last_split = any_split ? 1 : 0;
             c->last_splits = p.seqs[0].n_splits;
             c->last_ctas = p.total_ctas;

@@ -196,6 +196,7 @@ struct DecodeParams {
     int32_t total_tiles;   // tensor-core kernel: chunks of all (sequence, kv-head) items
     int32_t full_chunks;   // tensor-core kernel: ids below this are full chunks, the rest remainder chunks
     int32_t any_split;     // tensor-core kernel: some item has several chunks (a combine launch follows)
+    int32_t two_parts;     // tensor-core kernel: the form whose weights have two bf16 parts (TcCfg::kPRows)
     float scale_log2;      // softmax_scale * log2(e)
     DecodeSeq seqs[kMaxSegs];
     int32_t rem_seq[kMaxSegs];  // tensor-core kernel: the sequence of remainder block j (ids
