@@ -107,23 +107,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])
         : "memory");
 }
 
-// D[tmem] (+)= A[tmem] * B[smem] (A = P, bf16 packed two per column).
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// The same tcgen05 operations executed by a whole converged warp: one elected lane issues them (elect.sync
+// tcgen05 operations executed by a whole converged warp: one elected lane issues them (elect.sync
 // names the same lane every time, so a commit covers the MMAs issued before it).  Issued this way the
 // operands stay in uniform registers.  Issued by one thread inside a divergent branch, each MMA spent
 // 84-93 cycles on moving its descriptors there, more than the 64 cycles a 128 x 128 x 16 MMA takes: a
 // GB300 microbenchmark ran 16 P V and 16 S MMAs in 2690-2970 cycles from one thread, 2350 from a warp.
+// D[tmem] (+)= A[smem] * B[smem], kind::f16 (bf16 inputs, fp32 accumulate), cta_group::1.
 __device__ __forceinline__ void mma_bf16_warp(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                               uint32_t accumulate)
 {
@@ -136,6 +125,7 @@ __device__ __forceinline__ void mma_bf16_warp(uint32_t d_tmem, uint64_t a_desc, 
         : "memory");
 }
 
+// The same with A = P in TMEM, bf16 packed two per column.
 __device__ __forceinline__ void mma_bf16_ts_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                                  uint32_t accumulate)
 {
@@ -148,6 +138,7 @@ __device__ __forceinline__ void mma_bf16_ts_warp(uint32_t d_tmem, uint32_t a_tme
         : "memory");
 }
 
+// Arrive once on `bar` when every tcgen05 op that the elected lane issued so far completes.
 __device__ __forceinline__ void mma_commit_warp(uint32_t bar)
 {
     asm volatile(
