@@ -910,7 +910,7 @@ cudaError_t launch_replay_attn(int head_dim, bool split, const CUtensorMap &tm_q
 }
 
 template <int HD, int COLS, int BATCH>
-static cudaError_t launch_combine_t(const AttnParams &p, int ns, cudaStream_t st)
+static cudaError_t launch_combine_t(const AttnParams &p, int ns, int64_t sms, cudaStream_t st)
 {
     constexpr int kCombSmSmem = 226 * 1024;  // shared memory of an SM, nearly
     const int64_t warps = static_cast<int64_t>(p.total_comb + 31) / 32 * (HD / COLS);  // row blocks x column groups
@@ -918,7 +918,6 @@ static cudaError_t launch_combine_t(const AttnParams &p, int ns, cudaStream_t st
     // and the merge runs on those alone.  So, from 8 MB of partials on, a block an SM (up to 8 warps each), kept
     // to that many an SM by its shared memory: 2 agents x 133 tokens on 1.3k, 3 splits, 17.8 -> 15.5 us a layer,
     // attention included (d = 128).  Below, blocks of one warp, waiting early: 5.2 MB 10.7 us against 11.2.
-    const int64_t sms = p.next_stride > 0 ? p.next_stride : 152;
     const bool small = static_cast<int64_t>(p.total_comb) * ns * HD * 4 < (8 << 20);
     const int per_block = small ? 1 : static_cast<int>(std::min<int64_t>(8, (warps + sms - 1) / sms));
     const int64_t blocks = (warps + per_block - 1) / per_block;
@@ -941,13 +940,13 @@ static cudaError_t launch_combine_t(const AttnParams &p, int ns, cudaStream_t st
     return cudaLaunchKernelEx(&cfg, splitkv_combine_kernel<HD, COLS, BATCH>, p);
 }
 
-cudaError_t launch_splitkv_combine(int head_dim, const AttnParams &p, cudaStream_t st)
+cudaError_t launch_splitkv_combine(int head_dim, const AttnParams &p, int num_sms, cudaStream_t st)
 {
     if (p.total_comb <= 0) return cudaSuccess;
     int ns = 0;
     for (int i = 0; i < p.n_seqs; ++i) ns = std::max(ns, static_cast<int>(p.seqs[i].n_splits));
-    if (head_dim == 128) return ns <= 4 ? launch_combine_t<128, 32, 4>(p, ns, st) : launch_combine_t<128, 16, 8>(p, ns, st);
-    if (head_dim == 64) return ns <= 4 ? launch_combine_t<64, 32, 4>(p, ns, st) : launch_combine_t<64, 16, 8>(p, ns, st);
+    if (head_dim == 128) return ns <= 4 ? launch_combine_t<128, 32, 4>(p, ns, num_sms, st) : launch_combine_t<128, 16, 8>(p, ns, num_sms, st);
+    if (head_dim == 64) return ns <= 4 ? launch_combine_t<64, 32, 4>(p, ns, num_sms, st) : launch_combine_t<64, 16, 8>(p, ns, num_sms, st);
     return cudaErrorInvalidValue;
 }
 

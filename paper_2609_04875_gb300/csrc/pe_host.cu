@@ -1561,7 +1561,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         if (!rec) c->launches++;
         if (split && !rec) {
             if (injected_failure(c)) return launch_fault("split-KV combine");
-            e = launch_splitkv_combine(d, p, st);
+            e = launch_splitkv_combine(d, p, c->num_sms, st);
             if (e != cudaSuccess) return cuda_fail(e, "split-KV combine launch");
             c->launches++;
         }
@@ -1588,7 +1588,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
             if (e != cudaSuccess) return cuda_fail(e, "replay attention tail launch");
             c->launches++;
             if (injected_failure(c)) return launch_fault("split-KV combine");
-            e = launch_splitkv_combine(d, p, st);
+            e = launch_splitkv_combine(d, p, c->num_sms, st);
             if (e != cudaSuccess) return cuda_fail(e, "split-KV combine launch");
             c->launches++;
         }
@@ -2149,7 +2149,7 @@ pe_status pe_replay_attn_static_scratch(pe_cache *c, int32_t seq, int32_t layer,
     if (e != cudaSuccess) return cuda_fail(e, "replay attention launch");
     c->launches++;
     if (injected_failure(c)) return launch_fault("split-KV combine");
-    e = launch_splitkv_combine(d, p, st);
+    e = launch_splitkv_combine(d, p, c->num_sms, st);
     if (e != cudaSuccess) return cuda_fail(e, "split-KV combine launch");
     c->launches++;
     return PE_OK;

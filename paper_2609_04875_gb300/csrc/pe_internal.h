@@ -219,7 +219,7 @@ cudaError_t launch_cow_copy(const CowParams &p, cudaStream_t st);
 // tm_o: the output as a map of the same shape as tm_q (full q-tiles are stored by TMA); unused when split
 cudaError_t launch_replay_attn(int head_dim, bool split, const CUtensorMap &tm_q, const CUtensorMap &tm_k,
                                const CUtensorMap &tm_v, const CUtensorMap &tm_o, const AttnParams &p, cudaStream_t st);
-cudaError_t launch_splitkv_combine(int head_dim, const AttnParams &p, cudaStream_t st);
+cudaError_t launch_splitkv_combine(int head_dim, const AttnParams &p, int num_sms, cudaStream_t st);
 // Persistent stream-K attention (p.n_ctas CTAs), cut units merged in the kernel.
 cudaError_t launch_replay_attn_sk(int head_dim, const CUtensorMap &tm_q, const CUtensorMap &tm_k,
                                   const CUtensorMap &tm_v, const SkParams &p, cudaStream_t st);
