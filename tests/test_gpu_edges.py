@@ -2,8 +2,10 @@
 gives way to the next: one-q-tile launches of a few key tiles, pairs whose
 q-tiles end at different key tiles (with V's producer apart or not), split
 merges around their batch of splits and their block shapes, persistent pieces of
-one or two q-tiles, decode merges of one and of many chunks, and appends, crops
-and copy-on-write around the limits of their parameter blocks.  Attention is held
+one or two q-tiles, the plans taken by default (small workspaces too), decode
+merges of one and of many chunks and the decode weights' parts, NaN and infinite
+inputs, rounds against their calls made one by one, and appends, crops and
+copy-on-write around the limits of their parameter blocks.  Attention is held
 to the gate of tests/parity.py against the fp64 oracle; everything that moves
 bytes is compared exactly."""
 import math
@@ -81,16 +83,63 @@ def test_split_merge_shapes(d, splits, wide):
     assert plan[1] == -(-17 // -(-17 // splits)), plan
 
 
-@pytest.mark.parametrize("d", [64, 128])
-def test_default_plans_of_mixed_launches(d):
-    """The plan's own choice over launches of few and of many units, with units of one q-tile among pairs."""
-    kinds = set()
-    for i, (lens, nqs, hq, hkv) in enumerate([
-            ([1500, 900, 2000, 700], [200, 33, 129, 60], 32, 8), ([600] * 24, [40] * 24, 16, 8),
-            ([3000], [700], 32, 8), ([900] * 3, [300] * 3, 64, 8), ([2500, 2600], [20, 20], 32, 8)]):
-        split, _, ctas = _batch(d, hq, hkv, 16, lens, nqs, {}, seed=40 + i)
-        kinds.add((split, ctas == 152))
-    assert len(kinds) > 1, kinds
+# (d, Hq, Hkv, keys, queries): the plan's kernel and whether keys are cut, on 152 SMs
+DEFAULT_PLANS = [
+    # one-item: pairs and lone q-tiles with key splits and in one pass, lone ones with key splits
+    (64, 32, 8, [1500, 900, 2000, 700], [200, 33, 129, 60], "one_item", True),
+    (128, 32, 8, [1500, 900, 2000, 700], [200, 33, 129, 60], "one_item", True),
+    (64, 16, 4, [376], [72], "one_item", False),
+    (128, 32, 4, [376, 231, 244, 290, 241, 275, 256, 343, 395, 320, 271, 298, 328, 223, 314, 377, 327, 332, 338, 331],
+     [87, 67, 169, 144, 56, 30, 146, 72, 177, 138, 121, 32, 187, 70, 150, 170, 52, 192, 65, 111], "one_item", False),
+    (64, 32, 8, [2500, 2600], [20, 20], "one_item", True),
+    (128, 32, 8, [2500, 2600], [20, 20], "one_item", True),
+    (64, 16, 8, [600] * 24, [40] * 24, "persistent", False),
+    (128, 16, 8, [600] * 24, [40] * 24, "one_item", False),
+    # persistent with cuts: pairs only, pairs and lone q-tiles, lone ones only
+    (64, 8, 8, [914, 1658, 1325], [768, 512, 1024], "persistent", True),
+    (128, 32, 8, [2490, 1746], [256, 384], "persistent", True),
+    (64, 8, 8, [959, 1577], [784, 1501], "persistent", True),
+    (128, 8, 8, [1522, 2254], [1115, 1297], "persistent", True),
+    (64, 32, 8, [793, 744, 522, 607, 510, 605, 577, 599, 618, 721, 732, 680, 791, 654, 467, 765, 808, 760, 658, 578],
+     [26, 9, 31, 8, 7, 7, 27, 22, 5, 29, 16, 6, 7, 13, 6, 8, 10, 11, 6, 16], "persistent", True),
+    (128, 32, 8, [4176, 8101, 5250, 4692, 4445, 4434, 6705, 5325, 4922, 6424, 5707, 7662],
+     [21, 23, 24, 7, 5, 31, 7, 31, 15, 27, 30, 27], "persistent", True),
+    # persistent, at least two units a SM: rounds of whole units before the cut ones
+    (64, 32, 4, [767, 990, 949, 741, 598, 938, 746, 915, 872, 618, 935, 955, 746, 806, 802, 911, 976, 824, 688, 939],
+     [188, 21, 60, 171, 126, 82, 57, 67, 126, 182, 79, 148, 75, 169, 190, 154, 46, 93, 45, 145], "persistent", True),
+    (128, 32, 4, [939, 1043, 948, 1549, 1695, 902, 1282, 1427, 1300, 1173, 1350, 1536, 1680, 1579, 1743, 1023, 1511, 1736,
+                  1447, 1000],
+     [159, 140, 171, 83, 105, 37, 71, 185, 139, 116, 101, 107, 171, 78, 76, 172, 46, 29, 77, 40], "persistent", True),
+]
+
+
+@pytest.mark.parametrize("d,hq,hkv,lens,nqs,kind,cut", DEFAULT_PLANS)
+def test_default_plans_of_mixed_launches(d, hq, hkv, lens, nqs, kind, cut):
+    """The plan's own choice over launches of few and of many units, of pairs, lone q-tiles and both: the kernel it
+    takes, with and without cut keys, and a sample of every sequence's rows against the oracle."""
+    npg = sum(-(-n // 16) for n in lens) + 4
+    pair = Pair(1, hkv, d, 16, npg, len(lens), max(-(-n // 16) for n in lens) + 1, seed=len(lens) + d)
+    g = synth.rng(d + len(lens), 79)
+    seqs = []
+    for n in lens:
+        s = pair.seq()
+        pair.append(s, synth.normal_bf16(g, (1, n, hkv, d)), synth.normal_bf16(g, (1, n, hkv, d)))
+        seqs.append(s)
+    plan = pair.gpu.plan_launches(seqs, nqs, hq)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert [(x["kind"], bool(x["split"])) for x in plan] == [(kind, cut)]
+        if kind == "persistent":
+            p = pair.gpu.plan_persistent(seqs, nqs, hq)
+            assert (p["rounds"] > 0) == (len(p["unit_tiles"]) >= 2 * 152) and (p["n_slots"] > 0) == cut
+    cu = [0] + [int(x) for x in np.cumsum(nqs)]
+    q = synth.normal_bf16(g, (cu[-1], hq, d))
+    out = pair.gpu.replay_attn_batch(seqs, 0, dev(q), cu)
+    torch.cuda.synchronize()
+    for i, s in enumerate(seqs):
+        rows = np.unique(np.concatenate([np.arange(0, nqs[i], 11), [nqs[i] // 2, nqs[i] - 1]]))
+        ref = oracle.replay_attention(pair.orc, s, 0, q[cu[i]:cu[i + 1]], 1 / math.sqrt(d), rows=rows)
+        assert_close(out[cu[i]:cu[i + 1]][torch.from_numpy(rows).cuda()], ref, f"d={d} {kind} seq {i}")
+    assert pair.gpu.device_status() == 0
 
 
 @pytest.mark.parametrize("d,hq,hkv", [(128, 8, 2), (64, 16, 1), (128, 32, 8)])
@@ -165,34 +214,36 @@ def test_copy_on_write_of_many_branches_in_one_append(branches):
     _check_pools(pair, L, hkv, ps, d)
 
 
-@pytest.mark.parametrize("keys", [(60, 90), (700, 1300), (100, 3000)])
-def test_rounds_equal_their_calls_one_by_one(keys):
+@pytest.mark.parametrize("layers,keys", [(1, (60, 90)), (1, (700, 1300)), (1, (100, 3000)), (3, (700, 1300))])
+def test_rounds_equal_their_calls_one_by_one(layers, keys):
     """Decode rounds in one call, where a round's append runs beside the merge before it, against the same
     appends and attention calls made one by one: the same output bits, pages and lengths.  Items of one
     chunk (no merge), of several, and both; a fork's copy-on-write before the first append."""
     hq, hkv, d, ps, rounds = 32, 8, 128, 16, 12
     g = synth.rng(sum(keys), 74)
-    base = [(synth.normal_bf16(g, (1, n, hkv, d)), synth.normal_bf16(g, (1, n, hkv, d))) for n in keys]
+    base = [(synth.normal_bf16(g, (layers, n, hkv, d)), synth.normal_bf16(g, (layers, n, hkv, d))) for n in keys]
     n = len(keys) + 1
     cu = [rounds * i for i in range(n + 1)]
-    K, V, Q = (dev(synth.normal_bf16(g, (1, cu[-1], h, d))) for h in (hkv, hkv, hq))
+    K, V, Q = (dev(synth.normal_bf16(g, (layers, cu[-1], h, d))) for h in (hkv, hkv, hq))
     outs, pools = [], []
     for whole in (True, False):
-        pair = Pair(1, hkv, d, ps, sum(-(-k // ps) for k in keys) + 2 * n + 8, n, 220, seed=6)
+        pair = Pair(layers, hkv, d, ps, sum(-(-k // ps) for k in keys) + 2 * n + 8, n, 220, seed=6)
         seqs = []
         for k, v in base:
             s = pair.seq()
             pair.append(s, k, v)
             seqs.append(s)
         seqs.append(pair.gpu.seq_fork(seqs[0]))
-        out = torch.zeros((1, cu[-1], hq, d), dtype=torch.bfloat16, device="cuda")
+        out = torch.zeros((layers, cu[-1], hq, d), dtype=torch.bfloat16, device="cuda")
         if whole:
             pair.gpu.replay_rounds(seqs, [[1] * n] * rounds, cu, K, V, Q, out=out)
         else:
             for r in range(rounds):
                 idx = torch.tensor([c + r for c in cu[:-1]], device="cuda")
                 pair.gpu.append_kv_batch(seqs, K[:, idx].contiguous(), V[:, idx].contiguous(), list(range(n + 1)))
-                out[0, idx] = pair.gpu.replay_attn_batch(seqs, 0, Q[0, idx].contiguous(), list(range(n + 1)))
+                for layer in range(layers):
+                    out[layer, idx] = pair.gpu.replay_attn_batch(seqs, layer, Q[layer, idx].contiguous(),
+                                                                 list(range(n + 1)))
         torch.cuda.synchronize()
         assert pair.gpu.device_status() == 0
         outs.append(out)
@@ -282,3 +333,62 @@ def test_a_nan_key_reaches_every_output_that_attends_it(d, nq, options, where):
     assert pair.gpu.device_status() == 0
     assert_close(out[:, :4], ref[:, :4], f"{options}")
     assert torch.isnan(out[:, 4:]).all(), (options, pair.gpu.last_attn_plan())
+
+
+@pytest.mark.parametrize("keys", [(700, 1300), (100, 3000)])
+def test_rounds_with_out_over_the_next_keys(keys):
+    """Decode rounds whose out row j is K's row j + 1 (one buffer): a round's output is the next round's key, so its
+    append must not run beside the merge that writes it.  Against the same calls made one by one."""
+    h, d, ps, rounds = 8, 128, 16, 24
+    g = synth.rng(sum(keys), 80)
+    base = [(synth.normal_bf16(g, (1, n, h, d)), synth.normal_bf16(g, (1, n, h, d))) for n in keys]
+    n = len(keys)
+    cu = [rounds * i for i in range(n + 1)]
+    first, V, Q = (dev(synth.normal_bf16(g, (1, cu[-1] + 1, h, d))) for _ in range(3))
+    V, Q = V[:, :-1].contiguous(), Q[:, :-1].contiguous()
+    got = []
+    for whole in (True, False):
+        pair = Pair(1, h, d, ps, sum(-(-k // ps) for k in keys) + 2 * n + 8, n, 220, seed=7)
+        seqs = []
+        for k, v in base:
+            s = pair.seq()
+            pair.append(s, k, v)
+            seqs.append(s)
+        buf = first.clone()
+        K, out = buf[:, :-1], buf[:, 1:]
+        if whole:
+            pair.gpu.replay_rounds(seqs, [[1] * n] * rounds, cu, K, V, Q, out=out)
+        else:
+            for r in range(rounds):
+                idx = torch.tensor([c + r for c in cu[:-1]], device="cuda")
+                pair.gpu.append_kv_batch(seqs, K[:, idx].contiguous(), V[:, idx].contiguous(), list(range(n + 1)))
+                out[0, idx] = pair.gpu.replay_attn_batch(seqs, 0, Q[0, idx].contiguous(), list(range(n + 1)))
+        torch.cuda.synchronize()
+        assert pair.gpu.device_status() == 0
+        got.append(buf)
+    assert torch.equal(got[0], got[1])
+    assert not torch.equal(got[0], first)
+
+
+@pytest.mark.parametrize("d,lens,nqs,hq,ws", [(64, [8192] * 3, [20] * 3, 64, 1 << 20), (128, [2490, 1746], [256, 384], 32, 4 << 20),
+                                              (128, [2490, 1746], [256, 384], 32, 24 << 20)])
+def test_default_plans_with_a_small_workspace(d, lens, nqs, hq, ws):
+    """The default plan where the workspace holds none or some of the parts that cuts would need."""
+    hkv = 8
+    npg = sum(-(-n // 16) for n in lens) + 4
+    pair = Pair(1, hkv, d, 16, npg, len(lens), max(lens) // 16 + 2, seed=d, pe_kwargs={"workspace_bytes": ws})
+    g = synth.rng(d + ws, 81)
+    seqs = []
+    for n in lens:
+        s = pair.seq()
+        pair.append(s, synth.normal_bf16(g, (1, n, hkv, d)), synth.normal_bf16(g, (1, n, hkv, d)))
+        seqs.append(s)
+    cu = [0] + [int(x) for x in np.cumsum(nqs)]
+    q = synth.normal_bf16(g, (cu[-1], hq, d))
+    out = pair.gpu.replay_attn_batch(seqs, 0, dev(q), cu)
+    torch.cuda.synchronize()
+    for i, s in enumerate(seqs):
+        rows = np.arange(0, nqs[i], 7)
+        ref = oracle.replay_attention(pair.orc, s, 0, q[cu[i]:cu[i + 1]], 1 / math.sqrt(d), rows=rows)
+        assert_close(out[cu[i]:cu[i + 1]][torch.from_numpy(rows).cuda()], ref, f"ws={ws} seq {i}")
+    assert pair.gpu.device_status() == 0
