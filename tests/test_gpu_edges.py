@@ -110,6 +110,15 @@ DEFAULT_PLANS = [
     (128, 32, 4, [939, 1043, 948, 1549, 1695, 902, 1282, 1427, 1300, 1173, 1350, 1536, 1680, 1579, 1743, 1023, 1511, 1736,
                   1447, 1000],
      [159, 140, 171, 83, 105, 37, 71, 185, 139, 116, 101, 107, 171, 78, 76, 172, 46, 29, 77, 40], "persistent", True),
+    # the same with lone q-tiles only
+    (64, 32, 8, [747, 907, 874, 793, 864, 884, 520, 737, 909, 561, 751, 501, 715, 643, 697, 611, 749, 712, 909, 797, 652, 788,
+                 520, 893, 826, 844, 514, 580, 495, 574, 810, 596, 682, 572, 861, 864, 692, 836, 899],
+     [31, 26, 15, 30, 12, 10, 17, 22, 15, 24, 15, 11, 16, 9, 29, 28, 18, 11, 25, 15, 24, 5, 10, 17, 6, 6, 14, 20, 12, 24, 10,
+      23, 29, 13, 31, 13, 26, 6, 8], "persistent", True),
+    (128, 64, 8, [221, 216, 278, 342, 296, 236, 215, 295, 252, 253, 385, 339, 219, 298, 209, 219, 400, 246, 384, 400, 215, 384,
+                  300, 259, 274, 310, 386, 280, 355, 398, 221, 250, 234, 276, 211, 276, 281, 283, 389],
+     [9, 16, 3, 4, 14, 15, 8, 14, 14, 3, 9, 3, 8, 16, 7, 11, 12, 5, 16, 12, 16, 12, 10, 13, 6, 12, 3, 9, 13, 8, 3, 11, 10, 9,
+      4, 13, 15, 11, 3], "persistent", False),
 ]
 
 
