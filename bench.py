@@ -309,20 +309,20 @@ def oracle_tokens_per_s(units, budget_s, seed=7):
 # while the kernel source is the one that was captured.
 NCU_TRAFFIC = {
     "tiny": {"bytes": 1.510912e6, "profile": "profiles/traffic_attention_configs.md", "kernels": ["prefill"],
-             "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f"}},
-    "agent_batch": {"bytes": 685.47584e6 + 315.327744e6, "profile": "profiles/traffic_attention_configs.md",
-                    "kernels": ["prefill"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f"}},
-    "short_suffix": {"bytes": 1.08885632e9 + 5.18144e6, "profile": "profiles/traffic_attention_configs.md",
-                     "kernels": ["prefill_sk"], "src_sha256": {"prefill_sk": "d87018c7e548d16cb249d9d52d359f90916e3d8dd6982d6660c72bead3f55b6a"}},
-    "long_suffix": {"bytes": 1.41151616e9 + 1.03740288e9, "profile": "profiles/traffic_attention_configs.md",
-                    "kernels": ["prefill"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f"}},
-    # one sweep step's 224 attention launches (5 forget requests x 32 layers, two launches per layer where a
+             "src_sha256": {"prefill": "2d832440c6589db32d3d476157626a9c118b9d57f1b94e78b8ac82a81e71eacb"}},
+    "agent_batch": {"bytes": 684.892928e6 + 315.216384e6, "profile": "profiles/traffic_attention_configs.md",
+                    "kernels": ["prefill"], "src_sha256": {"prefill": "2d832440c6589db32d3d476157626a9c118b9d57f1b94e78b8ac82a81e71eacb"}},
+    "short_suffix": {"bytes": 1.088975872e9 + 5.404672e6, "profile": "profiles/traffic_attention_configs.md",
+                     "kernels": ["prefill_sk"], "src_sha256": {"prefill_sk": "ce48ccbfdcf5cddb3c29b0c9a2f3fcb1eb298e33bbd25aeab9da20abd269e752"}},
+    "long_suffix": {"bytes": 1.4108928e9 + 1.0369536e9, "profile": "profiles/traffic_attention_configs.md",
+                    "kernels": ["prefill"], "src_sha256": {"prefill": "2d832440c6589db32d3d476157626a9c118b9d57f1b94e78b8ac82a81e71eacb"}},
+    # one sweep step's 192 attention launches (5 forget requests x 32 layers, two launches per layer where a
     # tail launch runs), per layer: bytes / 160
-    "tau_sweep": {"bytes": (47659.393e6 + 8008.357e6) / 160, "profile": "profiles/traffic_attention_configs.md",
-                  "kernels": ["prefill", "prefill_sk"], "src_sha256": {"prefill": "18aa52c21977c6408fe5a7b0c4f4ccb0602a4e5f7c09c61ad65ea54f100ecd0f", "prefill_sk": "d87018c7e548d16cb249d9d52d359f90916e3d8dd6982d6660c72bead3f55b6a"}},
-    "decode_batch": {"bytes": 341.534464e6 + 3.879168e6, "profile": "profiles/decode_tc_decode_batch.md",
+    "tau_sweep": {"bytes": (47444.38e6 + 8073.877e6) / 160, "profile": "profiles/traffic_attention_configs.md",
+                  "kernels": ["prefill", "prefill_sk"], "src_sha256": {"prefill": "2d832440c6589db32d3d476157626a9c118b9d57f1b94e78b8ac82a81e71eacb", "prefill_sk": "ce48ccbfdcf5cddb3c29b0c9a2f3fcb1eb298e33bbd25aeab9da20abd269e752"}},
+    "decode_batch": {"bytes": 341.534464e6 + 3.933184e6, "profile": "profiles/decode_tc_decode_batch.md",
                      "kernels": ["decode"],
-                     "src_sha256": {"decode": "92c511c1911bfb21c61432aa9bdf4df8b5b389e7497f2625650667460bf98173"}},
+                     "src_sha256": {"decode": "9afb7597d4a46f6bacd82afca7ce98c9e9b576a6d049d4a91e8ff87a7d73ef63"}},
 }
 CSRC = os.path.join(ROOT, "paper_2609_04875_gb300", "csrc")
 # (file, first line of the kernel's source, the text that follows it): the span that is hashed

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __grid_constant__ 
     // p.beside that kernel is a decode merge, which lets dependents in once the decode kernel, and so all
     // before it, is complete, and which reads only partials: the append runs beside it and waits at its
     // end, so that whatever waits for the append waits for the merge too (16 agents, some 120 rounds of an
-    // append, a decode and a merge: 6630 -> 6418 us)
+    // append, a decode and a merge: 6630 -> 6404 us)
     if (!p.beside) ptx::griddep_wait();
     // 1) mirror the new page ids and lengths into the device tables
     if (blockIdx.x == 0) {
