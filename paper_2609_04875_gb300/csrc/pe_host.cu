@@ -958,21 +958,18 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
         q.pair_top = (q.n_qtiles + 1) / 2;
         q.n_splits = 1;
         q.item0 = static_cast<int32_t>(n_all.size());
-        for (int32_t local = 0; local < q.pair_top * hkv; ++local) {
-            const int32_t pair = q.pair_top - 1 - local / hkv;
+        for (int32_t pair = q.pair_top - 1; pair >= 0; --pair) {
             const int32_t qt_last = std::min(2 * pair + 1, q.n_qtiles - 1);
             const int64_t q_last = std::min<int64_t>((qt_last + 1) * static_cast<int64_t>(bmq), it.n_q) - 1;
             const int32_t n = static_cast<int32_t>(ceil_div(c->len[it.seq] - it.n_q + q_last + 1, kBN));
-            n_all.push_back(n);
-            wt.push_back(2 * pair + 1 < q.n_qtiles ? 1.0 : lone_cost);
-            cum.push_back(cum.back() + n * wt.back() + kSkUnitCost);
+            const double w = 2 * pair + 1 < q.n_qtiles ? 1.0 : lone_cost;
+            n_all.insert(n_all.end(), hkv, n);
+            wt.insert(wt.end(), hkv, w);
+            for (int h = 0; h < hkv; ++h) cum.push_back(cum.back() + n * w + kSkUnitCost);
         }
     }
     const int32_t U = static_cast<int32_t>(n_all.size());
     auto unit_cost = [&](int32_t u) { return n_all[u] * wt[u] + kSkUnitCost; };
-    auto unit_at = [&](double x) {  // the unit whose cost range holds x
-        return static_cast<int32_t>(std::upper_bound(cum.begin(), cum.end(), x) - cum.begin()) - 1;
-    };
 
     // A plan for nc CTAs.  Whole units first, in lockstep rounds: in round r CTA k takes unit
     // r nc + k (k reversed in odd rounds), so the CTAs running at once work on neighbouring units
@@ -989,9 +986,13 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
         pl.R = U >= 2 * nc ? U / nc - 1 : 0;
         const int32_t T0 = pl.R * nc;  // first tail unit
         pl.own.assign(nc, 0.0);
-        for (int32_t r = 0; r < pl.R; ++r)
-            for (int32_t k = 0; k < nc; ++k)
-                pl.own[k] += unit_cost(r * nc + ((r & 1) ? nc - 1 - k : k));
+        for (int32_t r = 0; r < pl.R; ++r) {
+            const int32_t r0 = r * nc;
+            if (r & 1)
+                for (int32_t k = 0; k < nc; ++k) pl.own[k] += unit_cost(r0 + nc - 1 - k);
+            else
+                for (int32_t k = 0; k < nc; ++k) pl.own[k] += unit_cost(r0 + k);
+        }
         const double W = cum.back() - cum[T0];
         const double mean = cum.back() / nc;
         std::vector<double> want(nc), pos(nc + 1, 0.0);
@@ -1000,13 +1001,14 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
         for (int32_t k = 0; k < nc; ++k) pos[k + 1] = pos[k] + (sum_want > 0 ? want[k] * W / sum_want : W / nc);
         pl.b.assign(nc + 1, SkBound{T0, 0});
         pl.b[nc] = SkBound{U, 0};
+        int32_t u = T0;  // the unit whose cost range holds x (the boundaries ascend)
         for (int32_t k = 1; k < nc; ++k) {
             const double x = cum[T0] + pos[k];
             SkBound bd{U, 0};
             if (x < cum.back()) {
-                const int32_t u = std::min(unit_at(x), U - 1);
+                while (u + 1 < U && cum[u + 1] <= x) ++u;
                 const double off = x - cum[u];
-                const int32_t t = static_cast<int32_t>(std::lround((off - kSkUnitCost) / wt[u]));
+                const int32_t t = static_cast<int32_t>(std::floor((off - kSkUnitCost) / wt[u] + 0.5));
                 bd = SkBound{u, 0};
                 if (cuts && t >= kSkMinPiece && n_all[u] - t >= kSkMinPiece) bd.t = t;
                 else if (off > 0.5 * unit_cost(u)) bd = SkBound{u + 1, 0};
@@ -1093,8 +1095,13 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
         p.part_lse = c->d_ws ? c->d_ws + static_cast<int64_t>(n_slots) * max_parts * 2 * kBM * d : nullptr;
     }
     P.tickets = c->d_tickets ? c->d_tickets + kMaxSegs * hkv + 2 : nullptr;
+    int32_t part = 0, part_unit = -1;  // interior boundaries of part_unit so far, each counted once (they ascend)
     for (int32_t k = 0; k < pl.nc; ++k) {
         const SkBound &a = pl.b[k], &z = pl.b[k + 1];
+        if (a.t > 0 && !(k > 0 && pl.b[k - 1] == a)) {
+            part = a.u == part_unit ? part + 1 : 1;
+            part_unit = a.u;
+        }
         SkCta &w = P.cta[k];
         w.slot0 = w.slot1 = -1;
         w.part0 = w.part1 = 0;
@@ -1110,12 +1117,7 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
         w.t1 = z.t;
         if (cuts && slot_of[a.u] >= 0) {
             w.slot0 = slot_of[a.u];
-            int32_t part = 0;  // interior boundaries of unit a.u at or before tile a.t, each counted once
-            for (size_t i = 0; i < pl.b.size(); ++i) {
-                const SkBound &x = pl.b[i];
-                if (x.u == a.u && x.t > 0 && x.t <= a.t && !(i > 0 && pl.b[i - 1] == x)) ++part;
-            }
-            w.part0 = part;
+            w.part0 = a.t > 0 ? part : 0;
         }
         if (cuts && z.u != a.u && z.t > 0) {
             w.slot1 = slot_of[z.u];
