@@ -1132,15 +1132,15 @@ pe_status plan_sk(pe_cache *c, const std::vector<AttnItem> &order, size_t lo, si
 // A CTA (the persistent kernel: a unit) costs a set-up and its key tiles.  It is a pair of q-tiles, a lone q-tile
 // in a launch that has pairs too, or one in a launch of lone q-tiles only (which has a kernel form of its own at
 // d = 128).  CTAs start in order, the heaviest first, so a launch lasts as long as its longest CTA, or as the SMs'
-// equal share with the last, partly filled wave's CTAs counted for the idle SMs beside them too; and never less
-// than reading K and V once takes.  Every term is continuous in the sizes but for the waves themselves.
+// equal share with the last, partly filled wave's CTAs counted for the idle SMs beside them too, and with reading
+// K and V once (span_and_read).  Every term is continuous in the sizes but for the waves themselves.
 // The constants are least-squares fits (of the logarithm) to 37,700 launches: 1 to 64 sequences, equal and ragged, of 50
 // to 40k keys and 17 to 20k queries, 3 to 16 kv-heads, g = 1 to 8, d = 64 and 128, up to 900 key tiles per SM, each
 // timed in one pass, as the persistent kernel and with several splits.  The estimates are off by 4 to 10 % (standard
-// deviation; one pass least), and the plans they choose 0.9 % slower than the best of those timed (geometric mean,
-// with the margins that a second launch and the longer plan ask for; 0.6 % without).  Estimates in tile times with
-// a step wherever the kind of launch changed were 1.7 %, and 53 % at the worst (one sequence of 159 units: a tail launch
-// for 44.6 us where one pass takes 29.2).
+// deviation; one pass least).  The plans they choose were 0.75 % slower than the best of one pass, the one-item plan and
+// the persistent kernel over 7,300 fresh launches with pages of 8 to 128 tokens (geometric mean; 99th percentile 12 %).
+// Estimates in tile times with a step wherever the kind of launch changed were 1.7 %, and 53 % at the worst (one
+// sequence of 159 units: a tail launch for 44.6 us where one pass takes 29.2).
 struct PrefillCosts {
     double setup[3], tile[3];        // one-item kernel: pair, lone among pairs, all lone
     double split_setup[2], split_tile[2];  // its CTAs with key splits: with pairs, all lone
@@ -1154,11 +1154,19 @@ constexpr PrefillCosts kCosts64 = {{4.9, 4.3, 4.2}, {1.01, 0.85, 0.85}, {3.1, 3.
 constexpr PrefillCosts kCosts128 = {{5.6, 5.2, 4.8}, {1.255, 1.21, 0.77}, {3.8, 5.25}, {1.34, 0.77}, {0.68, 0.66}, {0.26, 3.1},
                                     {3.0, 0.9}, {8.15e6, 6.3e6}, {5.3, 3.0, 2.5}, {1.357, 1.5, 1.3}, 2.35, 11.5, 1.75};
 
-// K and V read once, after `start`: out of L2 (about 110 MB of it) at 9 TB/s, beyond at `rate` bytes per us.
+// K and V read once, after `start`: out of L2 (about 110 MB of it) at 10 TB/s, beyond at `rate` bytes per us.
 double kv_read_us(double bytes, double start, double rate)
 {
     constexpr double kL2 = 110e6;
-    return start + std::min(bytes, kL2) / 9e6 + std::max(0.0, bytes - kL2) / rate;
+    return start + std::min(bytes, kL2) / 10e6 + std::max(0.0, bytes - kL2) / rate;
+}
+
+// The CTAs' span and the reading beside it: the longer one, and up to 19 % more where they are alike (few CTAs do not
+// draw the full rate: 16 units of 291 tiles, 5 splits 63 us a layer, 9 splits 54).
+double span_and_read(double span, double read)
+{
+    const double a = span * span, b = read * read;
+    return std::sqrt(std::sqrt(a * a + b * b));
 }
 
 // What the estimates need of a launch group; tables by kind (pair, lone among pairs, all lone).
@@ -1226,7 +1234,7 @@ double shape_span(const GroupShape &s, const double (&setup)[3], const double (&
 
 double one_pass_us(const PrefillCosts &t, const GroupShape &s, double n_sm)
 {
-    return std::max(shape_span(s, t.setup, t.tile, n_sm), kv_read_us(s.kv_bytes, 5.0, 5.6e6));
+    return span_and_read(shape_span(s, t.setup, t.tile, n_sm), kv_read_us(s.kv_bytes, 4.5, 6.2e6));
 }
 
 // The combine launch of `rows` partial rows (of one split) in ns splits.
@@ -1248,19 +1256,19 @@ double split_us(const PrefillCosts &t, const GroupShape &s, double n_sm, double 
         span = std::max(one, S / n_sm + t.wave[s.lone] * one * (1.0 - r / n_sm) +
                                  t.uneven[s.lone] * std::max(0.0, one - S / pieces));
     }
-    return std::max(span, kv_read_us(s.kv_bytes, 2.6, 5.0e6)) + merge_us(t, s.lone, head_dim, rows, ns);
+    return span_and_read(span, kv_read_us(s.kv_bytes, 2.3, 5.5e6)) + merge_us(t, s.lone, head_dim, rows, ns);
 }
 
 // The persistent kernel with whole units, and with the work cut equally over n_cta CTAs.
 double sk_whole_us(const PrefillCosts &t, const GroupShape &s, double n_sm)
 {
-    return std::max(t.sk_whole + shape_span(s, t.sk_setup, t.sk_tile, n_sm), kv_read_us(s.kv_bytes, 6.5, 6.2e6));
+    return span_and_read(t.sk_whole + shape_span(s, t.sk_setup, t.sk_tile, n_sm), kv_read_us(s.kv_bytes, 5.8, 6.9e6));
 }
 
 double sk_cut_us(const PrefillCosts &t, const GroupShape &s, double n_cta)
 {
-    return std::max(t.sk_cut + shape_sum(s, t.sk_setup, t.sk_tile) / n_cta + t.sk_part * n_cta / s.units,
-                    kv_read_us(s.kv_bytes, 6.5, 6.2e6));
+    return span_and_read(t.sk_cut + shape_sum(s, t.sk_setup, t.sk_tile) / n_cta + t.sk_part * n_cta / s.units,
+                         kv_read_us(s.kv_bytes, 5.8, 6.9e6));
 }
 
 // Plan query (pe_attn_plan_launches): one launch as words -- kind, split,
@@ -1331,7 +1339,9 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
     if (!rec && (s = encode_q(&tm_q, Q, q_rows, hq, d, g)) != PE_OK) return s;
     if (!rec && (s = encode_q(&tm_o, out, q_rows, hq, d, g)) != PE_OK) return s;
 
-    const PrefillCosts &costs = d == 64 ? kCosts64 : kCosts128;
+    PrefillCosts costs = d == 64 ? kCosts64 : kCosts128;
+    // pages of 8 tokens: a producer's 32 boxes a tile of 128 columns take longer than the lone form's softmax
+    if (d == 128 && cf.page_size == 8) costs.tile[2] = costs.split_tile[1] = 1.2;
     const double n_sm = c->num_sms;
     // split-KV decision over the whole launch group; shape: the group's, plan_us: the chosen plan's estimated time
     GroupShape shape;
@@ -1372,7 +1382,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
             // keep the single pass unless clearly faster; by more where a pass is short, for a second launch costs
             // the host about 2 us, which the GPU's time no longer hides (8 CTAs of 5 key tiles, d = 64: one pass 10 us
             // by estimate, 5 splits 8, and the request is no faster; 2 sequences of 1.4k keys, 16.0 and 14.9: slower)
-            const double gain = std::max(0.02 * plan_us, 0.5 + 1.5 * std::min(1.0, std::max(0.0, (24.0 - plan_us) / 8.0)));
+            const double gain = std::max(0.02 * plan_us, 0.5 + 1.4 * std::min(1.0, std::max(0.0, (24.0 - plan_us) / 8.0)));
             if (splitkv == -1 && best > 1 && best_t > plan_us - gain) best = 1;
             if (best > 1) plan_us = best_t;
         }
@@ -1516,7 +1526,7 @@ pe_status run_attention(pe_cache *c, const std::vector<AttnItem> &items, int32_t
         const int64_t cut_ctas = std::min<int64_t>(c->num_sms, sk_ctas_that_fit(c, units));
         const double whole_us = sk_whole_us(costs, shape, n_sm), cut_us = sk_cut_us(costs, shape, static_cast<double>(cut_ctas));
         const bool sk_fits = 4 * units >= c->num_sms && units <= 16384 && !(one_pass && c->splitkv == 0);
-        // (2 % and half a microsecond for the host, whose plan takes some 5 us longer)
+        // (2 % and half a microsecond for the host, whose plan takes a few us longer)
         const double sk_limit = std::min(0.98 * one_us, one_us - 0.5);
         const bool sk_wins = sk_fits && std::min(whole_us, cut_us) <= sk_limit;
         bool sk = c->num_splits == 0 && (c->attn_kernel == 2 || (c->attn_kernel == 1 && sk_wins));

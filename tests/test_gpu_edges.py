@@ -83,6 +83,14 @@ def test_split_merge_shapes(d, splits, wide):
     assert plan[1] == -(-17 // -(-17 // splits)), plan
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("split", [0, 1])
+def test_one_q_tile_units_in_rounds(d, split):
+    """14 units of one q-tile on 4 persistent CTAs: rounds of whole units, then the rest whole or cut."""
+    _batch(d, 8, 2, 16, [40, 128, 129, 256, 300, 511, 640], [32, 20, 17, 32, 31, 9, 32],
+           {"attn_kernel": 2, "attn_ctas": 4, "splitkv": split}, seed=5 + d)
+
+
 # (d, Hq, Hkv, keys, queries): the plan's kernel and whether keys are cut, on 152 SMs
 DEFAULT_PLANS = [
     # one-item: pairs and lone q-tiles with key splits and in one pass, lone ones with key splits
@@ -95,30 +103,26 @@ DEFAULT_PLANS = [
     (128, 32, 8, [2500, 2600], [20, 20], "one_item", True),
     (64, 16, 8, [600] * 24, [40] * 24, "persistent", False),
     (128, 16, 8, [600] * 24, [40] * 24, "one_item", False),
-    # persistent with cuts: pairs only, pairs and lone q-tiles, lone ones only
-    (64, 8, 8, [914, 1658, 1325], [768, 512, 1024], "persistent", True),
-    (128, 32, 8, [2490, 1746], [256, 384], "persistent", True),
-    (64, 8, 8, [959, 1577], [784, 1501], "persistent", True),
-    (128, 8, 8, [1522, 2254], [1115, 1297], "persistent", True),
-    (64, 32, 8, [793, 744, 522, 607, 510, 605, 577, 599, 618, 721, 732, 680, 791, 654, 467, 765, 808, 760, 658, 578],
-     [26, 9, 31, 8, 7, 7, 27, 22, 5, 29, 16, 6, 7, 13, 6, 8, 10, 11, 6, 16], "persistent", True),
-    (128, 32, 8, [4176, 8101, 5250, 4692, 4445, 4434, 6705, 5325, 4922, 6424, 5707, 7662],
-     [21, 23, 24, 7, 5, 31, 7, 31, 15, 27, 30, 27], "persistent", True),
+    # persistent with cuts (each far enough from the line that 10 to 20 % more or fewer keys keep it): pairs only, pairs and
+    # lone q-tiles, lone ones only
+    (64, 8, 8, [2152, 1731], [1280, 1280], "persistent", True),
+    (128, 32, 8, [3105, 2492], [320, 320], "persistent", True),
+    (64, 8, 8, [1686, 2153], [1243, 1449], "persistent", True),
+    (128, 8, 8, [1976, 2455], [1364, 1004], "persistent", True),
+    (64, 32, 8, [657, 651, 703, 791, 649, 701, 855, 769, 711, 651, 801, 634, 733, 642, 757, 831, 767, 826, 754, 857],
+     [23, 10, 17, 21, 18, 19, 17, 23, 21, 19, 14, 27, 32, 27, 16, 26, 21, 17, 10, 18], "persistent", True),
+    (128, 16, 16, [10979, 9572, 10189, 8719, 9407], [111, 111, 111, 86, 115], "persistent", True),
     # persistent, at least two units a SM: rounds of whole units before the cut ones
-    (64, 32, 4, [767, 990, 949, 741, 598, 938, 746, 915, 872, 618, 935, 955, 746, 806, 802, 911, 976, 824, 688, 939],
-     [188, 21, 60, 171, 126, 82, 57, 67, 126, 182, 79, 148, 75, 169, 190, 154, 46, 93, 45, 145], "persistent", True),
-    (128, 32, 4, [939, 1043, 948, 1549, 1695, 902, 1282, 1427, 1300, 1173, 1350, 1536, 1680, 1579, 1743, 1023, 1511, 1736,
-                  1447, 1000],
-     [159, 140, 171, 83, 105, 37, 71, 185, 139, 116, 101, 107, 171, 78, 76, 172, 46, 29, 77, 40], "persistent", True),
+    (64, 32, 4, [827, 786, 833, 1016, 1016, 1046, 782, 763, 949, 984, 878, 1035, 765, 947, 964, 760, 1032, 841, 872, 828],
+     [104, 150, 148, 70, 165, 29, 153, 107, 21, 134, 81, 140, 42, 190, 174, 114, 98, 80, 84, 96], "persistent", True),
+    (128, 32, 4, [1323, 1173, 1495, 1331, 1456, 1203, 1548, 1315, 1593, 1252, 1551, 1527, 1172, 1465, 1238, 1430, 1488, 1498,
+                  1572, 1188],
+     [186, 128, 130, 95, 47, 41, 129, 98, 70, 83, 189, 130, 72, 132, 97, 85, 112, 141, 54, 81], "persistent", True),
     # the same with lone q-tiles only
     (64, 32, 8, [747, 907, 874, 793, 864, 884, 520, 737, 909, 561, 751, 501, 715, 643, 697, 611, 749, 712, 909, 797, 652, 788,
                  520, 893, 826, 844, 514, 580, 495, 574, 810, 596, 682, 572, 861, 864, 692, 836, 899],
      [31, 26, 15, 30, 12, 10, 17, 22, 15, 24, 15, 11, 16, 9, 29, 28, 18, 11, 25, 15, 24, 5, 10, 17, 6, 6, 14, 20, 12, 24, 10,
       23, 29, 13, 31, 13, 26, 6, 8], "persistent", True),
-    (128, 64, 8, [221, 216, 278, 342, 296, 236, 215, 295, 252, 253, 385, 339, 219, 298, 209, 219, 400, 246, 384, 400, 215, 384,
-                  300, 259, 274, 310, 386, 280, 355, 398, 221, 250, 234, 276, 211, 276, 281, 283, 389],
-     [9, 16, 3, 4, 14, 15, 8, 14, 14, 3, 9, 3, 8, 16, 7, 11, 12, 5, 16, 12, 16, 12, 10, 13, 6, 12, 3, 9, 13, 8, 3, 11, 10, 9,
-      4, 13, 15, 11, 3], "persistent", False),
 ]
 
 
